@@ -264,8 +264,7 @@ int mp_set_precision(mp_ctx* ctx, int precision);
  * CTAs per block of particles (1 to 64; default 1), whose partial sums are
  * added atomically into the Gauss-Newton sums (summation order, so the last
  * bits, then depend on scheduling). Splitting puts more CTAs to work when the
- * particles are few (a 4096-particle instance has 16 particle blocks for 152
- * SMs); mp_batch_create picks it per instance by timing. */
+ * particles are very few; mp_batch_create picks it per instance by timing. */
 int mp_set_likelihood_split(mp_ctx* ctx, int split);
 
 /* ---- Scan-to-scan GICP odometry (Sec. III-B, prediction step) ----------

@@ -4,8 +4,8 @@
 //    smaller index); Sigma = I - (1 - eps_cov) n n^T is carried as n.
 //  * the nearest neighbour field m^nnf: per voxel, the nearest valid map point
 //    to the voxel centre within r_max (-1 if none).
-//  * per-step scan Gaussians and the compaction of the valid scan points into
-//    the 32-byte records the likelihood kernel streams through shared memory.
+//  * per-step scan Gaussians and the sorted compaction of the valid scan points
+//    into the chunks the likelihood kernel stages in shared memory.
 #include "mp_internal.cuh"
 
 #include <algorithm>
@@ -209,19 +209,46 @@ struct ScanArgs {
     int n;
     float r2;
     int k, kmin;
-    float4* tmp4;
+    float inv_cell;      // 1 / (4 NNF voxels): the cells of scan_key
+    float4* tmp4;        // x, y, z and the bits of scan_key
     float* normals;
     uint8_t* valid;
-    float4* pair;
+    float4* pair;        // the valid points in input order, broadcast pairs, and
+    float* soa;          // sorted, the likelihood's chunks
     int32_t* nvalid;
 };
+
+// Order of the scan points for the likelihood: range shells of 64 NNF voxels
+// (16 of them at most), and in a shell the Morton code of the point's cell of 4
+// voxels. Whatever a particle's heading, a shell of the scan falls on a ring
+// around the particle, so particles near each other that work on one part of
+// the scan read one part of the NNF; and the points of a warp, neighbours in a
+// shell, read few lines of it. Results depend on the order only by rounding.
+__device__ __forceinline__ uint32_t scan_key(float x, float y, float z, float inv_cell) {
+    const float r = sqrtf(x * x + y * y + z * z) * inv_cell;
+    const uint32_t shell = (uint32_t)fminf(r * (1.f / 16.f), 15.f);
+    const float p[3] = {x, y, z};
+    uint32_t code = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        uint32_t c = (uint32_t)fminf(fmaxf(floorf(p[a] * inv_cell) + 256.f, 0.f), 511.f);
+        c = (c | (c << 16)) & 0x030000FFu;
+        c = (c | (c << 8)) & 0x0300F00Fu;
+        c = (c | (c << 4)) & 0x030C30C3u;
+        c = (c | (c << 2)) & 0x09249249u;
+        code |= c << a;
+    }
+    return (shell << 27) | code;
+}
 
 struct ScanF4Op {
     using Args = ScanArgs;
     static constexpr int THREADS = 256, MINB = 1;
     static __device__ __forceinline__ void run(const ScanArgs& A, unsigned bx, unsigned) {
         int i = (int)bx * THREADS + threadIdx.x;
-        if (i < A.n) A.tmp4[i] = make_float4(A.raw[3 * i], A.raw[3 * i + 1], A.raw[3 * i + 2], 0.f);
+        if (i >= A.n) return;
+        const float x = A.raw[3 * i], y = A.raw[3 * i + 1], z = A.raw[3 * i + 2];
+        A.tmp4[i] = make_float4(x, y, z, __uint_as_float(scan_key(x, y, z, A.inv_cell)));
     }
 };
 
@@ -307,59 +334,87 @@ __device__ __forceinline__ void ScanNormalsOp::run(const ScanArgs& args, unsigne
     valid[iq] = 1;
 }
 
-// Order-preserving compaction of the valid scan points into 48-byte records of
-// broadcast pairs (every value twice, the operand layout of the packed pipe);
-// one CTA per scan.
-struct ScanCompactOp {
+// Compaction: the valid points in the order of (key, index) into the chunks of
+// the point-major likelihood, and in input order into the broadcast pairs of
+// the particle-major one. A point's slot is the number of valid points before it,
+// counted over the whole scan by SCAN_PARTS threads a point, like the
+// neighbours above (a few us at 8192 points; one CTA that compacts in input
+// order took 17 us at 5000).
+struct ScanSortOp {
     using Args = ScanArgs;
-    static constexpr int THREADS = 1024, MINB = 1;
-    static __device__ __forceinline__ void run(const ScanArgs& A, unsigned, unsigned);
+    static constexpr int THREADS = SCAN_CTA, MINB = 1;
+    static __device__ __forceinline__ void run(const ScanArgs& A, unsigned bx, unsigned);
 };
 
-__device__ __forceinline__ void ScanCompactOp::run(const ScanArgs& args, unsigned, unsigned) {
+__device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned bx, unsigned) {
+    constexpr uint32_t NONE = 0xffffffffu;   // above every key
     const float* __restrict__ raw = args.raw;
     const float* __restrict__ normals = args.normals;
     const uint8_t* __restrict__ valid = args.valid;
+    const float4* __restrict__ pts = args.tmp4;
     const int n = args.n;
-    float4* __restrict__ pair = args.pair;
-    int32_t* __restrict__ nvalid = args.nvalid;
-    __shared__ int warp_tot[32];
-    __shared__ int base_s;
-    if (threadIdx.x == 0) base_s = 0;
-    __syncthreads();
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int start = 0; start < n; start += blockDim.x) {
-        int i = start + threadIdx.x;
-        int f = (i < n && valid[i]) ? 1 : 0;
-        unsigned bal = __ballot_sync(0xffffffffu, f);
-        int in_warp = __popc(bal & ((1u << lane) - 1u));
-        if (lane == 0) warp_tot[w] = __popc(bal);
+    __shared__ __align__(16) uint32_t sk[SCAN_TILE];
+    const int part = threadIdx.x % SCAN_PARTS, pl = threadIdx.x / SCAN_PARTS;
+    const int i = (int)bx * SCAN_PTS + pl;
+    const uint32_t key = (i < n && valid[i]) ? __float_as_uint(pts[i].w) : NONE;
+    uint32_t before = 0, earlier = 0, all = 0;   // valid points before this one by key, by index; all
+    for (int base = 0; base < n; base += SCAN_TILE) {
         __syncthreads();
-        int off = 0, tot = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-            if (k < w) off += warp_tot[k];
-            tot += warp_tot[k];
-        }
-        int base = base_s;
-        if (f) {
-            int o = base + off + in_warp;
-            if (!MP_DCHECK(o < n, "compacted scan index", o)) o = 0;
-            const float mx = raw[3 * i], my = raw[3 * i + 1], mz = raw[3 * i + 2];
-            const float nx = normals[3 * i], ny = normals[3 * i + 1], nz = normals[3 * i + 2];
-            pair[3 * o] = make_float4(mx, mx, my, my);
-            pair[3 * o + 1] = make_float4(mz, mz, nx, nx);
-            pair[3 * o + 2] = make_float4(ny, ny, nz, nz);
+        for (int t = threadIdx.x; t < SCAN_TILE; t += SCAN_CTA) {
+            const int j = base + t;
+            sk[t] = (j < n && valid[j]) ? __float_as_uint(pts[j].w) : NONE;
         }
         __syncthreads();
-        if (threadIdx.x == 0) base_s = base + tot;
-        __syncthreads();
+        const uint32_t lim = key + (base + SCAN_TILE <= i ? 1u : 0u);   // equal keys of an earlier tile count
+        const bool own = i >= base && i < base + SCAN_TILE;
+        for (int t = 4 * part; t < SCAN_TILE; t += 4 * SCAN_PARTS) {
+            const uint4 k4 = *reinterpret_cast<const uint4*>(sk + t);
+            before += (k4.x < lim) + (k4.y < lim) + (k4.z < lim) + (k4.w < lim);
+            const uint32_t here = (k4.x != NONE) + (k4.y != NONE) + (k4.z != NONE) + (k4.w != NONE);
+            all += here;
+            if (base + SCAN_TILE <= i) earlier += here;
+            if (own) {
+                const int j = base + t;
+                earlier += (k4.x != NONE && j < i) + (k4.y != NONE && j + 1 < i) + (k4.z != NONE && j + 2 < i) +
+                           (k4.w != NONE && j + 3 < i);
+                before += (k4.x == key && j < i) + (k4.y == key && j + 1 < i) + (k4.z == key && j + 2 < i) +
+                          (k4.w == key && j + 3 < i);
+            }
+        }
     }
-    if (threadIdx.x == 0) *nvalid = base_s;
+#pragma unroll
+    for (int o = 1; o < SCAN_PARTS; o <<= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        earlier += __shfl_xor_sync(0xffffffffu, earlier, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    if (bx == 0) {
+        if (threadIdx.x == 0) *args.nvalid = (int32_t)all;
+        // the last chunk's unused slots hold a point 1e18 m away, which no pose
+        // brings into a grid: the likelihood looks up whole chunks
+        static_assert(MP_SCAN_CHUNK == SCAN_CTA, "one thread per slot of a chunk");
+        const int64_t slot = (int64_t)(all / MP_SCAN_CHUNK) * MP_SCAN_CHUNK + threadIdx.x;
+        if (slot >= all && all % MP_SCAN_CHUNK != 0)
+            for (int k = 0; k < 6; ++k) args.soa[scan_word(slot, k)] = 1e18f;
+    }
+    if (part != 0 || key == NONE) return;
+    int64_t o = before, oe = earlier;
+    if (!MP_DCHECK(o < n && oe < n, "compacted scan index", o)) o = oe = 0;
+    float v[6];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        v[k] = raw[3 * i + k];
+        v[3 + k] = normals[3 * i + k];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) args.soa[scan_word(o, k)] = v[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) args.pair[3 * oe + k] = make_float4(v[2 * k], v[2 * k], v[2 * k + 1], v[2 * k + 1]);
 }
 
 __global__ void __launch_bounds__(256) k_scan_to_float4(const ScanArgs A) { ScanF4Op::run(A, blockIdx.x, 0); }
 __global__ void __launch_bounds__(SCAN_CTA) k_scan_normals(const ScanArgs A) { ScanNormalsOp::run(A, blockIdx.x, 0); }
-__global__ void __launch_bounds__(1024) k_scan_compact(const ScanArgs A) { ScanCompactOp::run(A, 0, 0); }
+__global__ void __launch_bounds__(SCAN_CTA) k_scan_sort(const ScanArgs A) { ScanSortOp::run(A, blockIdx.x, 0); }
 
 // NNF: nearest valid map point to each voxel centre within r_max.
 __global__ void k_nnf_build(const float4* __restrict__ pts, CellGridDev g, int nx, int ny, int64_t nvox, float ox,
@@ -605,10 +660,12 @@ ScanArgs scan_args(mp_ctx* c, const float* raw, int n) {
     A.r2 = c->p.r_cov * c->p.r_cov;
     A.k = c->p.cov_k;
     A.kmin = c->p.cov_min;
+    A.inv_cell = 0.25f / c->p.nnf_res;
     A.tmp4 = c->scan_tmp4;
     A.normals = c->scan_normals;
     A.valid = c->scan_valid;
     A.pair = c->scan_pair;
+    A.soa = c->scan_soa;
     A.nvalid = c->scan_nvalid;
     return A;
 }
@@ -628,7 +685,7 @@ int mp_launch_scan_prepare(mp_ctx* c) {
     MP_LAUNCHED(c);
     k_scan_normals<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
-    k_scan_compact<<<1, 1024, 0, c->stream>>>(A);
+    k_scan_sort<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -642,6 +699,7 @@ int mp_launch_point_gaussians(mp_ctx* c, const float* raw_dev, int n, float4* tm
     A.normals = normals;
     A.valid = valid;
     A.pair = nullptr;
+    A.soa = nullptr;
     A.nvalid = nullptr;
     k_scan_to_float4<<<grid_for(n, 256), 256, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
@@ -654,13 +712,12 @@ int mp_launch_point_gaussians(mp_ctx* c, const float* raw_dev, int n, float4* tm
 // scan buffer; the outputs go to each instance's own scan buffers.
 int mp_plan_scan(mp_group* G, int, std::vector<GOp>& plan) {
     std::vector<ScanArgs> tab;
-    std::vector<int64_t> b256, b64, b1;
+    std::vector<int64_t> b256, b64;
     for (int i = 0; i < G->size(); ++i) {
         const int n = G->n_scan[i];
         tab.push_back(scan_args(G->ctx[i], G->scan_dev + G->scan_off[i], n));
         b256.push_back((n + 255) / 256);
         b64.push_back((n + SCAN_PTS - 1) / SCAN_PTS);
-        b1.push_back(1);
     }
     const ScanArgs* t = G->upload(tab);
     unsigned nblk = 0;
@@ -668,8 +725,7 @@ int mp_plan_scan(mp_group* G, int, std::vector<GOp>& plan) {
     plan_kernel<ScanF4Op>(plan, t, m, nblk);
     m = G->block_map(b64, &nblk);
     plan_kernel<ScanNormalsOp>(plan, t, m, nblk);
-    m = G->block_map(b1, &nblk);
-    plan_kernel<ScanCompactOp>(plan, t, m, nblk);
+    plan_kernel<ScanSortOp>(plan, t, m, nblk);
     return G->err;
 }
 

@@ -168,7 +168,7 @@ void free_particles(mp_ctx* c) {
     dfree(c->poses[0]); dfree(c->poses[1]);
     dfree(c->logprior); dfree(c->post); dfree(c->post_tmp); dfree(c->post_init); dfree(c->post_invden); dfree(c->post_w);
     dfree(c->post_ids);
-    dfree(c->loglik); dfree(c->n_in); dfree(c->keys); dfree(c->buckets); dfree(c->sorted_ids); dfree(c->rank); dfree(c->visit);
+    dfree(c->loglik); dfree(c->n_in); dfree(c->keys); dfree(c->buckets); dfree(c->sorted_ids); dfree(c->rank); dfree(c->visit); dfree(c->lk_ticket);
     dfree(c->seg); dfree(c->sort_keys[0]); dfree(c->sort_keys[1]); dfree(c->sort_ids[0]); dfree(c->sort_ids[1]);
     dfree(c->radix_counts); dfree(c->scan_tmp);
     dfree(c->nbr_ids[0]); dfree(c->nbr_ids[1]); dfree(c->nbr_k); dfree(c->nbr_d);
@@ -196,6 +196,7 @@ int alloc_particles(mp_ctx* c, int64_t n) {
     A_(c->logprior, n); A_(c->post, n); A_(c->post_tmp, n); A_(c->post_init, n); A_(c->post_invden, n); A_(c->post_w, n * K);
     A_(c->post_ids, n * K);
     A_(c->loglik, n); A_(c->n_in, n); A_(c->keys, n); A_(c->buckets, n); A_(c->sorted_ids, n); A_(c->rank, n); A_(c->visit, n);
+    A_(c->lk_ticket, n / 256 + 3);
     A_(c->seg, 2 * ((int64_t)1 << c->p.n_buckets_log2));
     A_(c->sort_keys[0], n); A_(c->sort_keys[1], n); A_(c->sort_ids[0], n); A_(c->sort_ids[1], n);
     A_(c->radix_counts, MP_RADIX * nb);
@@ -225,7 +226,7 @@ void destroy(mp_ctx* c) {
         dfree(c->nnf);
     }
     c->map_refs = nullptr;
-    dfree(c->scan_raw); dfree(c->scan_normals); dfree(c->scan_valid); dfree(c->scan_pair); dfree(c->scan_h2); dfree(c->scan_tmp4);
+    dfree(c->scan_raw); dfree(c->scan_normals); dfree(c->scan_valid); dfree(c->scan_pair); dfree(c->scan_soa); dfree(c->scan_h2); dfree(c->scan_tmp4);
     dfree(c->scan_nvalid);
     dfree(c->scalars); dfree(c->best_idx); dfree(c->best_pose); dfree(c->dev_error); dfree(c->post_bar); dfree(c->pairs);
     dfree(c->step_dev);
@@ -393,6 +394,7 @@ static int ctx_setup(mp_ctx* c) {
         if ((rc = dalloc(c, &c->scan_normals, 3 * ms))) break;
         if ((rc = dalloc(c, &c->scan_valid, ms))) break;
         if ((rc = dalloc(c, &c->scan_pair, 3 * ms))) break;
+        if ((rc = dalloc(c, &c->scan_soa, scan_word((ms + MP_SCAN_CHUNK - 1) / MP_SCAN_CHUNK * MP_SCAN_CHUNK, 0)))) break;
         if ((rc = dalloc(c, &c->scan_h2, 2 * ms))) break;
         if ((rc = dalloc(c, &c->scan_tmp4, ms))) break;
         if ((rc = dalloc(c, &c->scan_nvalid, 1))) break;

@@ -25,6 +25,7 @@
 #define MP_RADIX_BITS 8
 #define MP_RADIX 256
 #define MP_SORT_TILE 2048   // elements per radix-sort block (256 threads x 8)
+#define MP_SCAN_CHUNK 256   // scan points per staged chunk of the likelihood
 
 // Per-step values the kernels read from device memory rather than from
 // their arguments, so that a captured step can be replayed: the LSH draw (as
@@ -76,6 +77,7 @@ struct mp_ctx {
     uint32_t* buckets;
     int32_t* sorted_ids;
     int32_t* rank;
+    int* lk_ticket;         // item counter and finished parts of the likelihood's particle blocks
     int32_t* visit;         // the likelihood's visiting order (position cells, LSH order within a cell)
     int32_t* seg;           // 2 per particle
     uint32_t* sort_keys[2];
@@ -100,6 +102,7 @@ struct mp_ctx {
     uint8_t* scan_valid;    // max_scan
     float4* scan_pair;      // 3 per valid point, every value twice (a broadcast pair):
                             // (mx,mx,my,my), (mz,mz,nx,nx), (ny,ny,nz,nz)
+    float* scan_soa;        // valid points in chunks of MP_SCAN_CHUNK, six planes each (scan_word)
     float4* scan_tmp4;      // max_scan float4 copy of the raw scan
     int32_t* scan_nvalid;   // device scalar
 
@@ -152,6 +155,11 @@ struct mp_ctx {
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
+// Word of component k (mu.xyz, normal.xyz) of valid scan point i in scan_soa.
+__host__ __device__ __forceinline__ size_t scan_word(int64_t i, int k) {
+    return ((size_t)(i / MP_SCAN_CHUNK) * 6 + k) * MP_SCAN_CHUNK + (size_t)(i % MP_SCAN_CHUNK);
+}
+
 struct Quat {
     float x, y, z, w;
 };

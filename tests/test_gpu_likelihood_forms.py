@@ -1,0 +1,78 @@
+"""The likelihood's two forms: point-major (a warp, or four, per particle; the
+scan in parts of up to 1536 staged points, looked up 256 or 64 at a time and
+queued in groups of 64) at the edges of those sizes, against the oracle; and
+particle-major (many particles on a small map) against point-major, in every
+precision."""
+import numpy as np
+import pytest
+
+from gpu_util import check_sums
+from paper_2404_16370_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def room(oracle):
+    w = synth.box_room_workload(n_particles=8192)
+    scan = synth.scan(w.scene, w.gt[0], synth.spherical_dirs(3200), 0.02, 7)
+    P = oracle.Params.box_room(4096)
+    return dict(w=w, om=oracle.OracleMap(w.map_points, P), P=P, scan=scan)
+
+
+def sums(room, poses, scan, precision=0):
+    from paper_2404_16370_gb300 import mp
+    n = len(poses)
+    ctx = mp.mp_init_map(room["w"].map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n))
+    try:
+        mp.mp_set_precision(ctx, precision)
+        mp.mp_init_particles(ctx, n, poses=poses)
+        mp.mp_set_scan(ctx, scan)
+        mp.mp_run_stages(ctx, mp.MP_STAGE_SCAN | mp.MP_STAGE_LIKELIHOOD)
+        return mp.mp_get_buffer(ctx, mp.MP_BUF_GN), mp.mp_get_buffer(ctx, mp.MP_BUF_SCAN_VALID)
+    finally:
+        mp.mp_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [2, 1024, 1025])      # four warps a particle up to 1024, one beyond
+@pytest.mark.parametrize("m", [64, 65, 255, 256, 257, 1536, 1537, 3200])
+def test_point_major_sizes(room, oracle, n, m):
+    # the densest part of the scan first, so that its points are valid and the
+    # parts are full: m points are m staged points
+    order = np.argsort(np.linalg.norm(room["scan"], axis=1), kind="stable")
+    sc = np.ascontiguousarray(room["scan"][order][:m])
+    gn, valid = sums(room, room["w"].particles[:n], sc)
+    P = room["P"]
+    sn, sv, _, _ = oracle.point_normals(sc, P.r_cov, P.cov_k, P.cov_min)
+    assert np.array_equal(valid.astype(bool), sv.astype(bool))
+    ref = oracle.likelihood(room["om"], room["w"].particles[:n], sc, sn, sv, P, amb_tol=1e-4)
+    msg = check_sums(gn, ref)
+    assert not msg, msg
+
+
+def test_scan_order_changes_only_the_rounding(room):
+    """The scan stage sorts the valid points: any input order of the same
+    points gives the same sums up to FP32 rounding, and the same inliers."""
+    poses = room["w"].particles[:1500]
+    a, va = sums(room, poses, room["scan"][:1100])
+    perm = np.random.default_rng(1).permutation(1100)
+    b, vb = sums(room, poses, np.ascontiguousarray(room["scan"][:1100][perm]))
+    assert np.array_equal(va[perm], vb)
+    assert np.array_equal(a[:, 28], b[:, 28])
+    assert np.all(np.abs(a - b) <= 2e-5 * (np.abs(a).max(axis=0, keepdims=True) + 1e-6))
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("n,m", [(81920, 129), (82001, 700)])
+def test_particle_major_equals_point_major(room, precision, n, m):
+    """The same pairs with the same arithmetic, summed in another order: equal
+    inliers, and sums within 1100 roundings of FP32 (6e-8 each) of their
+    largest, 2e-5 with the cancellation between terms."""
+    poses = np.tile(room["w"].particles, (n // 8192 + 1, 1))[:n]
+    sc = np.ascontiguousarray(room["scan"][:m])
+    pm, _ = sums(room, poses, sc, precision)
+    pt, _ = sums(room, poses[:1500], sc, precision)
+    assert np.array_equal(pm[:1500, 28], pt[:, 28])
+    assert np.all(np.abs(pm[:1500] - pt) <= 2e-5 * (np.abs(pt).max(axis=0, keepdims=True) + 1e-6))
+    assert np.array_equal(pm[:8192], pm[8192:16384])        # the same poses in other slots, to the last particle
+    assert np.array_equal(pm[n - 1], pm[(n - 1) % 8192])
