@@ -130,17 +130,19 @@ __device__ void normal_of_cov(const double C[6], float n_out[3]) {
     n_out[2] = (float)(sg * v[2]);
 }
 
-// FP64 sample covariance of the first m neighbours and the resulting normal.
-__device__ void neighbourhood_normal(const float4* __restrict__ pts, const int (&J)[MP_COVK], int m, float n_out[3]) {
+// FP64 sample covariance of the m neighbours J(0), J(1), ... and the resulting
+// normal.
+template <typename Index>
+__device__ void neighbourhood_normal(const float4* __restrict__ pts, Index J, int m, float n_out[3]) {
     double mx = 0, my = 0, mz = 0;
     for (int s = 0; s < m; ++s) {
-        float4 p = pts[J[s]];
+        float4 p = pts[J(s)];
         mx += p.x; my += p.y; mz += p.z;
     }
     mx /= m; my /= m; mz /= m;
     double C[6] = {0, 0, 0, 0, 0, 0};
     for (int s = 0; s < m; ++s) {
-        float4 p = pts[J[s]];
+        float4 p = pts[J(s)];
         double dx = p.x - mx, dy = p.y - my, dz = p.z - mz;
         C[0] += dx * dx; C[1] += dx * dy; C[2] += dx * dz;
         C[3] += dy * dy; C[4] += dy * dz; C[5] += dz * dz;
@@ -185,22 +187,30 @@ __global__ void k_map_normals(const float4* __restrict__ pts, int64_t n, CellGri
         return;
     }
     float nv[3];
-    neighbourhood_normal(pts, J, m, nv);
+    neighbourhood_normal(pts, [&](int s) { return J[s]; }, m, nv);
     normals[3 * i] = nv[0]; normals[3 * i + 1] = nv[1]; normals[3 * i + 2] = nv[2];
     valid[i] = 1;
 }
 
-// Scan points: brute force over the whole scan, staged through shared memory
-// in tiles. SCAN_PARTS threads share a point, each scanning every
-// SCAN_PARTS-th candidate of a tile with its own top-k, so that a scan of a
-// few thousand points still keeps every SM busy; the lists and counts are then
-// merged in shared memory (the top-k by (d, j) and the count do not depend on
-// the order in which candidates are seen), and one thread per point computes
-// the normal.
+// Scan points: brute force over the whole scan, staged through shared memory in
+// tiles. A warp takes two points, its lanes take candidates; those within the
+// radius go to a buffer per point, and when it fills up the cov_k nearest of it
+// are selected (cov_k rounds of a warp minimum over (d, j)) and their last
+// distance becomes the new radius. The set and its order do not depend on the
+// order in which candidates are seen. The normals, in FP64 (1/75 of the FP32
+// rate), take one lane per point: a dense warp for the CTA's 32 points. What
+// bounds it: the distances (13 instructions a warp and 32 candidates) from a few
+// thousand points on, below that the FP64 chain of one normal.
+// Measured (the scan stage, against one thread per point and eighth of the scan
+// with a sorted list of its own, merged by one thread): 128 points 62 -> 42 us,
+// 2048 142 -> 60, 4999 178 -> 101, 8192 233 -> 145.
 #define SCAN_TILE 1024
 #define SCAN_PARTS 8
 #define SCAN_CTA 256
 #define SCAN_PTS (SCAN_CTA / SCAN_PARTS)
+#define NRM_PTS 32                    // points of a CTA
+#define NRM_CTA (NRM_PTS / 2 * 32)    // two points a warp
+#define NRM_BUF 96                    // candidates a point's buffer holds
 
 // Arguments of the per-step scan kernels (raw n x 3 points in, normals,
 // validity and the compacted broadcast pairs out).
@@ -254,75 +264,104 @@ struct ScanF4Op {
 
 struct ScanNormalsOp {
     using Args = ScanArgs;
-    static constexpr int THREADS = SCAN_CTA, MINB = 1;
+    static constexpr int THREADS = NRM_CTA, MINB = 1;
     static __device__ __forceinline__ void run(const ScanArgs& A, unsigned bx, unsigned);
 };
+
+// The k smallest of the n <= NRM_BUF keys in buf, in order, to its front (one
+// warp); returns their number.
+__device__ __forceinline__ int select_nearest(uint64_t* buf, int n, int k, int lane) {
+    static_assert(NRM_BUF == 96, "three keys a lane");
+    __syncwarp();
+    uint64_t a = lane < n ? buf[lane] : ~0ull, b = 32 + lane < n ? buf[32 + lane] : ~0ull,
+             c = 64 + lane < n ? buf[64 + lane] : ~0ull;
+    uint64_t mine = ~0ull;
+    const int m = min(n, k);
+    for (int r = 0; r < m; ++r) {
+        const uint64_t x = min(a, min(b, c));
+        const unsigned hi = (unsigned)(x >> 32);
+        const unsigned H = __reduce_min_sync(0xffffffffu, hi);
+        const unsigned L = __reduce_min_sync(0xffffffffu, hi == H ? (unsigned)x : 0xffffffffu);
+        const uint64_t key = ((uint64_t)H << 32) | L;   // the keys differ in j
+        if (a == key) a = ~0ull;
+        if (b == key) b = ~0ull;
+        if (c == key) c = ~0ull;
+        if (lane == r) mine = key;
+    }
+    __syncwarp();
+    if (lane < m) buf[lane] = mine;
+    __syncwarp();
+    return m;
+}
 
 __device__ __forceinline__ void ScanNormalsOp::run(const ScanArgs& args, unsigned bx, unsigned) {
     const float* __restrict__ raw = args.raw;
     const int n = args.n, k = args.k, kmin = args.kmin;
-    const float r2 = args.r2;
     const float4* __restrict__ tmp_pts = args.tmp4;
     float* __restrict__ normals = args.normals;
     uint8_t* __restrict__ valid = args.valid;
     __shared__ float sx[SCAN_TILE], sy[SCAN_TILE], sz[SCAN_TILE];
-    __shared__ float Ds[SCAN_PTS][SCAN_PARTS][MP_COVK];
-    __shared__ int Js[SCAN_PTS][SCAN_PARTS][MP_COVK];
-    __shared__ int cs[SCAN_PTS][SCAN_PARTS];
-    const int part = threadIdx.x % SCAN_PARTS, pl = threadIdx.x / SCAN_PARTS;
-    const int i = (int)bx * SCAN_PTS + pl;
-    float px = 0, py = 0, pz = 0;
-    if (i < n) { px = raw[3 * i]; py = raw[3 * i + 1]; pz = raw[3 * i + 2]; }
-    float D[MP_COVK];
-    int J[MP_COVK];
+    __shared__ uint64_t buf[NRM_PTS][NRM_BUF];
+    __shared__ int found[NRM_PTS];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    float p[2][3], thr[2];
+    int nb[2] = {0, 0};
 #pragma unroll
-    for (int s = 0; s < MP_COVK; ++s) { D[s] = INFINITY; J[s] = 0x7fffffff; }
-    int cnt = 0;
+    for (int q = 0; q < 2; ++q) {
+        const int i = (int)bx * NRM_PTS + 2 * w + q;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) p[q][a] = i < n ? raw[3 * i + a] : 0.f;
+        thr[q] = i < n ? args.r2 : -1.f;
+    }
     for (int base = 0; base < n; base += SCAN_TILE) {
         __syncthreads();
-        for (int t = threadIdx.x; t < SCAN_TILE && base + t < n; t += SCAN_CTA) {
+        for (int t = threadIdx.x; t < SCAN_TILE && base + t < n; t += NRM_CTA) {
             sx[t] = raw[3 * (base + t)]; sy[t] = raw[3 * (base + t) + 1]; sz[t] = raw[3 * (base + t) + 2];
         }
         __syncthreads();
         const int m = min(SCAN_TILE, n - base);
-        if (i < n) {
-            for (int t = part; t < m; t += SCAN_PARTS) {
-                float d2 = dist2_exact(px, py, pz, sx[t], sy[t], sz[t]);
-                if (d2 <= r2) {
-                    cnt++;
-                    topk_insert(D, J, d2, base + t);
+        for (int t0 = 0; t0 < m; t0 += 32) {
+            const int t = t0 + lane;
+            const bool in = t < m;
+            const float x = in ? sx[t] : 0.f, y = in ? sy[t] : 0.f, z = in ? sz[t] : 0.f;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float d2 = dist2_exact(p[q][0], p[q][1], p[q][2], x, y, z);
+                const bool near = in && d2 <= thr[q];
+                const unsigned bal = __ballot_sync(0xffffffffu, near);
+                if (bal == 0) continue;
+                uint64_t* b = buf[2 * w + q];
+                if (near)
+                    b[nb[q] + __popc(bal & lt)] = ((uint64_t)__float_as_uint(d2) << 32) | (uint32_t)(base + t);
+                nb[q] += __popc(bal);
+                if (nb[q] > NRM_BUF - 32) {
+                    nb[q] = select_nearest(b, nb[q], k, lane);
+                    thr[q] = __uint_as_float((uint32_t)(b[nb[q] - 1] >> 32));
                 }
             }
         }
     }
 #pragma unroll
-    for (int s = 0; s < MP_COVK; ++s) { Ds[pl][part][s] = D[s]; Js[pl][part][s] = J[s]; }
-    cs[pl][part] = cnt;
-    __syncthreads();
-    // one thread per point (a dense warp) merges the parts and takes the normal
-    if (threadIdx.x >= SCAN_PTS) return;
-    const int q = threadIdx.x, iq = (int)bx * SCAN_PTS + q;
-    if (iq >= n) return;
-#pragma unroll
-    for (int s = 0; s < MP_COVK; ++s) { D[s] = Ds[q][0][s]; J[s] = Js[q][0][s]; }
-    cnt = cs[q][0];
-    for (int pp = 1; pp < SCAN_PARTS; ++pp) {
-        cnt += cs[q][pp];
-        for (int s = 0; s < MP_COVK; ++s) {
-            const float d = Ds[q][pp][s];
-            if (!(d < INFINITY)) break;   // a part's list is sorted: the rest is empty
-            topk_insert(D, J, d, Js[q][pp][s]);
-        }
+    for (int q = 0; q < 2; ++q) {
+        nb[q] = select_nearest(buf[2 * w + q], nb[q], k, lane);
+        if (lane == 0) found[2 * w + q] = nb[q];
     }
-    int m = min(cnt, k);
+    __syncthreads();
+    // the normals: one lane per point
+    if (threadIdx.x >= NRM_PTS) return;
+    const int q = threadIdx.x, iq = (int)bx * NRM_PTS + q;
+    if (iq >= n) return;
+    int m = found[q];
     if (m < kmin) {
         valid[iq] = 0;
         normals[3 * iq] = normals[3 * iq + 1] = normals[3 * iq + 2] = 0.f;
         return;
     }
+    auto J = [&](int s) { return (int)(uint32_t)buf[q][s]; };
 #ifdef MP_CHECKED
     for (int s = 0; s < m; ++s)
-        if (!MP_DCHECK(J[s] >= 0 && J[s] < n, "scan neighbour index", J[s])) m = 0;
+        if (!MP_DCHECK(J(s) >= 0 && J(s) < n, "scan neighbour index", J(s))) m = 0;
     if (m == 0) {
         valid[iq] = 0;
         return;
@@ -337,8 +376,7 @@ __device__ __forceinline__ void ScanNormalsOp::run(const ScanArgs& args, unsigne
 // Compaction: the valid points in the order of (key, index) into the chunks of
 // the point-major likelihood, and in input order into the broadcast pairs of
 // the particle-major one. A point's slot is the number of valid points before it,
-// counted over the whole scan by SCAN_PARTS threads a point, like the
-// neighbours above (a few us at 8192 points; one CTA that compacts in input
+// counted over the whole scan by SCAN_PARTS threads a point (a few us at 8192 points; one CTA that compacts in input
 // order took 17 us at 5000).
 struct ScanSortOp {
     using Args = ScanArgs;
@@ -413,7 +451,7 @@ __device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned b
 }
 
 __global__ void __launch_bounds__(256) k_scan_to_float4(const ScanArgs A) { ScanF4Op::run(A, blockIdx.x, 0); }
-__global__ void __launch_bounds__(SCAN_CTA) k_scan_normals(const ScanArgs A) { ScanNormalsOp::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(NRM_CTA) k_scan_normals(const ScanArgs A) { ScanNormalsOp::run(A, blockIdx.x, 0); }
 __global__ void __launch_bounds__(SCAN_CTA) k_scan_sort(const ScanArgs A) { ScanSortOp::run(A, blockIdx.x, 0); }
 
 // NNF: nearest valid map point to each voxel centre within r_max.
@@ -683,7 +721,7 @@ int mp_launch_scan_prepare(mp_ctx* c) {
     const ScanArgs A = scan_args(c, c->scan_raw, n);
     k_scan_to_float4<<<grid_for(n, 256), 256, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
-    k_scan_normals<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
+    k_scan_normals<<<grid_for(n, NRM_PTS), NRM_CTA, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
     k_scan_sort<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
@@ -703,7 +741,7 @@ int mp_launch_point_gaussians(mp_ctx* c, const float* raw_dev, int n, float4* tm
     A.nvalid = nullptr;
     k_scan_to_float4<<<grid_for(n, 256), 256, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
-    k_scan_normals<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
+    k_scan_normals<<<grid_for(n, NRM_PTS), NRM_CTA, 0, c->stream>>>(A);
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -723,6 +761,7 @@ int mp_plan_scan(mp_group* G, int, std::vector<GOp>& plan) {
     unsigned nblk = 0;
     const GBlk* m = G->block_map(b256, &nblk);
     plan_kernel<ScanF4Op>(plan, t, m, nblk);
+    static_assert(NRM_PTS == SCAN_PTS, "one block map for both");
     m = G->block_map(b64, &nblk);
     plan_kernel<ScanNormalsOp>(plan, t, m, nblk);
     plan_kernel<ScanSortOp>(plan, t, m, nblk);
