@@ -653,16 +653,20 @@ struct SortPhase {
 
 constexpr int SORT_PHASE_THREADS = 256;
 
-__device__ __forceinline__ bool sort_phase_sync(const SortPhase& P, unsigned& expect) {
-    const bool ok = grid_sync(P.bar, expect, P.budget);
-    expect = gridDim.x;
+struct SortPhaseBar {
+    unsigned expect, target;   // CTAs the next barrier waits for, arrivals of all so far
+};
+
+__device__ __forceinline__ bool sort_phase_sync(const SortPhase& P, SortPhaseBar& b) {
+    const bool ok = grid_sync(P.bar, b.target, b.expect, P.budget);
+    b.expect = gridDim.x;
     if (!ok && threadIdx.x == 0)
         for (int k = 0; k < P.n_inst; ++k) atomicOr(P.err[k], MP_ERR_WAIT);
     return ok;
 }
 
 // the radix passes [0, passes) of the sorts in tab (one per instance)
-__device__ __forceinline__ bool sort_passes(const SortPhase& P, const SortArgs* tab, int passes, unsigned& expect) {
+__device__ __forceinline__ bool sort_passes(const SortPhase& P, const SortArgs* tab, int passes, SortPhaseBar& expect) {
     for (int pss = 0; pss < passes; ++pss) {
         for (int w = blockIdx.x; w < P.n_sblk; w += gridDim.x) {
             const GBlk g = P.sblk[w];
@@ -686,7 +690,7 @@ __device__ __forceinline__ bool sort_passes(const SortPhase& P, const SortArgs* 
 }
 
 __global__ void __launch_bounds__(SORT_PHASE_THREADS) k_sort_phase(const __grid_constant__ SortPhase P) {
-    unsigned expect = gridDim.x + (P.starve ? 1u : 0u);
+    SortPhaseBar expect = {gridDim.x + (P.starve ? 1u : 0u), 0u};
     for (int w = blockIdx.x; w < P.n_pblk; w += gridDim.x) {
         const GBlk g = P.pblk[w];
         LshOp::run(P.lsh[g.inst], (unsigned)g.bx, 0);

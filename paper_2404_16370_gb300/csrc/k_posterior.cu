@@ -5,15 +5,16 @@
 //   w_ij = k_ij / sum_j k_ij fixed for the step (one thread per particle, FP64
 //   fused multiply-adds);
 //   normalise; best = argmax (smallest index on ties); log prior <- log p'.
-// Grid-wide max / sum / argmax are two-level (block partials, then one CTA
-// per instance), so results do not depend on atomics' order.
+// Grid-wide max / sum / argmax are two-level (block partials, then the partials
+// in one fixed order), so results do not depend on atomics' order.
 //
 // The whole stage is one cooperative (persistent) kernel, k_post_phase: its
 // CTAs, all resident, take the particle blocks of one instance (a context's
 // own launch) or of every instance of a batch in turn, with a bounded grid
-// barrier (grid_sync) between the sub-steps: block maxima | per-instance max |
-// exp, block sums and sweep weights | per-instance sum and sweep 1 | sweeps
-// 2..iters | final block partials | per-instance sum and argmax | normalise.
+// barrier (grid_sync) between the sub-steps: block maxima | max, exp, block
+// sums and sweep weights | sweep 1 | ... | the last sweep and the final block
+// partials | sum, argmax and normalise: iters + 2 barriers. Every CTA reduces
+// an instance's block partials for itself.
 // A barrier that gives up records MP_ERR_WAIT for every instance and the
 // kernel returns. A context's launch and a batch's launch run the same code
 // per block and per instance, so they compute the same bits.
@@ -45,7 +46,8 @@ struct PostArgs {
     double* post;
     double* post_tmp;
     double* post_init;
-    double* part;         // nb block partials (max, then sums)
+    double* part;         // nb block maxima of l, then the sums of the final pass
+    double* part_sum;     // nb block sums of exp(l - max l)
     double* part2;        // nb block maxima of the final pass
     int64_t* part_idx;    // nb block argmaxes
     double* scalars;      // [0] max l, [1] sum exp, [2] sum post, [3] best prob
@@ -82,29 +84,30 @@ __device__ __forceinline__ void post_l(const PostArgs& A, unsigned bx) {
     }
 }
 
-// the instance's max l over its block maxima
-__device__ __forceinline__ void reduce_max(const PostArgs& A) {
+// the instance's max l over its block maxima (every CTA takes it for itself:
+// no further barrier; in every thread)
+__device__ __forceinline__ double reduce_max(const PostArgs& A) {
     __shared__ double s[PB / 32];
     double v = -INFINITY;
-    for (int k = threadIdx.x; k < A.nb; k += PB) v = fmax(v, A.part[k]);
+    for (int k = threadIdx.x; k < A.nb; k += PB) v = fmax(v, __ldcg(A.part + k));
     v = warp_max(v);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < PB / 32 ? s[threadIdx.x] : -INFINITY;
-        v = warp_max(v);
-        if (threadIdx.x == 0) A.scalars[0] = v;
-    }
+    v = s[0];
+#pragma unroll
+    for (int k = 1; k < PB / 32; ++k) v = fmax(v, s[k]);
+    __syncthreads();
+    return v;
 }
 
 // p = exp(max(l - max l, floor)) into post_init and post_tmp (the sweeps'
 // input); block sums
-__device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx) {
+__device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx, double lmax) {
     __shared__ double s[PB / 32];
     int64_t i = (int64_t)bx * PB + threadIdx.x;
     double v = 0.0;
     if (i < A.n) {
-        v = exp(fmax(A.post[i] - A.scalars[0], A.lfloor));
+        v = exp(fmax(A.post[i] - lmax, A.lfloor));
         A.post_init[i] = v;
         A.post_tmp[i] = v;
     }
@@ -114,7 +117,10 @@ __device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx) {
     if (threadIdx.x < 32) {
         double w = threadIdx.x < PB / 32 ? s[threadIdx.x] : 0.0;
         w = warp_sum(w);
-        if (threadIdx.x == 0) A.part[bx] = w;
+        if (threadIdx.x == 0) {
+            A.part_sum[bx] = w;
+            if (bx == 0) A.scalars[0] = lmax;
+        }
     }
 }
 
@@ -122,7 +128,7 @@ __device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx) {
 __device__ __forceinline__ void reduce_sum(const PostArgs& A) {
     __shared__ double s[PB / 32];
     double v = 0.0;
-    for (int k = threadIdx.x; k < A.nb; k += PB) v += A.part[k];
+    for (int k = threadIdx.x; k < A.nb; k += PB) v += __ldcg(A.part_sum + k);
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -248,14 +254,19 @@ __device__ __forceinline__ void final_part(const PostArgs& A, unsigned bx) {
 }
 
 // the instance's sum of the smoothed posterior, its best value and index
-__device__ __forceinline__ void final_reduce(const PostArgs& A) {
+// (every CTA for itself; in every thread)
+struct PostFinal {
+    double sum, best;
+    int64_t idx;
+};
+__device__ __forceinline__ PostFinal final_reduce(const PostArgs& A) {
     __shared__ double ss[PB / 32], sm[PB / 32];
     __shared__ int64_t si[PB / 32];
     double S = 0.0, M = -INFINITY;
     int64_t I = INT64_MAX;
     for (int k = threadIdx.x; k < A.nb; k += PB) {
-        S += A.part[k];
-        argmax_merge(M, I, A.part2[k], A.part_idx[k]);
+        S += __ldcg(A.part + k);
+        argmax_merge(M, I, __ldcg(A.part2 + k), __ldcg(reinterpret_cast<const long long*>(A.part_idx) + k));
     }
     S = warp_sum(S);
 #pragma unroll
@@ -270,30 +281,31 @@ __device__ __forceinline__ void final_reduce(const PostArgs& A) {
         si[threadIdx.x >> 5] = I;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double S2 = 0.0, M2 = -INFINITY;
-        int64_t I2 = INT64_MAX;
-        for (int k = 0; k < PB / 32; ++k) {
-            S2 += ss[k];
-            argmax_merge(M2, I2, sm[k], si[k]);
-        }
-        A.scalars[2] = S2;
-        A.scalars[3] = M2 / S2;
-        *A.best_idx = I2;
+    PostFinal f = {0.0, -INFINITY, INT64_MAX};
+    for (int k = 0; k < PB / 32; ++k) {
+        f.sum += ss[k];
+        argmax_merge(f.best, f.idx, sm[k], si[k]);
     }
+    __syncthreads();
+    return f;
 }
 
 // normalise (post_tmp keeps the smoothed values), store the log prior, copy
 // the best pose
-__device__ __forceinline__ void normalise(const PostArgs& A, unsigned bx) {
+__device__ __forceinline__ void normalise(const PostArgs& A, unsigned bx, const PostFinal& f) {
     int64_t i = (int64_t)bx * PB + threadIdx.x;
+    if (bx == 0 && threadIdx.x == 0) {
+        A.scalars[2] = f.sum;
+        A.scalars[3] = f.best / f.sum;
+        *A.best_idx = f.idx;
+    }
     if (i < A.n) {
         const double sm = post_smoothed(A)[i];
         if (A.iters & 1) A.post_tmp[i] = sm;
-        const double v = sm / A.scalars[2];
+        const double v = sm / f.sum;
         A.post[i] = v;
         A.logprior[i] = log(v);
-        if (i == *A.best_idx) {
+        if (i == f.idx) {
             A.best_pose[0] = A.poses[2 * i];
             A.best_pose[1] = A.poses[2 * i + 1];
         }
@@ -314,13 +326,15 @@ struct PostPhase {
 __device__ __forceinline__ const PostArgs& phase_args(const PostPhase& P, int inst) {
     return P.tab ? P.tab[inst] : P.one;
 }
-__device__ __forceinline__ const PostArgs& phase_item(const PostPhase& P, int w, unsigned& bx) {
+__device__ __forceinline__ const PostArgs& phase_item(const PostPhase& P, int w, unsigned& bx, int& inst) {
     if (!P.blocks) {
         bx = (unsigned)w;
+        inst = 0;
         return P.one;
     }
     const GBlk g = P.blocks[w];
     bx = (unsigned)g.bx;
+    inst = g.inst;
     return P.tab[g.inst];
 }
 
@@ -328,65 +342,68 @@ __device__ __forceinline__ const PostArgs& phase_item(const PostPhase& P, int w,
 // more CTAs spill the sub-steps' FP64 values and measured slower)
 __global__ void __launch_bounds__(PB, 4) k_post_phase(const __grid_constant__ PostPhase P) {
     // the test knob: the first barrier waits for one CTA more than the grid
-    unsigned expect = gridDim.x + (P.starve ? 1u : 0u);
+    unsigned expect = gridDim.x + (P.starve ? 1u : 0u), target = 0;
     auto sync = [&]() {
-        const bool ok = grid_sync(P.bar, expect, P.budget);
+        const bool ok = grid_sync(P.bar, target, expect, P.budget);
         expect = gridDim.x;
         if (!ok && threadIdx.x == 0)
             for (int k = 0; k < P.n_inst; ++k) atomicOr(phase_args(P, k).err, MP_ERR_WAIT);
         return ok;
     };
+    // (phase_item sets bx and inst: a statement of its own)
     unsigned bx;
+    int inst, cur = -1;
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
-        const PostArgs& A = phase_item(P, w, bx);   // sets bx: a statement of its own
+        const PostArgs& A = phase_item(P, w, bx, inst);
         post_l(A, bx);
         __syncthreads();
     }
     if (!sync()) return;
-    for (int k = blockIdx.x; k < P.n_inst; k += gridDim.x) {
-        reduce_max(phase_args(P, k));
-        __syncthreads();
-    }
-    if (!sync()) return;
+    double lmax = 0.0;
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
-        const PostArgs& A = phase_item(P, w, bx);
-        post_exp(A, bx);
+        const PostArgs& A = phase_item(P, w, bx, inst);
+        if (inst != cur) {
+            lmax = reduce_max(A);
+            cur = inst;
+        }
+        post_exp(A, bx, lmax);
         post_weights(A, bx);
         __syncthreads();
     }
     if (!sync()) return;
-    // the sums read the block partials of post_exp; the first sweep reads
-    // post_tmp and the weights: both run after the same barrier
     for (int k = blockIdx.x; k < P.n_inst; k += gridDim.x) {
         reduce_sum(phase_args(P, k));
         __syncthreads();
     }
     for (int it = 0; it < P.max_iters; ++it) {
+        if (it > 0 && !sync()) return;
         for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
-            const PostArgs& A = phase_item(P, w, bx);
+            const PostArgs& A = phase_item(P, w, bx, inst);
             if (it < A.iters) {
                 if (A.K == 32) post_sweep<32>(A, bx, it);
                 else if (A.K == 16) post_sweep<16>(A, bx, it);
                 else post_sweep<0>(A, bx, it);
             }
         }
-        if (!sync()) return;
     }
-    if (P.max_iters == 0 && !sync()) return;   // the sums before final_part rewrites the partials
+    // a block's smoothed values are this CTA's own (the same blocks in every
+    // sub-step), and the block maxima were read before the last barrier
+    __syncthreads();
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
-        const PostArgs& A = phase_item(P, w, bx);
+        const PostArgs& A = phase_item(P, w, bx, inst);
         final_part(A, bx);
         __syncthreads();
     }
     if (!sync()) return;
-    for (int k = blockIdx.x; k < P.n_inst; k += gridDim.x) {
-        final_reduce(phase_args(P, k));
-        __syncthreads();
-    }
-    if (!sync()) return;
+    PostFinal f = {};
+    cur = -1;
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
-        const PostArgs& A = phase_item(P, w, bx);
-        normalise(A, bx);
+        const PostArgs& A = phase_item(P, w, bx, inst);
+        if (inst != cur) {
+            f = final_reduce(A);
+            cur = inst;
+        }
+        normalise(A, bx, f);
     }
 }
 
@@ -402,6 +419,7 @@ PostArgs post_args(mp_ctx* c, int cur) {
     A.part = c->red;
     A.part2 = c->red + A.nb;
     A.part_idx = (int64_t*)(c->red + 2 * (int64_t)A.nb);
+    A.part_sum = c->red + 3 * (int64_t)A.nb;
     A.scalars = c->scalars;
     A.best_idx = c->best_idx;
     A.ids = c->nbr_ids[cur];

@@ -415,15 +415,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 #define MP_ERR_WAIT 1
 
 // Grid-wide barrier of a cooperative (persistent) launch, whose CTAs are all
-// resident at once. Thread 0 of each CTA reads the generation, arrives on the
-// counter and, unless it is the last to arrive, spins until the generation
-// moves on; the last arrival resets the counter and advances the generation.
-// The spin is bounded by `budget` SM cycles and also ends when another CTA has
-// given up (abort); grid_sync then returns false and the caller records the
-// error and returns. Zero the barrier before every launch.
+// resident at once. Thread 0 of each CTA arrives on a counter that only grows
+// and spins until it reaches this barrier's target, the arrivals of all
+// barriers so far: one atomic and the reads of the spin (a counter that the
+// last arrival resets and a generation word cost four dependent L2 round
+// trips, 3 us a barrier with one CTA). A grid of one CTA needs no more than
+// __syncthreads. The spin is bounded by `budget` SM cycles and also ends when
+// another CTA has given up (abort); grid_sync then returns false and the caller
+// records the error and returns. Zero the barrier before every launch, and
+// start each CTA's target at 0.
 struct GridBar {
-    unsigned int count, gen;
-    int abort, pad;
+    unsigned int count;
+    int abort, pad[2];
 };
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
@@ -435,27 +438,26 @@ __device__ __forceinline__ int ld_relaxed_s32(const int* p) {
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned expected, long long budget) {
+__device__ __forceinline__ bool grid_sync(GridBar* gb, unsigned& target, unsigned expected, long long budget) {
     __shared__ int ok_s;
+    target += expected;
+    if (expected == 1) {
+        __syncthreads();
+        return true;
+    }
     __syncthreads();   // the CTA's share of the sub-step is done
     if (threadIdx.x == 0) {
         int ok = 1;
-        const unsigned g = ld_acquire_u32(&gb->gen);
         __threadfence();   // this CTA's writes before its arrival
-        if (atomicAdd(&gb->count, 1u) + 1u == expected) {
-            atomicExch(&gb->count, 0u);
-            __threadfence();
-            atomicAdd(&gb->gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (ld_acquire_u32(&gb->gen) == g) {
-                if (ld_relaxed_s32(&gb->abort) != 0 || clock64() - t0 > budget) {
-                    ok = 0;
-                    atomicExch(&gb->abort, 1);
-                    break;
-                }
-                __nanosleep(64);
+        atomicAdd(&gb->count, 1u);
+        const long long t0 = clock64();
+        while (ld_acquire_u32(&gb->count) < target) {
+            if (ld_relaxed_s32(&gb->abort) != 0 || clock64() - t0 > budget) {
+                ok = 0;
+                atomicExch(&gb->abort, 1);
+                break;
             }
+            __nanosleep(32);
         }
         __threadfence();   // the other CTAs' writes after the barrier
         ok_s = ok;
