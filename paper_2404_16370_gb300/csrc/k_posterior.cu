@@ -215,6 +215,52 @@ __device__ __forceinline__ void post_sweep(const PostArgs& A, unsigned bx, int i
     }
 }
 
+// The same weights and sweep with the particle's list held in registers for all
+// sweeps (one particle per thread of the whole launch; K <= KT, slots K.. and
+// missing neighbours have id -1): a sweep then waits for one L2 round trip, the
+// gathers of p, and not for ids and weights before them.
+template <int KT>
+struct PostList {
+    int32_t id[KT];
+    double w[KT];
+    double invden;
+};
+template <int KT>
+__device__ __forceinline__ void post_list(const PostArgs& A, unsigned bx, PostList<KT>& L) {
+    const int64_t i = (int64_t)bx * PB + threadIdx.x;
+    double den = 0.0;
+#pragma unroll
+    for (int l = 0; l < KT; ++l) {
+        const bool in = i < A.n && l < A.K;
+        L.id[l] = in ? A.ids[i * A.K + l] : -1;
+        L.w[l] = in ? (double)A.kk[i * A.K + l] : 0.0;
+    }
+#pragma unroll
+    for (int l = 0; l < KT; ++l)
+        if (L.id[l] >= 0) den += L.w[l];
+    L.invden = den > 0.0 ? 1.0 / den : 0.0;
+#pragma unroll
+    for (int l = 0; l < KT; ++l) {
+        if (!(L.id[l] < A.n && MP_DCHECK(L.id[l] >= -1, "neighbour id", L.id[l]))) L.id[l] = -1;
+        L.w[l] *= L.invden;
+    }
+}
+template <int KT>
+__device__ __forceinline__ void post_list_sweep(const PostArgs& A, unsigned bx, int it, const PostList<KT>& L) {
+    const double* pin = (it & 1) ? A.post : A.post_tmp;
+    double* pout = (it & 1) ? A.post_tmp : A.post;
+    const int64_t i = (int64_t)bx * PB + threadIdx.x;
+    if (i >= A.n) return;
+    double p[KT];
+#pragma unroll
+    for (int l = 0; l < KT; ++l) p[l] = L.id[l] >= 0 ? __ldcg(pin + L.id[l]) : 0.0;
+    double num = 0.0;
+#pragma unroll
+    for (int l = 0; l < KT; ++l)
+        if (L.id[l] >= 0) num = fma(L.w[l], p[l], num);
+    pout[i] = L.invden > 0.0 ? num : __ldcg(pin + i);
+}
+
 // the smoothed posterior after the sweeps
 __device__ __forceinline__ const double* post_smoothed(const PostArgs& A) { return (A.iters & 1) ? A.post : A.post_tmp; }
 
@@ -338,9 +384,14 @@ __device__ __forceinline__ const PostArgs& phase_item(const PostPhase& P, int w,
     return P.tab[g.inst];
 }
 
-// 4 CTAs of 256 threads per SM: 64 registers, no spill (fewer registers and
-// more CTAs spill the sub-steps' FP64 values and measured slower)
-__global__ void __launch_bounds__(PB, 4) k_post_phase(const __grid_constant__ PostPhase P) {
+// KT = 0: any number of particles, 4 CTAs of 256 threads per SM (64 registers,
+// no spill; fewer registers and more CTAs spill the sub-steps' FP64 values and
+// measured slower). KT = 16, 32: at most one particle block per CTA and lists of
+// at most KT entries, which stay in registers
+// (256 x 16: 57 -> 44 us, 4096 x 16: 91 -> 71; what is left is the sub-steps'
+// latency, an L2 round trip and a barrier per sweep).
+template <int KT>
+__global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_phase(const __grid_constant__ PostPhase P) {
     // the test knob: the first barrier waits for one CTA more than the grid
     unsigned expect = gridDim.x + (P.starve ? 1u : 0u), target = 0;
     auto sync = [&]() {
@@ -360,6 +411,7 @@ __global__ void __launch_bounds__(PB, 4) k_post_phase(const __grid_constant__ Po
     }
     if (!sync()) return;
     double lmax = 0.0;
+    PostList<KT == 0 ? 1 : KT> list;
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
         const PostArgs& A = phase_item(P, w, bx, inst);
         if (inst != cur) {
@@ -367,7 +419,8 @@ __global__ void __launch_bounds__(PB, 4) k_post_phase(const __grid_constant__ Po
             cur = inst;
         }
         post_exp(A, bx, lmax);
-        post_weights(A, bx);
+        if constexpr (KT == 0) post_weights(A, bx);
+        else post_list<KT>(A, bx, list);
         __syncthreads();
     }
     if (!sync()) return;
@@ -379,7 +432,10 @@ __global__ void __launch_bounds__(PB, 4) k_post_phase(const __grid_constant__ Po
         if (it > 0 && !sync()) return;
         for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
             const PostArgs& A = phase_item(P, w, bx, inst);
-            if (it < A.iters) {
+            if (it >= A.iters) continue;
+            if constexpr (KT != 0) {
+                post_list_sweep<KT>(A, bx, it, list);
+            } else {
                 if (A.K == 32) post_sweep<32>(A, bx, it);
                 else if (A.K == 16) post_sweep<16>(A, bx, it);
                 else post_sweep<0>(A, bx, it);
@@ -436,8 +492,9 @@ PostArgs post_args(mp_ctx* c, int cur) {
     return A;
 }
 
-// Resident CTAs of k_post_phase on the current device: the grid of a
+// Resident CTAs of k_post_phase<KT> on the current device: the grid of a
 // cooperative launch may not exceed it.
+template <int KT>
 unsigned post_capacity() {
     static int cap[64] = {};
     int dev = 0;
@@ -445,11 +502,24 @@ unsigned post_capacity() {
     if (!cap[dev]) {
         int sms = 0, per = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_post_phase, PB, 0) != cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_post_phase<KT>, PB, 0) != cudaSuccess)
             return 0;
         cap[dev] = sms * per;
     }
     return (unsigned)cap[dev];
+}
+
+// The form of a launch over n_blocks particle blocks with lists of at most K
+// entries, and its grid (0: none): registers hold the lists when every block
+// has a CTA of its own (about 38k particles at K <= 32, 77k at K <= 16).
+struct PostForm {
+    const void* func;
+    unsigned grid;
+};
+PostForm post_form(unsigned n_blocks, int K) {
+    if (K <= 16 && n_blocks <= post_capacity<16>()) return {(const void*)k_post_phase<16>, n_blocks};
+    if (K > 16 && n_blocks <= post_capacity<32>()) return {(const void*)k_post_phase<32>, n_blocks};
+    return {(const void*)k_post_phase<0>, std::min(n_blocks, post_capacity<0>())};
 }
 
 long long post_budget(const mp_ctx* c) { return c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET; }
@@ -465,11 +535,10 @@ int mp_launch_posterior(mp_ctx* c) {
     P.starve = c->starve_bar;
     P.bar = c->post_bar;
     P.budget = post_budget(c);
-    const unsigned cap = post_capacity();
-    if (!cap) return mp_fail(c, MP_ECUDA, "posterior: no resident CTAs for the cooperative launch");
+    const PostForm form = post_form((unsigned)P.n_blocks, P.one.K);
+    if (!form.grid) return mp_fail(c, MP_ECUDA, "posterior: no resident CTAs for the cooperative launch");
     MP_CUDA(c, cudaMemsetAsync(c->post_bar, 0, sizeof(GridBar), c->stream));
-    MP_CUDA(c, launch_coop((const void*)k_post_phase, std::min<unsigned>((unsigned)P.n_blocks, cap), PB, &P,
-                           c->stream));
+    MP_CUDA(c, launch_coop(form.func, form.grid, PB, &P, c->stream));
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -479,20 +548,21 @@ int mp_launch_posterior(mp_ctx* c) {
 int mp_plan_posterior(mp_group* G, int p, std::vector<GOp>& plan) {
     std::vector<PostArgs> tab;
     std::vector<int64_t> bpb;
-    int max_iters = 0;
+    int max_iters = 0, max_K = 0;
     for (int i = 0; i < G->size(); ++i) {
         mp_ctx* c = G->ctx[i];
         tab.push_back(post_args(c, c->nbr_cur ^ p ^ 1));   // the list the merge of this step wrote
         bpb.push_back(tab.back().nb);
         max_iters = std::max(max_iters, tab.back().iters);
+        max_K = std::max(max_K, tab.back().K);
     }
     GridBar* bar = static_cast<GridBar*>(G->scratch(sizeof(GridBar)));
     const PostArgs* t = G->upload(tab);
     unsigned nblk = 0;
     const GBlk* map = G->block_map(bpb, &nblk);
-    const unsigned cap = post_capacity();
     if (G->err) return G->err;
-    if (!cap) return MP_ECUDA;
+    const PostForm form = post_form(nblk, max_K);
+    if (!form.grid) return MP_ECUDA;
     PostPhase P = {};
     P.tab = t;
     P.blocks = map;
@@ -503,6 +573,6 @@ int mp_plan_posterior(mp_group* G, int p, std::vector<GOp>& plan) {
     P.bar = bar;
     P.budget = post_budget(G->ctx[0]);
     plan_memset(plan, bar, sizeof(GridBar));
-    plan_coop(plan, (const void*)k_post_phase, std::min(nblk, cap), PB, P);
+    plan_coop(plan, form.func, form.grid, PB, P);
     return MP_OK;
 }
