@@ -343,7 +343,8 @@ int mp_kernel_launches(mp_ctx* ctx, int64_t* count);
  * grid has, so every CTA's bounded wait gives up; the kernel records the error
  * for every instance it serves and returns. In a batch the first instance's
  * knob and wait budget when mp_batch_create captures the step apply, to the
- * posterior and to the batch's LSH/sort phase (also one cooperative launch). */
+ * posterior and, with instances of more than 16384 particles, to the batch's
+ * LSH/sort phase (also one cooperative launch). */
 #define MP_DEBUG_WAIT_BUDGET 1
 #define MP_DEBUG_STARVE_TX 2
 #define MP_DEBUG_STARVE_BARRIER 3

@@ -127,7 +127,7 @@ int run_plan(const std::vector<GOp>& plan, cudaStream_t s) {
     for (const GOp& o : plan) {
         if (o.kind == GOp::KERNEL) {
             void* args[2] = {(void*)&o.tab, (void*)&o.map};
-            B_CUDA(cudaLaunchKernel(o.func, dim3(o.grid), dim3(o.block), args, 0, s));
+            B_CUDA(cudaLaunchKernel(o.func, dim3(o.grid), dim3(o.block), args, o.smem, s));
         } else if (o.kind == GOp::COOP) {
             B_CUDA(launch_coop(o.func, o.grid, o.block, (void*)o.arg, s));
         } else if (o.kind == GOp::MEMSET) {

@@ -597,6 +597,7 @@ struct GOp {
     enum Kind { KERNEL, COOP, MEMSET, COPY } kind;
     const void* func;
     unsigned grid, block;
+    size_t smem;   // dynamic shared memory of a grouped kernel
     const void* tab;
     const GBlk* map;
     void* dst;
