@@ -223,8 +223,9 @@ struct ScanArgs {
     float4* tmp4;        // x, y, z and the bits of scan_key
     float* normals;
     uint8_t* valid;
-    float4* pair;        // the valid points in input order, broadcast pairs, and
-    float* soa;          // sorted, the likelihood's chunks
+    float4* pair;        // the valid points in input order, broadcast pairs (or null),
+    float* soa;          // and sorted, the likelihood's chunks
+    int32_t* idx;        // the sorted points' indices (or null)
     int32_t* nvalid;
 };
 
@@ -446,13 +447,28 @@ __device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned b
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) args.soa[scan_word(o, k)] = v[k];
+    if (args.idx) args.idx[o] = i;
+    if (!args.pair) return;
 #pragma unroll
     for (int k = 0; k < 3; ++k) args.pair[3 * oe + k] = make_float4(v[2 * k], v[2 * k], v[2 * k + 1], v[2 * k + 1]);
 }
 
-__global__ void __launch_bounds__(256) k_scan_to_float4(const ScanArgs A) { ScanF4Op::run(A, blockIdx.x, 0); }
-__global__ void __launch_bounds__(NRM_CTA) k_scan_normals(const ScanArgs A) { ScanNormalsOp::run(A, blockIdx.x, 0); }
-__global__ void __launch_bounds__(SCAN_CTA) k_scan_sort(const ScanArgs A) { ScanSortOp::run(A, blockIdx.x, 0); }
+// One scan, or two in one launch (blockIdx.y).
+struct ScanArgs2 {
+    ScanArgs s[2];
+};
+template <typename Op, int PTS>
+__device__ __forceinline__ void scan_run(const ScanArgs2& A) {
+    const ScanArgs& a = A.s[blockIdx.y];
+    if (blockIdx.x * PTS < (unsigned)a.n) Op::run(a, blockIdx.x, 0);
+}
+__global__ void __launch_bounds__(256) k_scan_to_float4(const __grid_constant__ ScanArgs2 A) { scan_run<ScanF4Op, 256>(A); }
+__global__ void __launch_bounds__(NRM_CTA) k_scan_normals(const __grid_constant__ ScanArgs2 A) {
+    scan_run<ScanNormalsOp, NRM_PTS>(A);
+}
+__global__ void __launch_bounds__(SCAN_CTA) k_scan_sort(const __grid_constant__ ScanArgs2 A) {
+    scan_run<ScanSortOp, SCAN_PTS>(A);
+}
 
 // NNF: nearest valid map point to each voxel centre within r_max.
 __global__ void k_nnf_build(const float4* __restrict__ pts, CellGridDev g, int nx, int ny, int64_t nvox, float ox,
@@ -702,6 +718,7 @@ ScanArgs scan_args(mp_ctx* c, const float* raw, int n) {
     A.tmp4 = c->scan_tmp4;
     A.normals = c->scan_normals;
     A.valid = c->scan_valid;
+    A.idx = nullptr;
     A.pair = c->scan_pair;
     A.soa = c->scan_soa;
     A.nvalid = c->scan_nvalid;
@@ -710,8 +727,20 @@ ScanArgs scan_args(mp_ctx* c, const float* raw, int n) {
 
 }  // namespace
 
+// The scan kernels over m scans.
+static int launch_scans(mp_ctx* c, const ScanArgs2& A, int m) {
+    const int n = m > 1 ? std::max(A.s[0].n, A.s[1].n) : A.s[0].n;
+    k_scan_to_float4<<<dim3(grid_for(n, 256), m), 256, 0, c->stream>>>(A);
+    MP_LAUNCHED(c);
+    k_scan_normals<<<dim3(grid_for(n, NRM_PTS), m), NRM_CTA, 0, c->stream>>>(A);
+    MP_LAUNCHED(c);
+    k_scan_sort<<<dim3(grid_for(n, SCAN_PTS), m), SCAN_CTA, 0, c->stream>>>(A);
+    MP_LAUNCHED(c);
+    return MP_OK;
+}
+
 // Per-step scan Gaussians (brute-force radius kNN in shared-memory tiles) and
-// compaction of the valid points.
+// the valid points, sorted and in input order.
 int mp_launch_scan_prepare(mp_ctx* c) {
     int n = c->n_scan;
     if (n == 0) {
@@ -719,31 +748,25 @@ int mp_launch_scan_prepare(mp_ctx* c) {
         return MP_OK;
     }
     const ScanArgs A = scan_args(c, c->scan_raw, n);
-    k_scan_to_float4<<<grid_for(n, 256), 256, 0, c->stream>>>(A);
-    MP_LAUNCHED(c);
-    k_scan_normals<<<grid_for(n, NRM_PTS), NRM_CTA, 0, c->stream>>>(A);
-    MP_LAUNCHED(c);
-    k_scan_sort<<<grid_for(n, SCAN_PTS), SCAN_CTA, 0, c->stream>>>(A);
-    MP_LAUNCHED(c);
-    return MP_OK;
+    return launch_scans(c, ScanArgs2{{A, A}}, 1);
 }
 
-// Point Gaussians of an arbitrary point array (the scan-Gaussian kernels
-// without the compaction): normals and validity of n points raw_dev (n x 3).
-int mp_launch_point_gaussians(mp_ctx* c, const float* raw_dev, int n, float4* tmp4, float* normals, uint8_t* valid) {
-    if (n == 0) return MP_OK;
-    ScanArgs A = scan_args(c, raw_dev, n);
-    A.tmp4 = tmp4;
-    A.normals = normals;
-    A.valid = valid;
-    A.pair = nullptr;
-    A.soa = nullptr;
-    A.nvalid = nullptr;
-    k_scan_to_float4<<<grid_for(n, 256), 256, 0, c->stream>>>(A);
-    MP_LAUNCHED(c);
-    k_scan_normals<<<grid_for(n, NRM_PTS), NRM_CTA, 0, c->stream>>>(A);
-    MP_LAUNCHED(c);
-    return MP_OK;
+// Point Gaussians of m <= 2 point arrays (n >= 1 points each): normals, validity, and
+// the valid points sorted into soa with their indices (idx may be null) and their number.
+int mp_launch_point_gaussians(mp_ctx* c, const PointScan* in, int m) {
+    ScanArgs2 A;
+    for (int k = 0; k < 2; ++k) {
+        const PointScan& p = in[k < m ? k : 0];
+        ScanArgs& a = A.s[k] = scan_args(c, p.raw, p.n);
+        a.tmp4 = p.tmp4;
+        a.normals = p.normals;
+        a.valid = p.valid;
+        a.pair = nullptr;
+        a.soa = p.soa;
+        a.idx = p.idx;
+        a.nvalid = p.nvalid;
+    }
+    return launch_scans(c, A, m);
 }
 
 // Grouped scan stage: every instance's scan is read from the batch's device

@@ -544,7 +544,16 @@ void fill_step_host(mp_ctx* c, StepDev* h);
 int upload_step(mp_ctx* c);
 int mp_launch_map_prepare(mp_ctx* c, const float* xyz_dev);
 int mp_launch_scan_prepare(mp_ctx* c);
-int mp_launch_point_gaussians(mp_ctx* c, const float* raw_dev, int n, float4* tmp4, float* normals, uint8_t* valid);
+struct PointScan {      // n x 3 points, and what is made of them
+    const float* raw;
+    int n;
+    float4* tmp4;
+    float* normals;
+    uint8_t* valid;
+    float* soa;
+    int32_t *idx, *nvalid;
+};
+int mp_launch_point_gaussians(mp_ctx* c, const PointScan* in, int m);
 int mp_launch_nnf_query(mp_ctx* c, const int32_t* vox_dev, int64_t m, int32_t* out_dev);
 // k_neighbors.cu
 int mp_launch_lsh_keys(mp_ctx* c);
