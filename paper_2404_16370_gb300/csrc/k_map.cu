@@ -151,6 +151,96 @@ __device__ void neighbourhood_normal(const float4* __restrict__ pts, Index J, in
     normal_of_cov(C, n_out);
 }
 
+// x / b, correctly rounded, from rb = 1 / b correctly rounded (Markstein 1990).
+__device__ __forceinline__ double div_by(double x, double b, double rb) {
+    const double q = x * rb;
+    return fma(fma(-b, q, x), rb, q);
+}
+__constant__ double nrm_inverse[MP_COVK + 1] = {0.,     1. / 1, 1. / 2,  1. / 3,  1. / 4,  1. / 5,  1. / 6,  1. / 7, 1. / 8,
+                                                1. / 9, 1. / 10, 1. / 11, 1. / 12, 1. / 13, 1. / 14, 1. / 15, 1. / 16};
+static_assert(MP_COVK == 16, "nrm_inverse");
+
+// The same normal, bit for bit, by four lanes: lane a of the quad works on
+// component or row a (the fourth as the third) and returns component a. m = 0: no
+// neighbours (the value is of no use). An FP64 instruction holds a quarter of the
+// SM for 64 cycles, whatever the number of active lanes: four warps of eight
+// points with the components side by side take half the instructions of a
+// chain that one warp of 32 points has on one quarter (10 us less for a scan).
+template <typename Index>
+__device__ __forceinline__ float neighbourhood_normal_quad(const float* __restrict__ raw, Index J, int m) {
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, quad = lane & ~3, a = min(lane & 3, 2);
+    auto get = [&](double x, int c) { return __shfl_sync(ALL, x, quad + c); };
+    const int most = __reduce_max_sync(ALL, m);
+    const double dm = m, rm = nrm_inverse[m];
+    double mean = 0.0, Cd = 0.0, Co = 0.0;   // Cd: entry (a, a), Co: entry (a, a + 1 mod 3)
+    for (int s = 0; s < most; ++s) mean += s < m ? (double)__ldg(raw + 3 * J(s) + a) : 0.0;
+    mean = div_by(mean, dm, rm);
+    for (int s = 0; s < most; ++s) {
+        const double d = s < m ? (double)__ldg(raw + 3 * J(s) + a) - mean : 0.0;
+        const double e = get(d, (a + 1) % 3);
+        Cd += d * d;
+        Co += d * e;
+    }
+    Cd = div_by(Cd, dm, rm);
+    Co = div_by(Co, dm, rm);
+    const double a00 = get(Cd, 0), a11 = get(Cd, 1), a22 = get(Cd, 2);
+    const double a01 = get(Co, 0), a12 = get(Co, 1), a02 = get(Co, 2);
+    const double sq = Co * Co, p1 = get(sq, 0) + get(sq, 2) + get(sq, 1);
+    const double q = div_by(a00 + a11 + a22, 3.0, 1.0 / 3.0);
+    const double b = Cd - q, bb = b * b;
+    const double p2 = get(bb, 0) + get(bb, 1) + get(bb, 2) + 2.0 * p1;
+    double lam;
+    {
+        const double p = sqrt(div_by(p2, 6.0, 1.0 / 6.0)), ip = 1.0 / p;
+        const double cb = b * ip, co = Co * ip;
+        const double c00 = get(cb, 0), c11 = get(cb, 1), c22 = get(cb, 2);
+        const double c01 = get(co, 0), c12 = get(co, 1), c02 = get(co, 2);
+        // the determinant's three terms
+        const double u = (a == 0 ? c11 : c01) * (a == 2 ? c12 : c22), w = (a == 2 ? c11 : c12) * (a == 0 ? c12 : c02);
+        const double t = (a == 0 ? c00 : a == 1 ? c01 : c02) * (u - w);
+        const double det = get(t, 0) - get(t, 1) + get(t, 2);
+        const double r = fmin(1.0, fmax(-1.0, 0.5 * det));
+        const double phi = div_by(acos(r), 3.0, 1.0 / 3.0);
+        lam = q + 2.0 * p * cos(phi + 2.0943951023931954923);   // + 2 pi / 3: the smallest root
+        if (p2 <= 0.0) lam = q;
+    }
+    double v = a == 2 ? 1.0 : 0.0;
+    bool stop = false;
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+        const double d = Cd - lam, d0 = get(d, 0), d1 = get(d, 1), d2 = get(d, 2);
+        // lane 0: rows 0 and 1, lane 1: 0 and 2, lane 2: 1 and 2
+        const double x0 = a == 2 ? a01 : d0, x1 = a == 2 ? d1 : a01, x2 = a == 2 ? a12 : a02;
+        const double y0 = a == 0 ? a01 : a02, y1 = a == 0 ? d1 : a12, y2 = a == 0 ? a12 : d2;
+        const double c0 = x1 * y2 - x2 * y1, c1 = x2 * y0 - x0 * y2, c2 = x0 * y1 - x1 * y0;
+        const double nn = c0 * c0 + c1 * c1 + c2 * c2;
+        const double n0 = get(nn, 0), n1 = get(nn, 1), n2 = get(nn, 2);
+        int best = 0;
+        double nb = n0;
+        if (n1 > nb) { best = 1; nb = n1; }
+        if (n2 > nb) { best = 2; nb = n2; }
+        if (!(nb > 0.0)) stop = true;   // (near) repeated smallest eigenvalue: keep v
+        const double sc = 1.0 / sqrt(nb);
+        const double e0 = get(c0, best), e1 = get(c1, best), e2 = get(c2, best);
+        const double nv = (a == 0 ? e0 : a == 1 ? e1 : e2) * sc;
+        if (!stop) v = nv;
+        if (it == 0) {
+            // Rayleigh quotient of the current vector refines lambda
+            const double v0 = get(v, 0), v1 = get(v, 1), v2 = get(v, 2);
+            const double Av = (a == 0 ? a00 : a == 1 ? a01 : a02) * v0 + (a == 0 ? a01 : a == 1 ? a11 : a12) * v1 +
+                              (a == 0 ? a02 : a == 1 ? a12 : a22) * v2;
+            const double t = v * Av;
+            lam = get(t, 0) + get(t, 1) + get(t, 2);
+        }
+    }
+    const double v0 = get(v, 0), v1 = get(v, 1), v2 = get(v, 2);
+    double big = v0;
+    if (fabs(v1) > fabs(big)) big = v1;
+    if (fabs(v2) > fabs(big)) big = v2;
+    return (float)(big < 0 ? -v : v);
+}
+
 // Map points: neighbourhoods through the cell grid.
 __global__ void k_map_normals(const float4* __restrict__ pts, int64_t n, CellGridDev g, float r2, int k, int kmin,
                               float* __restrict__ normals, uint8_t* __restrict__ valid) {
@@ -198,12 +288,13 @@ __global__ void k_map_normals(const float4* __restrict__ pts, int64_t n, CellGri
 // are selected (cov_k rounds of a warp minimum over (d, j)) and their last
 // distance becomes the new radius. The set and its order do not depend on the
 // order in which candidates are seen. The normals, in FP64 (1/75 of the FP32
-// rate), take one lane per point: a dense warp for the CTA's 32 points. What
-// bounds it: the distances (13 instructions a warp and 32 candidates) from a few
-// thousand points on, below that the FP64 chain of one normal.
+// rate), take four lanes per point. What bounds it: the distances (13
+// instructions a warp and 32 candidates) from a few thousand points on, below
+// that the FP64 chain of one normal.
 // Measured (the scan stage, against one thread per point and eighth of the scan
-// with a sorted list of its own, merged by one thread): 128 points 62 -> 42 us,
-// 2048 142 -> 60, 4999 178 -> 101, 8192 233 -> 145.
+// with a sorted list of its own, merged by one thread): 128 points 62 -> 32 us
+// (42 with a normal on one lane), 2048 142 -> 34 (60), 4999 178 -> 98 (101),
+// 8192 233 -> 143 (145).
 #define SCAN_TILE 1024
 #define SCAN_PARTS 8
 #define SCAN_CTA 256
@@ -298,7 +389,6 @@ __device__ __forceinline__ int select_nearest(uint64_t* buf, int n, int k, int l
 __device__ __forceinline__ void ScanNormalsOp::run(const ScanArgs& args, unsigned bx, unsigned) {
     const float* __restrict__ raw = args.raw;
     const int n = args.n, k = args.k, kmin = args.kmin;
-    const float4* __restrict__ tmp_pts = args.tmp4;
     float* __restrict__ normals = args.normals;
     uint8_t* __restrict__ valid = args.valid;
     __shared__ float sx[SCAN_TILE], sy[SCAN_TILE], sz[SCAN_TILE];
@@ -349,29 +439,20 @@ __device__ __forceinline__ void ScanNormalsOp::run(const ScanArgs& args, unsigne
         if (lane == 0) found[2 * w + q] = nb[q];
     }
     __syncthreads();
-    // the normals: one lane per point
-    if (threadIdx.x >= NRM_PTS) return;
-    const int q = threadIdx.x, iq = (int)bx * NRM_PTS + q;
-    if (iq >= n) return;
-    int m = found[q];
-    if (m < kmin) {
-        valid[iq] = 0;
-        normals[3 * iq] = normals[3 * iq + 1] = normals[3 * iq + 2] = 0.f;
-        return;
-    }
+    // the normals: four lanes per point, eight points a warp
+    if (threadIdx.x >= 4 * NRM_PTS) return;
+    const int q = threadIdx.x >> 2, iq = (int)bx * NRM_PTS + q;
+    int m = iq < n ? found[q] : 0;
+    if (m < kmin) m = 0;
     auto J = [&](int s) { return (int)(uint32_t)buf[q][s]; };
 #ifdef MP_CHECKED
     for (int s = 0; s < m; ++s)
         if (!MP_DCHECK(J(s) >= 0 && J(s) < n, "scan neighbour index", J(s))) m = 0;
-    if (m == 0) {
-        valid[iq] = 0;
-        return;
-    }
 #endif
-    float nv[3];
-    neighbourhood_normal(tmp_pts, J, m, nv);
-    normals[3 * iq] = nv[0]; normals[3 * iq + 1] = nv[1]; normals[3 * iq + 2] = nv[2];
-    valid[iq] = 1;
+    const float nv = neighbourhood_normal_quad(raw, J, m);
+    if (iq >= n) return;
+    if ((lane & 3) < 3) normals[3 * iq + (lane & 3)] = m > 0 ? nv : 0.f;
+    if ((lane & 3) == 0) valid[iq] = m > 0;
 }
 
 // Compaction: the valid points in the order of (key, index) into the chunks of
