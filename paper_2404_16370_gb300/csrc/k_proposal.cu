@@ -165,6 +165,122 @@ __global__ void __launch_bounds__(256) k_gemm(const float* __restrict__ A, const
     }
 }
 
+// The head's products, C[M x N] = op(A)[M x K] op(B)[K x N] with M, N or K the
+// batch: few rows, so what counts is latency and CTAs. A CTA of 128 threads takes
+// 16 x 32 outputs (4 a thread) and stages 128 of K at a time, whole slices in
+// flight at once. A 64 x 64 tile with 16 of K a step left 7 CTAs waiting for 16
+// loads in a row: 46 us for 4 x 416 x 256, 7 now; the six products and
+// four column sums and gates of a training step at batch 128 320 us, 44 now.
+// N and the extents along which op(A) and op(B) are contiguous are multiples of
+// 4, the matrices 16-byte aligned. Each output is one chain of fmaf over k.
+enum : int { HEAD_BIAS = 1, HEAD_RELU = 2, HEAD_GATE = 4, HEAD_COLSUM = 8 };
+constexpr int HM = 16, HN = 32, HK = 128;
+
+// aux: the bias [N] (HEAD_BIAS), or a matrix like C whose entries <= 0 zero the
+// output's (HEAD_GATE). colsum: column sums of op(B) (HEAD_COLSUM).
+template <bool TA, bool TB, int EPI>
+__global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const float* __restrict__ B,
+                                              float* __restrict__ C, const float* __restrict__ aux,
+                                              float* __restrict__ colsum, int M, int N, int K, int lda, int ldb,
+                                              int ldc) {
+    __shared__ __align__(16) float As[HM][HK + 4];
+    __shared__ __align__(16) float Bs[HK][HN + 4];
+    __shared__ float cs[4][HN];
+    const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
+    const int m0 = blockIdx.y * HM, n0 = blockIdx.x * HN;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, col = 0.f;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 ra[HM * HK / 512], rb[HN * HK / 512];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int e = 0; e < HM * HK / 512; ++e) {
+            const int v = e * 128 + tid;
+            if (TA) {   // A is [K][M]: 4 of m a thread, k along the lanes
+                const int k = k0 + v % HK, m = m0 + v / HK * 4;
+                ra[e] = k < K && m < M ? *reinterpret_cast<const float4*>(A + (int64_t)k * lda + m) : zero;
+            } else {
+                const int m = m0 + v / (HK / 4), k = k0 + v % (HK / 4) * 4;
+                ra[e] = k < K && m < M ? *reinterpret_cast<const float4*>(A + (int64_t)m * lda + k) : zero;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < HN * HK / 512; ++e) {
+            const int v = e * 128 + tid;
+            if (TB) {   // B is [N][K]: 4 of k a thread, n along the lanes
+                const int n = n0 + v % HN, k = k0 + v / HN * 4;
+                rb[e] = k < K && n < N ? *reinterpret_cast<const float4*>(B + (int64_t)n * ldb + k) : zero;
+            } else {
+                const int k = k0 + v / (HN / 4), n = n0 + v % (HN / 4) * 4;
+                rb[e] = k < K && n < N ? *reinterpret_cast<const float4*>(B + (int64_t)k * ldb + n) : zero;
+            }
+        }
+    };
+    load(0);
+    for (int k0 = 0; k0 < K; k0 += HK) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < HM * HK / 512; ++e) {
+            const int v = e * 128 + tid;
+            if (TA) {
+                const int k = v % HK, m = v / HK * 4;
+                As[m][k] = ra[e].x; As[m + 1][k] = ra[e].y; As[m + 2][k] = ra[e].z; As[m + 3][k] = ra[e].w;
+            } else {
+                *reinterpret_cast<float4*>(&As[v / (HK / 4)][v % (HK / 4) * 4]) = ra[e];
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < HN * HK / 512; ++e) {
+            const int v = e * 128 + tid;
+            if (TB) {
+                const int n = v % HN, k = v / HN * 4;
+                Bs[k][n] = rb[e].x; Bs[k + 1][n] = rb[e].y; Bs[k + 2][n] = rb[e].z; Bs[k + 3][n] = rb[e].w;
+            } else {
+                *reinterpret_cast<float4*>(&Bs[v / (HN / 4)][v % (HN / 4) * 4]) = rb[e];
+            }
+        }
+        __syncthreads();
+        if (k0 + HK < K) load(k0 + HK);
+        const int ke = min(HK, (K - k0 + 3) & ~3);   // beyond K both are 0
+#pragma unroll 4
+        for (int k = 0; k < ke; k += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(&As[ty][k]);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 b = *reinterpret_cast<const float4*>(&Bs[k + q][tx * 4]);
+                acc[0] = fmaf(av[q], b.x, acc[0]);
+                acc[1] = fmaf(av[q], b.y, acc[1]);
+                acc[2] = fmaf(av[q], b.z, acc[2]);
+                acc[3] = fmaf(av[q], b.w, acc[3]);
+            }
+        }
+        if ((EPI & HEAD_COLSUM) && m0 == 0)
+            for (int k = tid / HN * (HK / 4); k < (tid / HN + 1) * (HK / 4); ++k) col += Bs[k][tid % HN];
+    }
+    if ((EPI & HEAD_COLSUM) && m0 == 0) {
+        cs[tid / HN][tid % HN] = col;
+        __syncthreads();
+        if (tid < HN && n0 + tid < N) colsum[n0 + tid] = cs[0][tid] + cs[1][tid] + cs[2][tid] + cs[3][tid];
+    }
+    const int m = m0 + ty, n = n0 + tx * 4;
+    if (m >= M || n >= N) return;
+    if (EPI & HEAD_BIAS) {
+        const float4 b = *reinterpret_cast<const float4*>(aux + n);
+        acc[0] += b.x; acc[1] += b.y; acc[2] += b.z; acc[3] += b.w;
+    }
+    if (EPI & HEAD_GATE) {
+        const float4 h = *reinterpret_cast<const float4*>(aux + (int64_t)m * ldc + n);
+        if (!(h.x > 0.f)) acc[0] = 0.f;
+        if (!(h.y > 0.f)) acc[1] = 0.f;
+        if (!(h.z > 0.f)) acc[2] = 0.f;
+        if (!(h.w > 0.f)) acc[3] = 0.f;
+    }
+    if (EPI & HEAD_RELU)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = fmaxf(acc[j], 0.f);
+    *reinterpret_cast<float4*>(C + (int64_t)m * ldc + n) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+}
+
 // column sums of X [rows x n] added into out (bias gradients)
 __global__ void k_colsum(const float* __restrict__ X, int64_t rows, int n, int rows_per_cta, float* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -245,57 +361,47 @@ __device__ __forceinline__ float wrap_pi(float a) {
 }
 
 // Mixture negative log-likelihood of each sample and its gradient w.r.t. o,
-// scaled by 1/B (mean loss).
-__global__ void k_mdn_loss(const float* __restrict__ o, const float* __restrict__ y, int B,
-                           float* __restrict__ dO, float* __restrict__ loss) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// scaled by 1/B (mean loss). A warp takes a sample, a lane a component (one
+// thread a sample, components in turn: 80 us at batch 128, 4 now).
+__global__ void __launch_bounds__(64) k_mdn_loss(const float* __restrict__ o, const float* __restrict__ y, int B,
+                                                 float* __restrict__ dO, float* __restrict__ loss) {
+    static_assert(NCOMP == 32, "a lane per component");
+    const int b = blockIdx.x * 2 + (threadIdx.x >> 5), c = threadIdx.x & 31;
     if (b >= B) return;
     const float* ob = o + (int64_t)b * NOUT;
     float* db = dO + (int64_t)b * NOUT;
-    float yy[6];
+    auto warp_max = [](float v) {
 #pragma unroll
-    for (int d = 0; d < 6; ++d) yy[d] = y[b * 6 + d];
+        for (int k = 16; k > 0; k >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, k));
+        return v;
+    };
     // log pi = a - logsumexp(a)
-    float amax = -INFINITY;
-    for (int c = 0; c < NCOMP; ++c) amax = fmaxf(amax, ob[c]);
-    float asum = 0.f;
-    for (int c = 0; c < NCOMP; ++c) asum += expf(ob[c] - amax);
-    const float lse_a = amax + logf(asum);
-    float lj[NCOMP];
-    float jmax = -INFINITY;
+    const float a = ob[c];
+    const float amax = warp_max(a);
+    const float lse_a = amax + logf(warp_sum(expf(a - amax)));
     const float half_log_2pi6 = 3.f * 1.8378770664093453f;
-    for (int c = 0; c < NCOMP; ++c) {
-        float s = 0.f;
+    float th[6], dl[6], s = 0.f;
 #pragma unroll
-        for (int d = 0; d < 6; ++d) {
-            const float ls = LOGSTD_LIM * tanhf(ob[224 + 6 * c + d] / LOGSTD_LIM);
-            float dl = yy[d] - ob[32 + 6 * c + d];
-            if (d == 3) dl = wrap_pi(dl);
-            const float z = dl * expf(-ls);
-            s += -0.5f * z * z - ls;
-        }
-        lj[c] = ob[c] - lse_a + s - half_log_2pi6;
-        jmax = fmaxf(jmax, lj[c]);
+    for (int d = 0; d < 6; ++d) {
+        th[d] = tanhf(ob[224 + 6 * c + d] / LOGSTD_LIM);
+        const float ls = LOGSTD_LIM * th[d];
+        dl[d] = y[b * 6 + d] - ob[32 + 6 * c + d];
+        if (d == 3) dl[d] = wrap_pi(dl[d]);
+        const float z = dl[d] * expf(-ls);
+        s += -0.5f * z * z - ls;
     }
-    float jsum = 0.f;
-    for (int c = 0; c < NCOMP; ++c) jsum += expf(lj[c] - jmax);
-    const float L = -(jmax + logf(jsum));
-    atomicAdd(loss, L / B);
+    const float lj = a - lse_a + s - half_log_2pi6;
+    const float jmax = warp_max(lj);
+    const float L = -(jmax + logf(warp_sum(expf(lj - jmax))));
+    if (c == 0) atomicAdd(loss, L / B);
     const float invB = 1.f / B;
-    for (int c = 0; c < NCOMP; ++c) {
-        const float r = expf(lj[c] + L);               // responsibility
-        const float pi = expf(ob[c] - lse_a);
-        db[c] = (pi - r) * invB;
+    const float r = expf(lj + L);               // responsibility
+    db[c] = (expf(a - lse_a) - r) * invB;
 #pragma unroll
-        for (int d = 0; d < 6; ++d) {
-            const float th = tanhf(ob[224 + 6 * c + d] / LOGSTD_LIM);
-            const float ls = LOGSTD_LIM * th;
-            float dl = yy[d] - ob[32 + 6 * c + d];
-            if (d == 3) dl = wrap_pi(dl);
-            const float iv = expf(-2.f * ls);
-            db[32 + 6 * c + d] = -r * dl * iv * invB;
-            db[224 + 6 * c + d] = r * (1.f - dl * dl * iv) * (1.f - th * th) * invB;
-        }
+    for (int d = 0; d < 6; ++d) {
+        const float iv = expf(-2.f * (LOGSTD_LIM * th[d]));
+        db[32 + 6 * c + d] = -r * dl[d] * iv * invB;
+        db[224 + 6 * c + d] = r * (1.f - dl[d] * dl[d] * iv) * (1.f - th[d] * th[d]) * invB;
     }
 }
 
@@ -413,6 +519,15 @@ void gemm(cudaStream_t s, const float* A, const float* B, float* C, const float*
     k_gemm<TA, TB, EPI><<<grid, 256, 0, s>>>(A, B, C, bias, M, N, K, lda, ldb, ldc, kchunk);
 }
 
+template <bool TA, bool TB, int EPI>
+void head(cudaStream_t s, const float* A, const float* B, float* C, const float* aux, float* colsum, int M, int N, int K,
+          int lda, int ldb, int ldc) {
+    static_assert(OB1 % 4 == 0 && OW4 % 4 == 0 && OB4 % 4 == 0 && OW5 % 4 == 0 && OB5 % 4 == 0 && NOUT % 4 == 0,
+                  "k_head's loads of four floats");
+    const dim3 grid((N + HN - 1) / HN, (M + HM - 1) / HM);
+    k_head<TA, TB, EPI><<<grid, 128, 0, s>>>(A, B, C, aux, colsum, M, N, K, lda, ldb, ldc);
+}
+
 // split count for a weight gradient that reduces over `rows` rows: enough
 // CTAs to fill the GPU (~4 per SM)
 int splits_for(int64_t rows, int M, int N) {
@@ -451,8 +566,8 @@ int forward(mp_pn* net, const float* scans, int B, bool train) {
         gemm<false, false, EPI_BIAS | EPI_RELU>(s, net->h2, W + OW3, net->h3, W + OB3, (int)rows, C3, C2, C2, C3, C3);
         k_maxpool<<<dim3(C3 / 128, B), 128, 0, s>>>(net->h3, B, net->P, net->g, net->gi);
     }
-    gemm<false, false, EPI_BIAS | EPI_RELU>(s, net->g, W + OW4, net->h4, W + OB4, B, C4, C3, C3, C4, C4);
-    gemm<false, false, EPI_BIAS>(s, net->h4, W + OW5, net->o, W + OB5, B, NOUT, C4, C4, NOUT, NOUT);
+    head<false, false, HEAD_BIAS | HEAD_RELU>(s, net->g, W + OW4, net->h4, W + OB4, nullptr, B, C4, C3, C3, C4, C4);
+    head<false, false, HEAD_BIAS>(s, net->h4, W + OW5, net->o, W + OB5, nullptr, B, NOUT, C4, C4, NOUT, NOUT);
     PN_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -568,15 +683,12 @@ int mp_pn_loss_grad(mp_pn* net, const float* scans, const float* targets, int B,
     float* G = net->grad;
     PN_CUDA(cudaMemsetAsync(G, 0, sizeof(float) * NPARAM, s));
     PN_CUDA(cudaMemsetAsync(loss_dev, 0, sizeof(float), s));
-    k_mdn_loss<<<grid_for(B, 64), 64, 0, s>>>(net->o, targets, B, net->dO, loss_dev);
+    k_mdn_loss<<<grid_for(B, 2), 64, 0, s>>>(net->o, targets, B, net->dO, loss_dev);
     // head
-    gemm<true, false, EPI_ATOMIC>(s, net->h4, net->dO, G + OW5, nullptr, C4, NOUT, B, C4, NOUT, NOUT);
-    colsum(s, net->dO, B, NOUT, G + OB5);
-    gemm<false, true, 0>(s, net->dO, W + OW5, net->dh4, nullptr, B, C4, NOUT, NOUT, NOUT, C4);
-    k_relu_back<<<grid_for((int64_t)B * C4, 256), 256, 0, s>>>(net->dh4, net->h4, (int64_t)B * C4);
-    gemm<true, false, EPI_ATOMIC>(s, net->g, net->dh4, G + OW4, nullptr, C3, C4, B, C3, C4, C4);
-    colsum(s, net->dh4, B, C4, G + OB4);
-    gemm<false, true, 0>(s, net->dh4, W + OW4, net->dg, nullptr, B, C3, C4, C4, C4, C3);
+    head<true, false, HEAD_COLSUM>(s, net->h4, net->dO, G + OW5, nullptr, G + OB5, C4, NOUT, B, C4, NOUT, NOUT);
+    head<false, true, HEAD_GATE>(s, net->dO, W + OW5, net->dh4, net->h4, nullptr, B, C4, NOUT, NOUT, NOUT, C4);
+    head<true, false, HEAD_COLSUM>(s, net->g, net->dh4, G + OW4, nullptr, G + OB4, C3, C4, B, C3, C4, C4);
+    head<false, true, 0>(s, net->dh4, W + OW4, net->dg, nullptr, nullptr, B, C3, C4, C4, C4, C3);
     // max-pool and the shared layers, on the pooled rows (b, channel) only
     const int64_t rows_c = (int64_t)B * C3;
     k_dw3<<<C3, C2, 0, s>>>(net->dg, net->g, net->gi, net->h2, B, net->P, G + OW3, G + OB3);
