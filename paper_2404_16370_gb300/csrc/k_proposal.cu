@@ -3,14 +3,11 @@
 // definition are in include/mp_proposal.h.
 //
 // Layout: activations row-major [rows][channels] in FP32, rows = batch x
-// points for the shared per-point layers and = batch for the head. Every
-// dense layer of the FP32 form is one tiled GEMM (64 x 64 output tile per
-// CTA, 16-deep K slices in shared memory, 4 x 4 outputs per thread) with the
-// bias and ReLU fused into the store; weight gradients reduce over rows with
-// split-K CTAs adding into the gradient by atomics. The BF16 form's forward
-// pass through the per-point layers is one tensor-core kernel (k_pn_tc.cu).
-// The backward pass through the per-point layers runs on the max-pooled rows
-// only (k_pool_rows).
+// points for the shared per-point layers and = batch for the head. The FP32
+// form's per-point layers are tiled products (k_gemm) and a max over points, the
+// BF16 form's one tensor-core kernel (k_pn_tc.cu). The head's products are
+// k_head's, and the backward pass through the per-point layers runs on the
+// max-pooled rows only, in one kernel (k_pool_back).
 #include "mp_internal.cuh"
 #include "../../include/mp_proposal.h"
 
@@ -96,39 +93,29 @@ __global__ void k_sim_box_room(const float* __restrict__ boxes, int n_boxes, flo
 }
 
 // ---------------------------------------------------------------------------
-// dense layers: C[M x N] (+)= op(A)[M x K] op(B)[K x N], op = transpose when
-// TA / TB; A is [M][K] (or [K][M]), B is [K][N] (or [N][K]).
-enum : int { EPI_BIAS = 1, EPI_RELU = 2, EPI_ATOMIC = 4 };
+// per-point layers of the FP32 form: C[M x N] = relu(A[M x K] B[K x N] + bias)
 constexpr int GT = 64, GK = 16;
 
-template <bool TA, bool TB, int EPI>
 __global__ void __launch_bounds__(256) k_gemm(const float* __restrict__ A, const float* __restrict__ B,
                                               float* __restrict__ C, const float* __restrict__ bias, int M, int N,
-                                              int K, int lda, int ldb, int ldc, int kchunk) {
+                                              int K) {
     __shared__ float As[GK][GT + 4];
     __shared__ float Bs[GK][GT + 4];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
     const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     float acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int k0 = kb; k0 < ke; k0 += GK) {
+    for (int k0 = 0; k0 < K; k0 += GK) {
         for (int e = threadIdx.x; e < GT * GK; e += 256) {
-            const int mm = TA ? e % GT : e / GK, kk = TA ? e / GT : e % GK;
-            const int m = m0 + mm, k = k0 + kk;
-            float v = 0.f;
-            if (m < M && k < ke) v = TA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k];
-            As[kk][mm] = v;
+            const int m = m0 + e / GK, k = k0 + e % GK;
+            As[e % GK][e / GK] = m < M && k < K ? A[(int64_t)m * K + k] : 0.f;
         }
         for (int e = threadIdx.x; e < GT * GK; e += 256) {
-            const int nn = TB ? e / GK : e % GT, kk = TB ? e % GK : e / GT;
-            const int n = n0 + nn, k = k0 + kk;
-            float v = 0.f;
-            if (n < N && k < ke) v = TB ? B[(int64_t)n * ldb + k] : B[(int64_t)k * ldb + n];
-            Bs[kk][nn] = v;
+            const int n = n0 + e % GT, k = k0 + e / GT;
+            Bs[e / GT][e % GT] = n < N && k < K ? B[(int64_t)k * N + n] : 0.f;
         }
         __syncthreads();
 #pragma unroll
@@ -152,15 +139,7 @@ __global__ void __launch_bounds__(256) k_gemm(const float* __restrict__ A, const
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (EPI & EPI_ATOMIC) {
-                atomicAdd(C + (int64_t)m * ldc + n, v);
-            } else {
-                if (EPI & EPI_BIAS) v += bias[n];
-                if (EPI & EPI_RELU) v = fmaxf(v, 0.f);
-                C[(int64_t)m * ldc + n] = v;
-            }
+            if (n < N) C[(int64_t)m * N + n] = fmaxf(acc[i][j] + bias[n], 0.f);
         }
     }
 }
@@ -281,22 +260,6 @@ __global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const
     *reinterpret_cast<float4*>(C + (int64_t)m * ldc + n) = make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
 
-// column sums of X [rows x n] added into out (bias gradients)
-__global__ void k_colsum(const float* __restrict__ X, int64_t rows, int n, int rows_per_cta, float* __restrict__ out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const int64_t r0 = (int64_t)blockIdx.y * rows_per_cta, r1 = min(rows, r0 + rows_per_cta);
-    float s = 0.f;
-    for (int64_t r = r0; r < r1; ++r) s += X[r * n + c];
-    atomicAdd(out + c, s);
-}
-
-// dX = dH where H > 0 else 0 (ReLU backward, in place)
-__global__ void k_relu_back(float* __restrict__ dH, const float* __restrict__ H, int64_t n) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n && !(H[i] > 0.f)) dH[i] = 0.f;
-}
-
 __global__ void k_scale_points(const float* __restrict__ x, int64_t n, float inv, float* __restrict__ y) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) y[i] = x[i] * inv;
@@ -318,40 +281,169 @@ __global__ void k_maxpool(const float* __restrict__ h3, int B, int P, float* __r
     gi[b * C3 + c] = mi;
 }
 
-__global__ void k_pool_rows(const float* __restrict__ dg, const float* __restrict__ g, const int* __restrict__ gi,
-                            const float* __restrict__ xs, const float* __restrict__ h1, const float* __restrict__ h2,
-                            const float* __restrict__ W3, int B, int P, float* __restrict__ xc,
-                            float* __restrict__ h1c, float* __restrict__ h2c, float* __restrict__ dh2c) {
-    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // r = b * 256 + c
-    if (r >= (int64_t)B * C3) return;
-    const int64_t b = r / C3;
-    const int c = (int)(r % C3);
-    const float d = g[r] > 0.f ? dg[r] : 0.f;
-    const int64_t row = b * P + gi[r];
-    for (int k = 0; k < 3; ++k) xc[r * 3 + k] = xs[row * 3 + k];
-    for (int k = 0; k < C1; ++k) h1c[r * C1 + k] = h1[row * C1 + k];
-    for (int i = 0; i < C2; ++i) {
-        const float h = h2[row * C2 + i];
-        h2c[r * C2 + i] = h;
-        dh2c[r * C2 + i] = h > 0.f ? d * W3[i * C3 + c] : 0.f;
-    }
-}
+// Backward pass of the shared layers on the pooled rows (c, b): channel c of
+// sample b reaches them through its maximum's point alone, whose x, h1 and h2 it
+// reads back. Per row, with d = dg[b][c] where g > 0:
+//   dW3[i][c] += d h2[i], db3[c] += d, dh2[i] = d W3[i][c] where h2[i] > 0,
+//   db2 += dh2, dW2[j][i] += h1[j] dh2[i], dh1[j] = sum_i dh2[i] W2[j][i] where
+//   h1[j] > 0, db1 += dh1, dW1[k][j] += x[k] dh1[j].
+// Resident CTAs take tiles of 64 rows in the order of c, so that a tile of a
+// large batch has one column of W3; h2, dh2 and dh1 stay on chip and dW1, dW2,
+// db1 and db2 in registers until the CTA is done. Bound by the FP32 products (1.1
+// GFLOP at batch 128) and their shared-memory reads. As nine kernels that passed
+// the rows' h1, h2, dh1 and dh2 through memory, batch 128 took 360 us; 48 now.
+struct PoolArgs {
+    const float *dg, *g, *x, *h1, *h2, *W2, *W3;
+    const int* gi;
+    float inv;            // scale of x
+    int B, P;
+    float *dW1, *db1, *dW2, *db2, *dW3, *db3;
+};
+constexpr int PR = 64, PTH = 256;                                  // rows of a tile, threads
+constexpr int LD_H2 = C2 + 4, LD_H1 = C1 + 4;                      // padded rows
+constexpr int POOL_SMEM = 4 * (PR * LD_H2 + PR * LD_H1 + C2 * LD_H1 + PR * 4 + 2 * PR) + 4 * PR;
 
-// dW3[i][c] += sum_b dg[b][c] h2[b, gi[b][c], i] (pooled, gated) and db3[c]
-__global__ void k_dw3(const float* __restrict__ dg, const float* __restrict__ g, const int* __restrict__ gi,
-                      const float* __restrict__ h2, int B, int P, float* __restrict__ dW3, float* __restrict__ db3) {
-    const int c = blockIdx.x;          // channel
-    const int i = threadIdx.x;         // input channel (C2 threads)
-    float acc = 0.f, bacc = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const int64_t r = (int64_t)b * C3 + c;
-        if (!(g[r] > 0.f)) continue;
-        const float d = dg[r];
-        acc = fmaf(d, h2[((int64_t)b * P + gi[r]) * C2 + i], acc);
-        bacc += d;
+__global__ void __launch_bounds__(PTH, 2) k_pool_back(const PoolArgs A) {
+    extern __shared__ __align__(16) float pool_smem[];
+    float* dh2s = pool_smem;                  // [row][i]
+    float* h1s = dh2s + PR * LD_H2;           // [row][j]
+    float* W2s = h1s + PR * LD_H1;            // [i][j]
+    float* xs = W2s + C2 * LD_H1;             // [row][x, y, z, -]
+    float* ds = xs + PR * 4;                  // [row] d
+    int* cs = reinterpret_cast<int*>(ds + PR);   // [row] channel
+    int* ps = cs + PR;                           // [row] the point's row
+    const int tid = threadIdx.x;
+    for (int e = tid; e < C1 * C2; e += PTH) W2s[e % C2 * LD_H1 + e / C2] = A.W2[e];
+    const int tx = tid % 16, ty = tid / 16;
+    float acc2[4][8], acc1[4][4], b2 = 0.f;   // dW2[4 tx + .][..], (dW1, db1)[4 tx + .], db2 of the thread's i
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc2[j][i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc1[j][k] = 0.f;
     }
-    dW3[i * C3 + c] += acc;
-    if (i == 0) db3[c] += bacc;
+    const int rows = A.B * C3, ntile = (rows + PR - 1) / PR;
+    const int i2 = tid % C2, half = tid / C2;
+    for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+        __syncthreads();
+        if (tid < PR) {
+            const int r = t * PR + tid, c = min(r, rows - 1) / A.B, b = min(r, rows - 1) % A.B;
+            const float gv = A.g[b * C3 + c];
+            const int point = b * A.P + A.gi[b * C3 + c];
+            ds[tid] = r < rows && gv > 0.f ? A.dg[b * C3 + c] : 0.f;
+            cs[tid] = c;
+            ps[tid] = point;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) xs[tid * 4 + k] = A.x[(int64_t)point * 3 + k] * A.inv;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < PR * C1 / 4 / PTH; ++e) {
+            const int v = e * PTH + tid, r = v / (C1 / 4), j = v % (C1 / 4) * 4;
+            *reinterpret_cast<float4*>(h1s + r * LD_H1 + j) =
+                *reinterpret_cast<const float4*>(A.h1 + (int64_t)ps[r] * C1 + j);
+        }
+        // h2: a thread has one i and half of the rows
+        {
+            int c = cs[half * (PR / 2)];
+            float w = __ldg(A.W3 + i2 * C3 + c), a3 = 0.f, a3b = 0.f;
+            auto flush = [&] {
+                atomicAdd(A.dW3 + i2 * C3 + c, a3);
+                if (i2 == 0) atomicAdd(A.db3 + c, a3b);
+            };
+            for (int q0 = 0; q0 < PR / 2; q0 += 8) {
+                const int r0 = half * (PR / 2) + q0;
+                float h[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) h[q] = __ldg(A.h2 + (int64_t)ps[r0 + q] * C2 + i2);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int r = r0 + q;
+                    if (cs[r] != c) {
+                        flush();
+                        c = cs[r];
+                        w = __ldg(A.W3 + i2 * C3 + c);
+                        a3 = a3b = 0.f;
+                    }
+                    const float d = ds[r];
+                    a3 = fmaf(d, h[q], a3);
+                    a3b += d;
+                    const float dh = h[q] > 0.f ? d * w : 0.f;
+                    b2 += dh;
+                    dh2s[r * LD_H2 + i2] = dh;
+                }
+            }
+            flush();
+        }
+        __syncthreads();
+        // dh1 of rows 4 ty + ., channels 4 tx + .
+        float dh1[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dh1[r][j] = 0.f;
+#pragma unroll 2
+        for (int i = 0; i < C2; i += 4) {
+            float a[4][4], w[4][4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                *reinterpret_cast<float4*>(a[r]) = *reinterpret_cast<const float4*>(dh2s + (4 * ty + r) * LD_H2 + i);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                *reinterpret_cast<float4*>(w[k]) = *reinterpret_cast<const float4*>(W2s + (i + k) * LD_H1 + 4 * tx);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) dh1[r][j] = fmaf(a[r][k], w[k][j], dh1[r][j]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float4 h = *reinterpret_cast<const float4*>(h1s + (4 * ty + r) * LD_H1 + 4 * tx);
+            const float hv[4] = {h.x, h.y, h.z, h.w};
+            const float4 x = *reinterpret_cast<const float4*>(xs + (4 * ty + r) * 4);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float v = hv[j] > 0.f ? dh1[r][j] : 0.f;
+                acc1[j][0] = fmaf(x.x, v, acc1[j][0]);
+                acc1[j][1] = fmaf(x.y, v, acc1[j][1]);
+                acc1[j][2] = fmaf(x.z, v, acc1[j][2]);
+                acc1[j][3] += v;
+            }
+        }
+        // dW2[4 tx + .][4 ty + . and 64 + 4 ty + .]
+#pragma unroll 4
+        for (int r = 0; r < PR; ++r) {
+            float h[4], u[8];
+            *reinterpret_cast<float4*>(h) = *reinterpret_cast<const float4*>(h1s + r * LD_H1 + 4 * tx);
+            *reinterpret_cast<float4*>(u) = *reinterpret_cast<const float4*>(dh2s + r * LD_H2 + 4 * ty);
+            *reinterpret_cast<float4*>(u + 4) = *reinterpret_cast<const float4*>(dh2s + r * LD_H2 + 64 + 4 * ty);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc2[j][i] = fmaf(h[j], u[i], acc2[j][i]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            atomicAdd(reinterpret_cast<float4*>(A.dW2 + (4 * tx + j) * C2 + 64 * q + 4 * ty),
+                      make_float4(acc2[j][4 * q], acc2[j][4 * q + 1], acc2[j][4 * q + 2], acc2[j][4 * q + 3]));
+    atomicAdd(A.db2 + i2, b2);
+    // dW1 and db1: the sums over the 16 ty, through shared memory
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dh2s[(ty * 4 + k) * C1 + 4 * tx + j] = acc1[j][k];
+    __syncthreads();
+    const int j = tid % C1, k = tid / C1;
+    float v = 0.f;
+    for (int q = 0; q < 16; ++q) v += dh2s[(q * 4 + k) * C1 + j];
+    atomicAdd(k < 3 ? A.dW1 + k * C1 + j : A.db1 + j, v);
 }
 
 __device__ __forceinline__ float wrap_pi(float a) {
@@ -490,7 +582,7 @@ struct mp_pn {
     float *xs, *h1, *h2, *h3, *g, *h4, *o;
     int* gi;
     float *dO, *dh4, *dg;
-    float *xc, *h1c, *h2c, *dh2c, *dh1c;   // compact rows (b, channel) of the backward pass
+    int pool_grid;     // resident CTAs of k_pool_back
     uint2 key;
     int prec;          // MP_PREC_BF16: per-point layers on the tensor cores; MP_PREC_FP32: CUDA cores
     uint8_t* wimg;     // BF16 image of W2^T and W3^T for the tensor-core kernel
@@ -510,13 +602,8 @@ int pn_fail(const char* what, cudaError_t e) {
         if (e_ != cudaSuccess) return pn_fail(#x, e_); \
     } while (0)
 
-template <bool TA, bool TB, int EPI>
-void gemm(cudaStream_t s, const float* A, const float* B, float* C, const float* bias, int M, int N, int K, int lda,
-          int ldb, int ldc, int splits = 1) {
-    const int kchunk = ((K + splits - 1) / splits + GK - 1) / GK * GK;
-    const int nz = (K + kchunk - 1) / kchunk;
-    dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, nz);
-    k_gemm<TA, TB, EPI><<<grid, 256, 0, s>>>(A, B, C, bias, M, N, K, lda, ldb, ldc, kchunk);
+void gemm(cudaStream_t s, const float* A, const float* B, float* C, const float* bias, int M, int N, int K) {
+    k_gemm<<<dim3((N + GT - 1) / GT, (M + GT - 1) / GT), 256, 0, s>>>(A, B, C, bias, M, N, K);
 }
 
 template <bool TA, bool TB, int EPI>
@@ -526,21 +613,6 @@ void head(cudaStream_t s, const float* A, const float* B, float* C, const float*
                   "k_head's loads of four floats");
     const dim3 grid((N + HN - 1) / HN, (M + HM - 1) / HM);
     k_head<TA, TB, EPI><<<grid, 128, 0, s>>>(A, B, C, aux, colsum, M, N, K, lda, ldb, ldc);
-}
-
-// split count for a weight gradient that reduces over `rows` rows: enough
-// CTAs to fill the GPU (~4 per SM)
-int splits_for(int64_t rows, int M, int N) {
-    const int64_t tiles = (int64_t)((M + GT - 1) / GT) * ((N + GT - 1) / GT);
-    int64_t s = (4 * 152 + tiles - 1) / tiles;
-    s = std::min<int64_t>(s, std::max<int64_t>(1, rows / 256));
-    return (int)std::max<int64_t>(1, s);
-}
-
-void colsum(cudaStream_t s, const float* X, int64_t rows, int n, float* out) {
-    const int rpc = 512;
-    dim3 grid((n + 127) / 128, (unsigned)((rows + rpc - 1) / rpc));
-    k_colsum<<<grid, 128, 0, s>>>(X, rows, n, rpc, out);
 }
 
 // BF16 image of the per-point weights, refreshed after every parameter update
@@ -561,9 +633,9 @@ int forward(mp_pn* net, const float* scans, int B, bool train) {
                                         MP_WAIT_BUDGET, s);
         if (rc) return mp_fail_noctx(rc, "mp_pn: tensor-core forward launch failed");
     } else {
-        gemm<false, false, EPI_BIAS | EPI_RELU>(s, net->xs, W + OW1, net->h1, W + OB1, (int)rows, C1, 3, 3, C1, C1);
-        gemm<false, false, EPI_BIAS | EPI_RELU>(s, net->h1, W + OW2, net->h2, W + OB2, (int)rows, C2, C1, C1, C2, C2);
-        gemm<false, false, EPI_BIAS | EPI_RELU>(s, net->h2, W + OW3, net->h3, W + OB3, (int)rows, C3, C2, C2, C3, C3);
+        gemm(s, net->xs, W + OW1, net->h1, W + OB1, (int)rows, C1, 3);
+        gemm(s, net->h1, W + OW2, net->h2, W + OB2, (int)rows, C2, C1);
+        gemm(s, net->h2, W + OW3, net->h3, W + OB3, (int)rows, C3, C2);
         k_maxpool<<<dim3(C3 / 128, B), 128, 0, s>>>(net->h3, B, net->P, net->g, net->gi);
     }
     head<false, false, HEAD_BIAS | HEAD_RELU>(s, net->g, W + OW4, net->h4, W + OB4, nullptr, B, C4, C3, C3, C4, C4);
@@ -610,10 +682,13 @@ int mp_pn_create(mp_pn** netp, int n_points, int max_batch, float in_scale, cons
     A(&net->g, (size_t)max_batch * C3); A(&net->gi, (size_t)max_batch * C3); A(&net->h4, (size_t)max_batch * C4);
     A(&net->o, (size_t)max_batch * NOUT); A(&net->dO, (size_t)max_batch * NOUT);
     A(&net->dh4, (size_t)max_batch * C4); A(&net->dg, (size_t)max_batch * C3);
-    const int64_t rows_c = (int64_t)max_batch * C3;
-    A(&net->xc, rows_c * 3); A(&net->h1c, rows_c * C1); A(&net->h2c, rows_c * C2); A(&net->dh2c, rows_c * C2);
-    A(&net->dh1c, rows_c * C1);
     A(&net->wimg, mp_pn_tc_image_bytes()); A(&net->err, 1);
+    int dev = 0, sms = 0, per = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pool_back, cudaFuncAttributeMaxDynamicSharedMemorySize, POOL_SMEM);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pool_back, PTH, POOL_SMEM);
+    net->pool_grid = std::max(1, sms * per);
     if (e != cudaSuccess) {
         mp_pn_destroy(net);
         return pn_fail("allocation", e);
@@ -636,8 +711,7 @@ int mp_pn_create(mp_pn** netp, int n_points, int max_batch, float in_scale, cons
 int mp_pn_destroy(mp_pn* net) {
     if (!net) return mp_fail_noctx(MP_EINVAL, "mp_pn_destroy: invalid argument");
     void* bufs[] = {net->scale, net->offset, net->param, net->grad, net->am, net->av, net->xs, net->h1,
-                    net->h2, net->h3, net->g, net->gi, net->h4, net->o, net->dO, net->dh4, net->dg, net->xc,
-                    net->h1c, net->h2c, net->dh2c, net->dh1c, net->wimg, net->err};
+                    net->h2, net->h3, net->g, net->gi, net->h4, net->o, net->dO, net->dh4, net->dg, net->wimg, net->err};
     for (void* p : bufs)
         if (p) cudaFree(p);
     delete net;
@@ -678,7 +752,6 @@ int mp_pn_loss_grad(mp_pn* net, const float* scans, const float* targets, int B,
     int rc = forward(net, scans, B, true);
     if (rc) return rc;
     cudaStream_t s = net->stream;
-    const int64_t rows = (int64_t)B * net->P;
     const float* W = net->param;
     float* G = net->grad;
     PN_CUDA(cudaMemsetAsync(G, 0, sizeof(float) * NPARAM, s));
@@ -689,19 +762,15 @@ int mp_pn_loss_grad(mp_pn* net, const float* scans, const float* targets, int B,
     head<false, true, HEAD_GATE>(s, net->dO, W + OW5, net->dh4, net->h4, nullptr, B, C4, NOUT, NOUT, NOUT, C4);
     head<true, false, HEAD_COLSUM>(s, net->g, net->dh4, G + OW4, nullptr, G + OB4, C3, C4, B, C3, C4, C4);
     head<false, true, 0>(s, net->dh4, W + OW4, net->dg, nullptr, nullptr, B, C3, C4, C4, C4, C3);
-    // max-pool and the shared layers, on the pooled rows (b, channel) only
-    const int64_t rows_c = (int64_t)B * C3;
-    k_dw3<<<C3, C2, 0, s>>>(net->dg, net->g, net->gi, net->h2, B, net->P, G + OW3, G + OB3);
-    k_pool_rows<<<grid_for(rows_c, 256), 256, 0, s>>>(net->dg, net->g, net->gi, net->xs, net->h1, net->h2, W + OW3, B,
-                                                      net->P, net->xc, net->h1c, net->h2c, net->dh2c);
-    gemm<true, false, EPI_ATOMIC>(s, net->h1c, net->dh2c, G + OW2, nullptr, C1, C2, (int)rows_c, C1, C2, C2,
-                                  splits_for(rows_c, C1, C2));
-    colsum(s, net->dh2c, rows_c, C2, G + OB2);
-    gemm<false, true, 0>(s, net->dh2c, W + OW2, net->dh1c, nullptr, (int)rows_c, C1, C2, C2, C2, C1);
-    k_relu_back<<<grid_for(rows_c * C1, 256), 256, 0, s>>>(net->dh1c, net->h1c, rows_c * C1);
-    gemm<true, false, EPI_ATOMIC>(s, net->xc, net->dh1c, G + OW1, nullptr, 3, C1, (int)rows_c, 3, C1, C1,
-                                  splits_for(rows_c, 3, C1));
-    colsum(s, net->dh1c, rows_c, C1, G + OB1);
+    // max-pool and the shared layers, on the pooled rows (c, b) only
+    PoolArgs pa = {};
+    pa.dg = net->dg; pa.g = net->g; pa.gi = net->gi;
+    pa.x = scans; pa.inv = 1.f / net->in_scale;
+    pa.h1 = net->h1; pa.h2 = net->h2;
+    pa.W2 = W + OW2; pa.W3 = W + OW3;
+    pa.B = B; pa.P = net->P;
+    pa.dW1 = G + OW1; pa.db1 = G + OB1; pa.dW2 = G + OW2; pa.db2 = G + OB2; pa.dW3 = G + OW3; pa.db3 = G + OB3;
+    k_pool_back<<<std::min(net->pool_grid, (B * C3 + PR - 1) / PR), PTH, POOL_SMEM, s>>>(pa);
     PN_CUDA(cudaGetLastError());
     if (grad_out) PN_CUDA(cudaMemcpyAsync(grad_out, G, sizeof(float) * NPARAM, cudaMemcpyDefault, s));
     return MP_OK;
