@@ -357,6 +357,21 @@ __global__ void k_unpack(const float4* __restrict__ src, int64_t n, float* __res
     d[0] = a.x; d[1] = a.y; d[2] = a.z; d[3] = a.w; d[4] = b.x; d[5] = b.y; d[6] = b.z;
 }
 
+// Fresh particles: lists {self} with k = 1, identity orders, log-likelihood 0.
+__global__ void k_init_lists(int64_t n, int K, int32_t* __restrict__ ids, float* __restrict__ k,
+                             int32_t* __restrict__ sorted_ids, int32_t* __restrict__ rank, int32_t* __restrict__ visit,
+                             float* __restrict__ loglik) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= n * K) return;
+    const bool self = e % K == 0;
+    ids[e] = self ? (int32_t)(e / K) : -1;
+    k[e] = self ? 1.f : 0.f;
+    if (e < n) {
+        sorted_ids[e] = rank[e] = visit[e] = (int32_t)e;
+        loglik[e] = 0.f;
+    }
+}
+
 __global__ void k_gather_gn(const float* __restrict__ gn, int64_t stride, const int32_t* __restrict__ order, int64_t n,
                             float* __restrict__ dst) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -517,6 +532,13 @@ int mp_launch_init_uniform(mp_ctx* c, const float lo[6], const float hi[6]) {
     (void)two_pi;
     A.key = make_uint2((uint32_t)c->p.seed, (uint32_t)(c->p.seed >> 32));
     k_init_uniform<<<grid_for(c->n, 256), 256, 0, c->stream>>>(A);
+    MP_LAUNCHED(c);
+    return MP_OK;
+}
+
+int mp_launch_init_lists(mp_ctx* c) {
+    k_init_lists<<<grid_for(c->n * c->p.K, 256), 256, 0, c->stream>>>(c->n, c->p.K, c->nbr_ids[0], c->nbr_k, c->sorted_ids,
+                                                                      c->rank, c->visit, c->loglik);
     MP_LAUNCHED(c);
     return MP_OK;
 }

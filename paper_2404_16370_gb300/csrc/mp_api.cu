@@ -140,7 +140,7 @@ int upload_step(mp_ctx* c) {
         slot = c->step_ring;
         c->step_ring ^= 1;
         MP_CUDA(c, cudaEventSynchronize(c->step_ev[slot]));
-        h = c->step_host + slot;
+        h = c->host->step + slot;
     }
     fill_step_host(c, h);
     MP_CUDA(c, cudaMemcpyAsync(c->step_dev, h, sizeof(StepDev), cudaMemcpyHostToDevice, c->stream));
@@ -173,6 +173,7 @@ void free_particles(mp_ctx* c) {
     dfree(c->radix_counts); dfree(c->scan_tmp);
     dfree(c->nbr_ids[0]); dfree(c->nbr_ids[1]); dfree(c->nbr_k); dfree(c->nbr_d);
     dfree(c->gn); dfree(c->psi); dfree(c->pinv); dfree(c->phi); dfree(c->red);
+    dfree(c->io);
     c->cap = 0;
     c->n = 0;
 }
@@ -186,7 +187,13 @@ size_t scan_need(int64_t n) {
     return need + 1;
 }
 
+// Buffers for n particles; those of as many are kept (the parameters they
+// depend on are fixed when the context is made).
 int alloc_particles(mp_ctx* c, int64_t n) {
+    if (c->cap == n) {
+        c->cur = 0;
+        return MP_OK;
+    }
     free_particles(c);
     int64_t K = c->p.K;
     int64_t nb = (n + MP_SORT_TILE - 1) / MP_SORT_TILE;
@@ -231,7 +238,7 @@ void destroy(mp_ctx* c) {
     dfree(c->scalars); dfree(c->best_idx); dfree(c->best_pose); dfree(c->dev_error); dfree(c->post_bar); dfree(c->pairs);
     dfree(c->step_dev);
     mp_gicp_free(c);
-    if (c->step_host) cudaFreeHost(c->step_host);
+    if (c->host) cudaFreeHost(c->host);
     for (int k = 0; k < 2; ++k)
         if (c->step_ev[k]) cudaEventDestroy(c->step_ev[k]);
     for (int r = 0; r < MP_EV_RING; ++r)
@@ -317,6 +324,42 @@ void chol6(const double S[36], double L[6][6]) {
             L[r][k] = acc / d;
         }
     }
+}
+
+// p where a kernel on the context's device can use it as floats, else null:
+// poses go to and from such memory by one kernel, from anywhere else through
+// c->io (a call that allocated and freed a scratch took 0.2 ms longer).
+float* device_floats(mp_ctx* c, const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool here = at.type == cudaMemoryTypeDevice && at.device == c->device;
+    return here && reinterpret_cast<uintptr_t>(p) % sizeof(float) == 0 ? static_cast<float*>(const_cast<void*>(p)) : nullptr;
+}
+
+int io_floats(mp_ctx* c) { return dalloc(c, &c->io, 7 * (size_t)c->cap); }
+
+// c->n poses of seven floats at src, host or device memory, into dst; the caller waits
+int put_poses(mp_ctx* c, const void* src, float4* dst) {
+    const float* from = device_floats(c, src);
+    if (!from) {
+        const int rc = io_floats(c);
+        if (rc) return rc;
+        MP_CUDA(c, cudaMemcpyAsync(c->io, src, sizeof(float) * 7 * (size_t)c->n, cudaMemcpyDefault, c->stream));
+        from = c->io;
+    }
+    return mp_launch_pack_poses(c, from, dst);
+}
+
+// the current poses, seven floats each, into dst, host or device memory; the caller waits
+int get_poses(mp_ctx* c, void* dst) {
+    if (float* to = device_floats(c, dst)) return mp_launch_unpack_poses(c, c->poses[c->cur], to);
+    int rc = io_floats(c);
+    if (rc || (rc = mp_launch_unpack_poses(c, c->poses[c->cur], c->io))) return rc;
+    MP_CUDA(c, cudaMemcpyAsync(dst, c->io, sizeof(float) * 7 * (size_t)c->n, cudaMemcpyDefault, c->stream));
+    return MP_OK;
 }
 
 // a device scratch of `bytes` for layout conversions in getters/setters
@@ -405,7 +448,7 @@ static int ctx_setup(mp_ctx* c) {
         if ((rc = dalloc(c, &c->post_bar, 1))) break;
         if ((rc = dalloc(c, &c->step_dev, 1))) break;
         if ((rc = dalloc(c, &c->pairs, 1))) break;
-        cudaError_t e = cudaHostAlloc((void**)&c->step_host, 2 * sizeof(StepDev), cudaHostAllocDefault);
+        cudaError_t e = cudaHostAlloc((void**)&c->host, sizeof(PinnedHost), cudaHostAllocDefault);
         if (e != cudaSuccess) { rc = mp_cuda_check(c, e, "cudaHostAlloc"); break; }
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&c->step_ev[k], cudaEventDisableTiming);
         if (e != cudaSuccess) { rc = mp_cuda_check(c, e, "cudaEventCreate"); break; }
@@ -547,13 +590,7 @@ int mp_init_particles(mp_ctx* c, int64_t n, const float lo[6], const float hi[6]
     c->n = n;
     c->step = 0;
     if (poses) {
-        float* tmp = nullptr;
-        MP_CUDA(c, cudaMalloc(&tmp, sizeof(float) * 7 * (size_t)n));
-        MP_CUDA(c, cudaMemcpyAsync(tmp, poses, sizeof(float) * 7 * (size_t)n, cudaMemcpyDefault, c->stream));
-        rc = mp_launch_pack_poses(c, tmp, c->poses[0]);
-        cudaStreamSynchronize(c->stream);
-        cudaFree(tmp);
-        if (rc) return rc;
+        if ((rc = put_poses(c, poses, c->poses[0]))) return rc;
     } else {
         for (int a = 0; a < 6; ++a)
             if (!(hi[a] >= lo[a])) return mp_fail(c, MP_EINVAL, "bounds: hi < lo");
@@ -565,19 +602,9 @@ int mp_init_particles(mp_ctx* c, int64_t n, const float lo[6], const float hi[6]
         MP_CUDA(c, cudaMemsetAsync(c->logprior, 0, sizeof(double) * (size_t)n, c->stream));
     }
     // lists = {self}, k = 1
-    std::vector<int32_t> ids((size_t)(n * c->p.K), -1);
-    std::vector<float> kk((size_t)(n * c->p.K), 0.f);
-    for (int64_t i = 0; i < n; ++i) { ids[(size_t)(i * c->p.K)] = (int32_t)i; kk[(size_t)(i * c->p.K)] = 1.f; }
     c->nbr_cur = 0;
-    MP_CUDA(c, cudaMemcpyAsync(c->nbr_ids[0], ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice, c->stream));
-    MP_CUDA(c, cudaMemcpyAsync(c->nbr_k, kk.data(), sizeof(float) * kk.size(), cudaMemcpyHostToDevice, c->stream));
-    MP_CUDA(c, cudaMemsetAsync(c->nbr_d, 0, sizeof(float) * 6 * ids.size(), c->stream));
-    std::vector<int32_t> iota((size_t)n);
-    for (int64_t i = 0; i < n; ++i) iota[(size_t)i] = (int32_t)i;
-    MP_CUDA(c, cudaMemcpyAsync(c->sorted_ids, iota.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-    MP_CUDA(c, cudaMemcpyAsync(c->rank, iota.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-    MP_CUDA(c, cudaMemcpyAsync(c->visit, iota.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-    MP_CUDA(c, cudaMemsetAsync(c->loglik, 0, sizeof(float) * (size_t)n, c->stream));
+    if ((rc = mp_launch_init_lists(c))) return rc;
+    MP_CUDA(c, cudaMemsetAsync(c->nbr_d, 0, sizeof(float) * 6 * (size_t)(n * c->p.K), c->stream));
     MP_CUDA(c, cudaMemsetAsync(c->psi, 0, sizeof(float) * 8 * (size_t)n, c->stream));
     MP_CUDA(c, cudaMemsetAsync(c->phi, 0, sizeof(float) * 8 * (size_t)n, c->stream));
     MP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -679,24 +706,23 @@ int mp_step(mp_ctx* c, const float* scan, int32_t n_scan, const double odom_T[16
 int mp_get_posterior(mp_ctx* c, float* poses_out, double* prob_out, float best_pose[7], double* best_prob) {
     if (!c) return MP_EINVAL;
     if (c->n == 0) return mp_fail(c, MP_ENOTINIT, "particles not initialised");
-    int32_t err = 0;
-    MP_CUDA(c, cudaMemcpyAsync(&err, c->dev_error, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    PostHost* h = &c->host->post;
+    MP_CUDA(c, cudaMemcpyAsync(&h->err, c->dev_error, sizeof(h->err), cudaMemcpyDeviceToHost, c->stream));
     if (best_pose || best_prob) {
-        float4 bp[2];
-        double sc[4];
-        MP_CUDA(c, cudaMemcpyAsync(bp, c->best_pose, sizeof(bp), cudaMemcpyDeviceToHost, c->stream));
-        MP_CUDA(c, cudaMemcpyAsync(sc, c->scalars, sizeof(sc), cudaMemcpyDeviceToHost, c->stream));
-        MP_CUDA(c, cudaStreamSynchronize(c->stream));
-        if (best_pose) {
-            best_pose[0] = bp[0].x; best_pose[1] = bp[0].y; best_pose[2] = bp[0].z; best_pose[3] = bp[0].w;
-            best_pose[4] = bp[1].x; best_pose[5] = bp[1].y; best_pose[6] = bp[1].z;
-        }
-        if (best_prob) *best_prob = sc[3];
+        MP_CUDA(c, cudaMemcpyAsync(h->best, c->best_pose, sizeof(h->best), cudaMemcpyDeviceToHost, c->stream));
+        MP_CUDA(c, cudaMemcpyAsync(h->scalars, c->scalars, sizeof(h->scalars), cudaMemcpyDeviceToHost, c->stream));
     }
     int rc;
-    if (poses_out && (rc = mp_get_buffer(c, MP_BUF_POSES, poses_out, 7 * c->n))) return rc;
-    if (prob_out && (rc = mp_get_buffer(c, MP_BUF_POST, prob_out, c->n))) return rc;
+    if (poses_out && (rc = get_poses(c, poses_out))) return rc;
+    if (prob_out)
+        MP_CUDA(c, cudaMemcpyAsync(prob_out, c->post, sizeof(double) * (size_t)c->n, cudaMemcpyDefault, c->stream));
     MP_CUDA(c, cudaStreamSynchronize(c->stream));
+    const int32_t err = h->err;
+    if (best_pose) {
+        best_pose[0] = h->best[0].x; best_pose[1] = h->best[0].y; best_pose[2] = h->best[0].z; best_pose[3] = h->best[0].w;
+        best_pose[4] = h->best[1].x; best_pose[5] = h->best[1].y; best_pose[6] = h->best[1].z;
+    }
+    if (best_prob) *best_prob = h->scalars[3];
     if (err) {
         cudaMemsetAsync(c->dev_error, 0, sizeof(int32_t), c->stream);
         return mp_fail(c, MP_ETIMEOUT, "a bounded device-side wait gave up (error bits 0x%x)", err);
@@ -747,12 +773,16 @@ int mp_get_buffer(mp_ctx* c, int which, void* dst, int64_t count) {
     };
     switch (which) {
         case MP_BUF_POSES: {
-            DevTmp t;
-            MP_CUDA(c, cudaMalloc(&t.p, sizeof(float) * 7 * (size_t)n));
-            if ((rc = mp_launch_unpack_poses(c, c->poses[c->cur], (float*)t.p))) return rc;
-            return copy(t.p, sizeof(float) * 7 * (size_t)n);
+            if ((rc = get_poses(c, dst))) return rc;
+            MP_CUDA(c, cudaStreamSynchronize(c->stream));
+            return MP_OK;
         }
         case MP_BUF_GN: {
+            if (float* to = device_floats(c, dst)) {
+                if ((rc = mp_launch_gather_gn(c, to))) return rc;
+                MP_CUDA(c, cudaStreamSynchronize(c->stream));
+                return MP_OK;
+            }
             DevTmp t;
             MP_CUDA(c, cudaMalloc(&t.p, sizeof(float) * MP_GN * (size_t)n));
             if ((rc = mp_launch_gather_gn(c, (float*)t.p))) return rc;
@@ -832,10 +862,7 @@ int mp_set_buffer(mp_ctx* c, int which, const void* src, int64_t count) {
     };
     switch (which) {
         case MP_BUF_POSES: {
-            DevTmp t;
-            MP_CUDA(c, cudaMalloc(&t.p, sizeof(float) * 7 * (size_t)n));
-            MP_CUDA(c, cudaMemcpyAsync(t.p, src, sizeof(float) * 7 * (size_t)n, cudaMemcpyDefault, c->stream));
-            if ((rc = mp_launch_pack_poses(c, (const float*)t.p, c->poses[c->cur]))) return rc;
+            if ((rc = put_poses(c, src, c->poses[c->cur]))) return rc;
             MP_CUDA(c, cudaStreamSynchronize(c->stream));
             return MP_OK;
         }

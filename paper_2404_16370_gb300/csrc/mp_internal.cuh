@@ -38,6 +38,18 @@ struct StepDev {
     uint32_t step;
 };
 
+// mp_get_posterior's scalars, and the pinned host memory of a context.
+struct PostHost {
+    double scalars[4];
+    float4 best[2];
+    int32_t err;
+};
+
+struct PinnedHost {
+    StepDev step[2];
+    PostHost post;
+};
+
 struct mp_ctx {
     mp_params p;
     cudaStream_t stream;
@@ -118,7 +130,8 @@ struct mp_ctx {
     // host slots (an event per slot guards its reuse); batch_slot, when set,
     // replaces the ring (a captured step copies from a fixed slot)
     StepDev* step_dev;
-    StepDev* step_host;
+    PinnedHost* host;
+    float* io;               // 7 floats a particle between the stored poses and host memory, kept once used
     cudaEvent_t step_ev[2];
     int step_ring;
     StepDev* batch_slot;
@@ -567,6 +580,7 @@ int mp_launch_predict(mp_ctx* c);
 int mp_launch_solve(mp_ctx* c);
 int mp_launch_svgd(mp_ctx* c);
 int mp_launch_init_uniform(mp_ctx* c, const float lo[6], const float hi[6]);
+int mp_launch_init_lists(mp_ctx* c);
 int mp_launch_pack_poses(mp_ctx* c, const float* src7_dev, float4* dst);
 int mp_launch_unpack_poses(mp_ctx* c, const float4* src, float* dst7_dev);
 int mp_launch_gather_gn(mp_ctx* c, float* dst_dev);
