@@ -809,27 +809,27 @@ ScanArgs scan_args(mp_ctx* c, const float* raw, int n) {
 }  // namespace
 
 // The scan kernels over m scans.
-static int launch_scans(mp_ctx* c, const ScanArgs2& A, int m) {
+static int launch_scans(mp_ctx* c, const ScanArgs2& A, int m, cudaStream_t s) {
     const int n = m > 1 ? std::max(A.s[0].n, A.s[1].n) : A.s[0].n;
-    k_scan_to_float4<<<dim3(grid_for(n, 256), m), 256, 0, c->stream>>>(A);
+    k_scan_to_float4<<<dim3(grid_for(n, 256), m), 256, 0, s>>>(A);
     MP_LAUNCHED(c);
-    k_scan_normals<<<dim3(grid_for(n, NRM_PTS), m), NRM_CTA, 0, c->stream>>>(A);
+    k_scan_normals<<<dim3(grid_for(n, NRM_PTS), m), NRM_CTA, 0, s>>>(A);
     MP_LAUNCHED(c);
-    k_scan_sort<<<dim3(grid_for(n, SCAN_PTS), m), SCAN_CTA, 0, c->stream>>>(A);
+    k_scan_sort<<<dim3(grid_for(n, SCAN_PTS), m), SCAN_CTA, 0, s>>>(A);
     MP_LAUNCHED(c);
     return MP_OK;
 }
 
 // Per-step scan Gaussians (brute-force radius kNN in shared-memory tiles) and
 // the valid points, sorted and in input order.
-int mp_launch_scan_prepare(mp_ctx* c) {
+int mp_launch_scan_prepare(mp_ctx* c, cudaStream_t s) {
     int n = c->n_scan;
     if (n == 0) {
-        MP_CUDA(c, cudaMemsetAsync(c->scan_nvalid, 0, sizeof(int32_t), c->stream));
+        MP_CUDA(c, cudaMemsetAsync(c->scan_nvalid, 0, sizeof(int32_t), s));
         return MP_OK;
     }
     const ScanArgs A = scan_args(c, c->scan_raw, n);
-    return launch_scans(c, ScanArgs2{{A, A}}, 1);
+    return launch_scans(c, ScanArgs2{{A, A}}, 1, s);
 }
 
 // Point Gaussians of m <= 2 point arrays (n >= 1 points each): normals, validity, and
@@ -847,7 +847,7 @@ int mp_launch_point_gaussians(mp_ctx* c, const PointScan* in, int m) {
         a.idx = p.idx;
         a.nvalid = p.nvalid;
     }
-    return launch_scans(c, A, m);
+    return launch_scans(c, A, m, c->stream);
 }
 
 // Grouped scan stage: every instance's scan is read from the batch's device

@@ -53,6 +53,8 @@ struct PinnedHost {
 struct mp_ctx {
     mp_params p;
     cudaStream_t stream;
+    cudaStream_t side;            // the scan's kernels beside those of the particles, see SideBranch
+    cudaEvent_t fork, join;
     int device;
     char err[512];
     int64_t launches;
@@ -556,7 +558,7 @@ void mp_gicp_free(mp_ctx* c);
 void fill_step_host(mp_ctx* c, StepDev* h);
 int upload_step(mp_ctx* c);
 int mp_launch_map_prepare(mp_ctx* c, const float* xyz_dev);
-int mp_launch_scan_prepare(mp_ctx* c);
+int mp_launch_scan_prepare(mp_ctx* c, cudaStream_t s);
 struct PointScan {      // n x 3 points, and what is made of them
     const float* raw;
     int n;
