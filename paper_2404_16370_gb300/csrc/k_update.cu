@@ -357,6 +357,27 @@ __global__ void k_unpack(const float4* __restrict__ src, int64_t n, float* __res
     d[0] = a.x; d[1] = a.y; d[2] = a.z; d[3] = a.w; d[4] = b.x; d[5] = b.y; d[6] = b.z;
 }
 
+// What mp_get_posterior reads, in one launch: poses and probabilities into
+// device memory (either may be null) and the scalars into pinned host memory.
+__global__ void k_read_posterior(const float4* __restrict__ poses, const double* __restrict__ post, int64_t n,
+                                 float* __restrict__ poses7, double* __restrict__ prob,
+                                 const double* __restrict__ scalars, const float4* __restrict__ best,
+                                 const int32_t* __restrict__ err, PostHost* __restrict__ host) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i == 0) {
+        for (int k = 0; k < 4; ++k) host->scalars[k] = scalars[k];
+        for (int k = 0; k < 2; ++k) host->best[k] = best[k];
+        host->err = *err;
+    }
+    if (i >= n) return;
+    if (prob) prob[i] = post[i];
+    if (poses7) {
+        const float4 a = poses[2 * i], b = poses[2 * i + 1];
+        float* d = poses7 + 7 * i;
+        d[0] = a.x; d[1] = a.y; d[2] = a.z; d[3] = a.w; d[4] = b.x; d[5] = b.y; d[6] = b.z;
+    }
+}
+
 // Fresh particles: lists {self} with k = 1, identity orders, log-likelihood 0.
 __global__ void k_init_lists(int64_t n, int K, int32_t* __restrict__ ids, float* __restrict__ k,
                              int32_t* __restrict__ sorted_ids, int32_t* __restrict__ rank, int32_t* __restrict__ visit,
@@ -545,6 +566,14 @@ int mp_launch_init_lists(mp_ctx* c) {
 
 int mp_launch_pack_poses(mp_ctx* c, const float* src7_dev, float4* dst) {
     k_pack<<<grid_for(c->n, 256), 256, 0, c->stream>>>(src7_dev, c->n, dst);
+    MP_LAUNCHED(c);
+    return MP_OK;
+}
+
+int mp_launch_read_posterior(mp_ctx* c, float* poses7_dev, double* post_dev) {
+    const int64_t n = poses7_dev || post_dev ? c->n : 1;
+    k_read_posterior<<<grid_for(n, 256), 256, 0, c->stream>>>(c->poses[c->cur], c->post, n, poses7_dev, post_dev, c->scalars,
+                                                              c->best_pose, c->dev_error, &c->host->post);
     MP_LAUNCHED(c);
     return MP_OK;
 }

@@ -329,24 +329,25 @@ void chol6(const double S[36], double L[6][6]) {
     }
 }
 
-// p where a kernel on the context's device can use it as floats, else null:
-// poses go to and from such memory by one kernel, from anywhere else through
-// c->io (a call that allocated and freed a scratch took 0.2 ms longer).
-float* device_floats(mp_ctx* c, const void* p) {
+// p where a kernel on the context's device can use it as an array of T, else
+// null: poses go to and from such memory by one kernel, from anywhere else
+// through c->io (a call that allocated and freed a scratch took 0.2 ms longer).
+template <typename T>
+T* on_device(mp_ctx* c, const void* p) {
     cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
     const bool here = at.type == cudaMemoryTypeDevice && at.device == c->device;
-    return here && reinterpret_cast<uintptr_t>(p) % sizeof(float) == 0 ? static_cast<float*>(const_cast<void*>(p)) : nullptr;
+    return here && reinterpret_cast<uintptr_t>(p) % sizeof(T) == 0 ? static_cast<T*>(const_cast<void*>(p)) : nullptr;
 }
 
 int io_floats(mp_ctx* c) { return dalloc(c, &c->io, 7 * (size_t)c->cap); }
 
 // c->n poses of seven floats at src, host or device memory, into dst; the caller waits
 int put_poses(mp_ctx* c, const void* src, float4* dst) {
-    const float* from = device_floats(c, src);
+    const float* from = on_device<float>(c, src);
     if (!from) {
         const int rc = io_floats(c);
         if (rc) return rc;
@@ -358,7 +359,7 @@ int put_poses(mp_ctx* c, const void* src, float4* dst) {
 
 // the current poses, seven floats each, into dst, host or device memory; the caller waits
 int get_poses(mp_ctx* c, void* dst) {
-    if (float* to = device_floats(c, dst)) return mp_launch_unpack_poses(c, c->poses[c->cur], to);
+    if (float* to = on_device<float>(c, dst)) return mp_launch_unpack_poses(c, c->poses[c->cur], to);
     int rc = io_floats(c);
     if (rc || (rc = mp_launch_unpack_poses(c, c->poses[c->cur], c->io))) return rc;
     MP_CUDA(c, cudaMemcpyAsync(dst, c->io, sizeof(float) * 7 * (size_t)c->n, cudaMemcpyDefault, c->stream));
@@ -480,7 +481,7 @@ static int ctx_setup(mp_ctx* c) {
         if ((rc = dalloc(c, &c->post_bar, 1))) break;
         if ((rc = dalloc(c, &c->step_dev, 1))) break;
         if ((rc = dalloc(c, &c->pairs, 1))) break;
-        cudaError_t e = cudaHostAlloc((void**)&c->host, sizeof(PinnedHost), cudaHostAllocDefault);
+        cudaError_t e = cudaHostAlloc((void**)&c->host, sizeof(PinnedHost), cudaHostAllocMapped);
         if (e != cudaSuccess) { rc = mp_cuda_check(c, e, "cudaHostAlloc"); break; }
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&c->step_ev[k], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
@@ -751,15 +752,13 @@ int mp_step(mp_ctx* c, const float* scan, int32_t n_scan, const double odom_T[16
 int mp_get_posterior(mp_ctx* c, float* poses_out, double* prob_out, float best_pose[7], double* best_prob) {
     if (!c) return MP_EINVAL;
     if (c->n == 0) return mp_fail(c, MP_ENOTINIT, "particles not initialised");
-    PostHost* h = &c->host->post;
-    MP_CUDA(c, cudaMemcpyAsync(&h->err, c->dev_error, sizeof(h->err), cudaMemcpyDeviceToHost, c->stream));
-    if (best_pose || best_prob) {
-        MP_CUDA(c, cudaMemcpyAsync(h->best, c->best_pose, sizeof(h->best), cudaMemcpyDeviceToHost, c->stream));
-        MP_CUDA(c, cudaMemcpyAsync(h->scalars, c->scalars, sizeof(h->scalars), cudaMemcpyDeviceToHost, c->stream));
-    }
+    const PostHost* h = &c->host->post;
+    float* poses = on_device<float>(c, poses_out);
+    double* prob = on_device<double>(c, prob_out);
     int rc;
-    if (poses_out && (rc = get_poses(c, poses_out))) return rc;
-    if (prob_out)
+    if ((rc = mp_launch_read_posterior(c, poses, prob))) return rc;
+    if (poses_out && !poses && (rc = get_poses(c, poses_out))) return rc;
+    if (prob_out && !prob)
         MP_CUDA(c, cudaMemcpyAsync(prob_out, c->post, sizeof(double) * (size_t)c->n, cudaMemcpyDefault, c->stream));
     MP_CUDA(c, cudaStreamSynchronize(c->stream));
     const int32_t err = h->err;
@@ -823,7 +822,7 @@ int mp_get_buffer(mp_ctx* c, int which, void* dst, int64_t count) {
             return MP_OK;
         }
         case MP_BUF_GN: {
-            if (float* to = device_floats(c, dst)) {
+            if (float* to = on_device<float>(c, dst)) {
                 if ((rc = mp_launch_gather_gn(c, to))) return rc;
                 MP_CUDA(c, cudaStreamSynchronize(c->stream));
                 return MP_OK;

@@ -584,6 +584,7 @@ int mp_launch_svgd(mp_ctx* c);
 int mp_launch_init_uniform(mp_ctx* c, const float lo[6], const float hi[6]);
 int mp_launch_init_lists(mp_ctx* c);
 int mp_launch_pack_poses(mp_ctx* c, const float* src7_dev, float4* dst);
+int mp_launch_read_posterior(mp_ctx* c, float* poses7_dev, double* post_dev);
 int mp_launch_unpack_poses(mp_ctx* c, const float4* src, float* dst7_dev);
 int mp_launch_gather_gn(mp_ctx* c, float* dst_dev);
 // k_posterior.cu
