@@ -11,6 +11,8 @@
 #include "mp_internal.cuh"
 #include "../../include/mp_proposal.h"
 
+#include <cuda_bf16.h>
+
 #include <algorithm>
 #include <cstdio>
 
@@ -293,7 +295,8 @@ __global__ void k_maxpool(const float* __restrict__ h3, int B, int P, float* __r
 // GFLOP at batch 128) and their shared-memory reads. As nine kernels that passed
 // the rows' h1, h2, dh1 and dh2 through memory, batch 128 took 360 us; 48 now.
 struct PoolArgs {
-    const float *dg, *g, *x, *h1, *h2, *W2, *W3;
+    const float *dg, *g, *x, *W2, *W3;
+    const void *h1, *h2;  // FP32 rows, or the tensor-core form's BF16 operands (its values)
     const int* gi;
     float inv;            // scale of x
     int B, P;
@@ -303,6 +306,23 @@ constexpr int PR = 64, PTH = 256;                                  // rows of a 
 constexpr int LD_H2 = C2 + 4, LD_H1 = C1 + 4;                      // padded rows
 constexpr int POOL_SMEM = 4 * (PR * LD_H2 + PR * LD_H1 + C2 * LD_H1 + PR * 4 + 2 * PR) + 4 * PR;
 
+template <bool BF16>
+__device__ __forceinline__ float4 pool_h1(const void* h1, int64_t row, int j) {
+    if (!BF16) return *reinterpret_cast<const float4*>(static_cast<const float*>(h1) + row * C1 + j);
+    const uint8_t* b = static_cast<const uint8_t*>(h1) + (row >> 7) * MP_SW_BLOCK + sw128((uint32_t)row & 127u, (uint32_t)j);
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(b));
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xffff0000u));
+}
+template <bool BF16>
+__device__ __forceinline__ float pool_h2(const void* h2, int64_t row, int i) {
+    if (!BF16) return __ldg(static_cast<const float*>(h2) + row * C2 + i);
+    const uint8_t* b = static_cast<const uint8_t*>(h2) + ((row >> 7) * 2 + (i >> 6)) * (int64_t)MP_SW_BLOCK +
+                       sw128((uint32_t)row & 127u, (uint32_t)i & 63u);
+    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(b)) << 16);
+}
+
+template <bool BF16>
 __global__ void __launch_bounds__(PTH, 2) k_pool_back(const PoolArgs A) {
     extern __shared__ __align__(16) float pool_smem[];
     float* dh2s = pool_smem;                  // [row][i]
@@ -342,7 +362,7 @@ __global__ void __launch_bounds__(PTH, 2) k_pool_back(const PoolArgs A) {
         for (int e = 0; e < PR * C1 / 4 / PTH; ++e) {
             const int v = e * PTH + tid, r = v / (C1 / 4), j = v % (C1 / 4) * 4;
             *reinterpret_cast<float4*>(h1s + r * LD_H1 + j) =
-                *reinterpret_cast<const float4*>(A.h1 + (int64_t)ps[r] * C1 + j);
+                pool_h1<BF16>(A.h1, ps[r], j);
         }
         // h2: a thread has one i and half of the rows
         {
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(PTH, 2) k_pool_back(const PoolArgs A) {
                 const int r0 = half * (PR / 2) + q0;
                 float h[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) h[q] = __ldg(A.h2 + (int64_t)ps[r0 + q] * C2 + i2);
+                for (int q = 0; q < 8; ++q) h[q] = pool_h2<BF16>(A.h2, ps[r0 + q], i2);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int r = r0 + q;
@@ -579,7 +599,7 @@ struct mp_pn {
     cudaStream_t stream;
     float *param, *grad, *am, *av;
     int64_t t;       // Adam step
-    float *xs, *h1, *h2, *h3, *g, *h4, *o;
+    float *xs, *h1, *h2, *h3, *g, *h4, *o;   // (h1, h2: the tensor-core form's BF16 operands in that form)
     int* gi;
     float *dO, *dh4, *dg;
     int pool_grid;     // resident CTAs of k_pool_back
@@ -625,14 +645,15 @@ int pack_weights(mp_pn* net) {
 int forward(mp_pn* net, const float* scans, int B, bool train) {
     cudaStream_t s = net->stream;
     const int64_t rows = (int64_t)B * net->P;
-    k_scale_points<<<grid_for(rows * 3, 256), 256, 0, s>>>(scans, rows * 3, 1.f / net->in_scale, net->xs);
     const float* W = net->param;
     if (net->prec == MP_PREC_BF16) {
-        const int rc = mp_pn_tc_forward(net->xs, B, net->P, W + OW1, W + OB1, W + OB2, W + OB3, net->wimg, net->g,
-                                        net->gi, train ? net->h1 : nullptr, train ? net->h2 : nullptr, net->err,
-                                        MP_WAIT_BUDGET, s);
+        const int rc = mp_pn_tc_forward(scans, 1.f / net->in_scale, B, net->P, W + OW1, W + OB1, W + OB2, W + OB3,
+                                        net->wimg, net->g, net->gi, train ? reinterpret_cast<uint8_t*>(net->h1) : nullptr,
+                                        train ? reinterpret_cast<uint8_t*>(net->h2) : nullptr, net->err, MP_WAIT_BUDGET,
+                                        s);
         if (rc) return mp_fail_noctx(rc, "mp_pn: tensor-core forward launch failed");
     } else {
+        k_scale_points<<<grid_for(rows * 3, 256), 256, 0, s>>>(scans, rows * 3, 1.f / net->in_scale, net->xs);
         gemm(s, net->xs, W + OW1, net->h1, W + OB1, (int)rows, C1, 3);
         gemm(s, net->h1, W + OW2, net->h2, W + OB2, (int)rows, C2, C1);
         gemm(s, net->h2, W + OW3, net->h3, W + OB3, (int)rows, C3, C2);
@@ -686,8 +707,9 @@ int mp_pn_create(mp_pn** netp, int n_points, int max_batch, float in_scale, cons
     int dev = 0, sms = 0, per = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_pool_back, cudaFuncAttributeMaxDynamicSharedMemorySize, POOL_SMEM);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pool_back, PTH, POOL_SMEM);
+    for (auto k : {k_pool_back<false>, k_pool_back<true>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, POOL_SMEM);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pool_back<false>, PTH, POOL_SMEM);
     net->pool_grid = std::max(1, sms * per);
     if (e != cudaSuccess) {
         mp_pn_destroy(net);
@@ -770,7 +792,9 @@ int mp_pn_loss_grad(mp_pn* net, const float* scans, const float* targets, int B,
     pa.W2 = W + OW2; pa.W3 = W + OW3;
     pa.B = B; pa.P = net->P;
     pa.dW1 = G + OW1; pa.db1 = G + OB1; pa.dW2 = G + OW2; pa.db2 = G + OB2; pa.dW3 = G + OW3; pa.db3 = G + OB3;
-    k_pool_back<<<std::min(net->pool_grid, (B * C3 + PR - 1) / PR), PTH, POOL_SMEM, s>>>(pa);
+    const unsigned grid = (unsigned)std::min(net->pool_grid, (B * C3 + PR - 1) / PR);
+    if (net->prec == MP_PREC_BF16) k_pool_back<true><<<grid, PTH, POOL_SMEM, s>>>(pa);
+    else k_pool_back<false><<<grid, PTH, POOL_SMEM, s>>>(pa);
     PN_CUDA(cudaGetLastError());
     if (grad_out) PN_CUDA(cudaMemcpyAsync(grad_out, G, sizeof(float) * NPARAM, cudaMemcpyDefault, s));
     return MP_OK;

@@ -592,9 +592,16 @@ int mp_launch_posterior(mp_ctx* c);
 // k_pn_tc.cu: the proposal network's fused per-point layers on the tensor cores
 size_t mp_pn_tc_image_bytes();
 int mp_pn_tc_pack(const float* W2, const float* W3, uint8_t* image, cudaStream_t s);
-int mp_pn_tc_forward(const float* xs, int B, int P, const float* W1, const float* b1, const float* b2,
-                     const float* b3, const uint8_t* image, float* g, int* gi, float* h1_out, float* h2_out,
+int mp_pn_tc_forward(const float* x, float inv, int B, int P, const float* W1, const float* b1, const float* b2,
+                     const float* b3, const uint8_t* image, float* g, int* gi, uint8_t* h1_out, uint8_t* h2_out,
                      int32_t* err, long long budget, cudaStream_t s);
+// Its operands: blocks of 128 rows x 64 BF16 of MP_SW_BLOCK bytes in the 128-byte
+// swizzle, one block of h1 and two of h2 (by k) for every 128 points; element
+// (r, k) of a block lies at this byte.
+#define MP_SW_BLOCK 16384u
+__host__ __device__ __forceinline__ uint32_t sw128(uint32_t r, uint32_t k) {
+    return (r >> 3) * 1024u + (r & 7u) * 128u + ((((k >> 3) ^ r) & 7u) << 4) + (k & 7u) * 2u;
+}
 
 // ---------------------------------------------------------------------------
 // grouped launches (batched instances, mp_batch_*): one kernel over the blocks
