@@ -24,6 +24,9 @@
 
 namespace {
 
+// Particles of a block partial. A CTA of NT = 256 threads takes two such blocks,
+// one of NT = 128 one; the partials and their reductions are the same.
+constexpr int PP = 128;
 constexpr int PB = 256;
 
 __device__ __forceinline__ double warp_max(double v) {
@@ -42,7 +45,7 @@ struct PostArgs {
     const float* loglik;
     double* logprior;
     int64_t n;
-    int nb;               // blocks of PB particles
+    int nb;               // blocks of PP particles
     double* post;
     double* post_tmp;
     double* post_init;
@@ -65,10 +68,15 @@ struct PostArgs {
     int32_t* err;         // error bits (MP_ERR_WAIT when a grid barrier gives up)
 };
 
+// the block of PP particles of this thread
+template <int NT>
+__device__ __forceinline__ unsigned part_of(unsigned bx) { return bx * (NT / PP) + threadIdx.x / PP; }
+
 // block maxima of l = log prior + log likelihood (l kept in post)
+template <int NT>
 __device__ __forceinline__ void post_l(const PostArgs& A, unsigned bx) {
-    __shared__ double s[PB / 32];
-    int64_t i = (int64_t)bx * PB + threadIdx.x;
+    __shared__ double s[NT / 32];
+    int64_t i = (int64_t)bx * NT + threadIdx.x;
     double l = -INFINITY;
     if (i < A.n) {
         l = A.logprior[i] + (double)A.loglik[i];
@@ -77,34 +85,37 @@ __device__ __forceinline__ void post_l(const PostArgs& A, unsigned bx) {
     l = warp_max(l);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = l;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < PB / 32 ? s[threadIdx.x] : -INFINITY;
-        v = warp_max(v);
-        if (threadIdx.x == 0) A.part[bx] = v;
+    if (threadIdx.x % PP == 0 && part_of<NT>(bx) < (unsigned)A.nb) {
+        double v = s[threadIdx.x >> 5];
+#pragma unroll
+        for (int k = 1; k < PP / 32; ++k) v = fmax(v, s[(threadIdx.x >> 5) + k]);
+        A.part[part_of<NT>(bx)] = v;
     }
 }
 
 // the instance's max l over its block maxima (every CTA takes it for itself:
 // no further barrier; in every thread)
+template <int NT>
 __device__ __forceinline__ double reduce_max(const PostArgs& A) {
-    __shared__ double s[PB / 32];
+    __shared__ double s[NT / 32];
     double v = -INFINITY;
-    for (int k = threadIdx.x; k < A.nb; k += PB) v = fmax(v, __ldcg(A.part + k));
+    for (int k = threadIdx.x; k < A.nb; k += NT) v = fmax(v, __ldcg(A.part + k));
     v = warp_max(v);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     __syncthreads();
     v = s[0];
 #pragma unroll
-    for (int k = 1; k < PB / 32; ++k) v = fmax(v, s[k]);
+    for (int k = 1; k < NT / 32; ++k) v = fmax(v, s[k]);
     __syncthreads();
     return v;
 }
 
 // p = exp(max(l - max l, floor)) into post_init and post_tmp (the sweeps'
 // input); block sums
+template <int NT>
 __device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx, double lmax) {
-    __shared__ double s[PB / 32];
-    int64_t i = (int64_t)bx * PB + threadIdx.x;
+    __shared__ double s[NT / 32];
+    int64_t i = (int64_t)bx * NT + threadIdx.x;
     double v = 0.0;
     if (i < A.n) {
         v = exp(fmax(A.post[i] - lmax, A.lfloor));
@@ -114,28 +125,31 @@ __device__ __forceinline__ void post_exp(const PostArgs& A, unsigned bx, double 
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double w = threadIdx.x < PB / 32 ? s[threadIdx.x] : 0.0;
-        w = warp_sum(w);
-        if (threadIdx.x == 0) {
-            A.part_sum[bx] = w;
-            if (bx == 0) A.scalars[0] = lmax;
-        }
+    if (threadIdx.x % PP == 0 && part_of<NT>(bx) < (unsigned)A.nb) {
+        double w = 0.0;
+#pragma unroll
+        for (int k = 0; k < PP / 32; ++k) w += s[(threadIdx.x >> 5) + k];
+        A.part_sum[part_of<NT>(bx)] = w;
+        if (bx == 0 && threadIdx.x == 0) A.scalars[0] = lmax;
     }
 }
 
-// the instance's sum of exp(l - max l)
+// the instance's sum of exp(l - max l), by the first PP threads
+template <int NT>
 __device__ __forceinline__ void reduce_sum(const PostArgs& A) {
-    __shared__ double s[PB / 32];
-    double v = 0.0;
-    for (int k = threadIdx.x; k < A.nb; k += PB) v += __ldcg(A.part_sum + k);
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < PB / 32 ? s[threadIdx.x] : 0.0;
+    __shared__ double s[PP / 32];
+    if (threadIdx.x < PP) {
+        double v = 0.0;
+        for (int k = threadIdx.x; k < A.nb; k += PP) v += __ldcg(A.part_sum + k);
         v = warp_sum(v);
-        if (threadIdx.x == 0) A.scalars[1] = v;
+        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < PP / 32; ++k) v += s[k];
+        A.scalars[1] = v;
     }
 }
 
@@ -225,9 +239,9 @@ struct PostList {
     double w[KT];
     double invden;
 };
-template <int KT>
+template <int KT, int NT>
 __device__ __forceinline__ void post_list(const PostArgs& A, unsigned bx, PostList<KT>& L) {
-    const int64_t i = (int64_t)bx * PB + threadIdx.x;
+    const int64_t i = (int64_t)bx * NT + threadIdx.x;
     double den = 0.0;
 #pragma unroll
     for (int l = 0; l < KT; ++l) {
@@ -245,11 +259,11 @@ __device__ __forceinline__ void post_list(const PostArgs& A, unsigned bx, PostLi
         L.w[l] *= L.invden;
     }
 }
-template <int KT>
+template <int KT, int NT>
 __device__ __forceinline__ void post_list_sweep(const PostArgs& A, unsigned bx, int it, const PostList<KT>& L) {
     const double* pin = (it & 1) ? A.post : A.post_tmp;
     double* pout = (it & 1) ? A.post_tmp : A.post;
-    const int64_t i = (int64_t)bx * PB + threadIdx.x;
+    const int64_t i = (int64_t)bx * NT + threadIdx.x;
     if (i >= A.n) return;
     double p[KT];
 #pragma unroll
@@ -265,11 +279,12 @@ __device__ __forceinline__ void post_list_sweep(const PostArgs& A, unsigned bx, 
 __device__ __forceinline__ const double* post_smoothed(const PostArgs& A) { return (A.iters & 1) ? A.post : A.post_tmp; }
 
 // block partials of the smoothed posterior: sum, max and its index
+template <int NT>
 __device__ __forceinline__ void final_part(const PostArgs& A, unsigned bx) {
-    __shared__ double ss[PB / 32], sm[PB / 32];
-    __shared__ int64_t si[PB / 32];
+    __shared__ double ss[NT / 32], sm[NT / 32];
+    __shared__ int64_t si[NT / 32];
     const double* p = post_smoothed(A);
-    int64_t i = (int64_t)bx * PB + threadIdx.x;
+    int64_t i = (int64_t)bx * NT + threadIdx.x;
     double v = i < A.n ? p[i] : 0.0;
     double m = i < A.n ? v : -INFINITY;
     int64_t mi = i < A.n ? i : INT64_MAX;
@@ -286,16 +301,17 @@ __device__ __forceinline__ void final_part(const PostArgs& A, unsigned bx) {
         si[threadIdx.x >> 5] = mi;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x % PP == 0 && part_of<NT>(bx) < (unsigned)A.nb) {
         double S = 0.0, M = -INFINITY;
         int64_t I = INT64_MAX;
-        for (int k = 0; k < PB / 32; ++k) {
-            S += ss[k];
-            argmax_merge(M, I, sm[k], si[k]);
+#pragma unroll
+        for (int k = 0; k < PP / 32; ++k) {
+            S += ss[(threadIdx.x >> 5) + k];
+            argmax_merge(M, I, sm[(threadIdx.x >> 5) + k], si[(threadIdx.x >> 5) + k]);
         }
-        A.part[bx] = S;
-        A.part2[bx] = M;
-        A.part_idx[bx] = I;
+        A.part[part_of<NT>(bx)] = S;
+        A.part2[part_of<NT>(bx)] = M;
+        A.part_idx[part_of<NT>(bx)] = I;
     }
 }
 
@@ -306,29 +322,32 @@ struct PostFinal {
     int64_t idx;
 };
 __device__ __forceinline__ PostFinal final_reduce(const PostArgs& A) {
-    __shared__ double ss[PB / 32], sm[PB / 32];
-    __shared__ int64_t si[PB / 32];
-    double S = 0.0, M = -INFINITY;
-    int64_t I = INT64_MAX;
-    for (int k = threadIdx.x; k < A.nb; k += PB) {
-        S += __ldcg(A.part + k);
-        argmax_merge(M, I, __ldcg(A.part2 + k), __ldcg(reinterpret_cast<const long long*>(A.part_idx) + k));
-    }
-    S = warp_sum(S);
+    __shared__ double ss[PP / 32], sm[PP / 32];
+    __shared__ int64_t si[PP / 32];
+    if (threadIdx.x < PP) {
+        double S = 0.0, M = -INFINITY;
+        int64_t I = INT64_MAX;
+        for (int k = threadIdx.x; k < A.nb; k += PP) {
+            S += __ldcg(A.part + k);
+            argmax_merge(M, I, __ldcg(A.part2 + k), __ldcg(reinterpret_cast<const long long*>(A.part_idx) + k));
+        }
+        S = warp_sum(S);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        double m2 = __shfl_xor_sync(0xffffffffu, M, o);
-        int64_t i2 = __shfl_xor_sync(0xffffffffu, I, o);
-        argmax_merge(M, I, m2, i2);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        ss[threadIdx.x >> 5] = S;
-        sm[threadIdx.x >> 5] = M;
-        si[threadIdx.x >> 5] = I;
+        for (int o = 16; o > 0; o >>= 1) {
+            double m2 = __shfl_xor_sync(0xffffffffu, M, o);
+            int64_t i2 = __shfl_xor_sync(0xffffffffu, I, o);
+            argmax_merge(M, I, m2, i2);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            ss[threadIdx.x >> 5] = S;
+            sm[threadIdx.x >> 5] = M;
+            si[threadIdx.x >> 5] = I;
+        }
     }
     __syncthreads();
     PostFinal f = {0.0, -INFINITY, INT64_MAX};
-    for (int k = 0; k < PB / 32; ++k) {
+#pragma unroll
+    for (int k = 0; k < PP / 32; ++k) {
         f.sum += ss[k];
         argmax_merge(f.best, f.idx, sm[k], si[k]);
     }
@@ -338,8 +357,9 @@ __device__ __forceinline__ PostFinal final_reduce(const PostArgs& A) {
 
 // normalise (post_tmp keeps the smoothed values), store the log prior, copy
 // the best pose
+template <int NT>
 __device__ __forceinline__ void normalise(const PostArgs& A, unsigned bx, const PostFinal& f) {
-    int64_t i = (int64_t)bx * PB + threadIdx.x;
+    int64_t i = (int64_t)bx * NT + threadIdx.x;
     if (bx == 0 && threadIdx.x == 0) {
         A.scalars[2] = f.sum;
         A.scalars[3] = f.best / f.sum;
@@ -387,11 +407,14 @@ __device__ __forceinline__ const PostArgs& phase_item(const PostPhase& P, int w,
 // KT = 0: any number of particles, 4 CTAs of 256 threads per SM (64 registers,
 // no spill; fewer registers and more CTAs spill the sub-steps' FP64 values and
 // measured slower). KT = 16, 32: at most one particle block per CTA and lists of
-// at most KT entries, which stay in registers
-// (256 x 16: 57 -> 44 us, 4096 x 16: 91 -> 71; what is left is the sub-steps'
-// latency, an L2 round trip and a barrier per sweep).
-template <int KT>
-__global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_phase(const __grid_constant__ PostPhase P) {
+// at most KT entries, which stay in registers (256 x 16: 57 -> 44 us, 4096 x 16:
+// 91 -> 71); NT = 128: while there is an SM for each (an FP64 instruction holds a
+// quarter of the SM for 64 cycles, so two warps there take turns; 4096 x 16:
+// 71 -> 60). What is left is the sub-steps' latency, an L2 round trip and a barrier
+// per sweep.
+template <int KT, int NT>
+__global__ void __launch_bounds__(NT, KT == 0 ? 4 : KT == 16 ? 512 / NT : 256 / NT) k_post_phase(const __grid_constant__ PostPhase P) {
+    static_assert(KT != 0 || NT == PB, "post_weights and post_sweep take blocks of PB particles");
     // the test knob: the first barrier waits for one CTA more than the grid
     unsigned expect = gridDim.x + (P.starve ? 1u : 0u), target = 0;
     auto sync = [&]() {
@@ -406,7 +429,7 @@ __global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_pha
     int inst, cur = -1;
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
         const PostArgs& A = phase_item(P, w, bx, inst);
-        post_l(A, bx);
+        post_l<NT>(A, bx);
         __syncthreads();
     }
     if (!sync()) return;
@@ -415,17 +438,17 @@ __global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_pha
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
         const PostArgs& A = phase_item(P, w, bx, inst);
         if (inst != cur) {
-            lmax = reduce_max(A);
+            lmax = reduce_max<NT>(A);
             cur = inst;
         }
-        post_exp(A, bx, lmax);
+        post_exp<NT>(A, bx, lmax);
         if constexpr (KT == 0) post_weights(A, bx);
-        else post_list<KT>(A, bx, list);
+        else post_list<KT, NT>(A, bx, list);
         __syncthreads();
     }
     if (!sync()) return;
     for (int k = blockIdx.x; k < P.n_inst; k += gridDim.x) {
-        reduce_sum(phase_args(P, k));
+        reduce_sum<NT>(phase_args(P, k));
         __syncthreads();
     }
     for (int it = 0; it < P.max_iters; ++it) {
@@ -434,7 +457,7 @@ __global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_pha
             const PostArgs& A = phase_item(P, w, bx, inst);
             if (it >= A.iters) continue;
             if constexpr (KT != 0) {
-                post_list_sweep<KT>(A, bx, it, list);
+                post_list_sweep<KT, NT>(A, bx, it, list);
             } else {
                 if (A.K == 32) post_sweep<32>(A, bx, it);
                 else if (A.K == 16) post_sweep<16>(A, bx, it);
@@ -447,7 +470,7 @@ __global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_pha
     __syncthreads();
     for (int w = blockIdx.x; w < P.n_blocks; w += gridDim.x) {
         const PostArgs& A = phase_item(P, w, bx, inst);
-        final_part(A, bx);
+        final_part<NT>(A, bx);
         __syncthreads();
     }
     if (!sync()) return;
@@ -459,7 +482,7 @@ __global__ void __launch_bounds__(PB, KT == 0 ? 4 : KT == 16 ? 2 : 1) k_post_pha
             f = final_reduce(A);
             cur = inst;
         }
-        normalise(A, bx, f);
+        normalise<NT>(A, bx, f);
     }
 }
 
@@ -468,7 +491,7 @@ PostArgs post_args(mp_ctx* c, int cur) {
     A.loglik = c->loglik;
     A.logprior = c->logprior;
     A.n = c->n;
-    A.nb = (int)((c->n + PB - 1) / PB);
+    A.nb = (int)((c->n + PP - 1) / PP);
     A.post = c->post;
     A.post_tmp = c->post_tmp;
     A.post_init = c->post_init;
@@ -492,34 +515,48 @@ PostArgs post_args(mp_ctx* c, int cur) {
     return A;
 }
 
-// Resident CTAs of k_post_phase<KT> on the current device: the grid of a
-// cooperative launch may not exceed it.
-template <int KT>
-unsigned post_capacity() {
-    static int cap[64] = {};
+// Resident CTAs of k_post_phase<KT, NT> on the current device (the grid of a
+// cooperative launch may not exceed them), and its SMs.
+struct PostCapacity {
+    int ctas, sms;
+};
+template <int KT, int NT>
+PostCapacity post_capacity() {
+    static PostCapacity cap[64] = {};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (!cap[dev]) {
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return {0, 0};
+    if (!cap[dev].ctas) {
         int sms = 0, per = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_post_phase<KT>, PB, 0) != cudaSuccess)
-            return 0;
-        cap[dev] = sms * per;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_post_phase<KT, NT>, NT, 0) != cudaSuccess)
+            return {0, 0};
+        cap[dev] = {sms * per, sms};
     }
-    return (unsigned)cap[dev];
+    return cap[dev];
 }
 
-// The form of a launch over n_blocks particle blocks with lists of at most K
-// entries, and its grid (0: none): registers hold the lists when every block
-// has a CTA of its own (about 38k particles at K <= 32, 77k at K <= 16).
+// The form of a launch over n_blocks blocks of PB particles with lists of at most
+// K entries, its CTAs' threads and its grid (0: none): registers hold the lists
+// when every block has a CTA of its own (about 38k particles at K <= 32, 77k at
+// K <= 16).
 struct PostForm {
     const void* func;
+    int threads;
     unsigned grid;
 };
 PostForm post_form(unsigned n_blocks, int K) {
-    if (K <= 16 && n_blocks <= post_capacity<16>()) return {(const void*)k_post_phase<16>, n_blocks};
-    if (K > 16 && n_blocks <= post_capacity<32>()) return {(const void*)k_post_phase<32>, n_blocks};
-    return {(const void*)k_post_phase<0>, std::min(n_blocks, post_capacity<0>())};
+    if (K <= 16 && n_blocks <= (unsigned)post_capacity<16, PB>().ctas) return {(const void*)k_post_phase<16, PB>, PB, n_blocks};
+    if (K > 16 && n_blocks <= (unsigned)post_capacity<32, PB>().ctas) return {(const void*)k_post_phase<32, PB>, PB, n_blocks};
+    return {(const void*)k_post_phase<0, PB>, PB, std::min(n_blocks, (unsigned)post_capacity<0, PB>().ctas)};
+}
+// One instance of n particles: blocks of PP, lists in registers, while each has an
+// SM to itself (19456 particles) and there is more than one of PB (one CTA needs no
+// grid barrier).
+template <int KT>
+PostForm post_half_form(int64_t n) {
+    const PostCapacity c = post_capacity<KT, PP>();
+    if (n <= PB || n > (int64_t)PP * c.sms || c.ctas < c.sms) return {nullptr, 0, 0};
+    return {(const void*)k_post_phase<KT, PP>, PP, grid_for(n, PP)};
 }
 
 long long post_budget(const mp_ctx* c) { return c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET; }
@@ -529,16 +566,17 @@ long long post_budget(const mp_ctx* c) { return c->wait_budget > 0 ? c->wait_bud
 int mp_launch_posterior(mp_ctx* c) {
     PostPhase P = {};
     P.one = post_args(c, c->nbr_cur);
-    P.n_blocks = P.one.nb;
     P.n_inst = 1;
     P.max_iters = P.one.iters;
     P.starve = c->starve_bar;
     P.bar = c->post_bar;
     P.budget = post_budget(c);
-    const PostForm form = post_form((unsigned)P.n_blocks, P.one.K);
+    PostForm form = P.one.K <= 16 ? post_half_form<16>(c->n) : post_half_form<32>(c->n);
+    if (!form.grid) form = post_form(grid_for(c->n, PB), P.one.K);
     if (!form.grid) return mp_fail(c, MP_ECUDA, "posterior: no resident CTAs for the cooperative launch");
+    P.n_blocks = (int)grid_for(c->n, form.threads);
     MP_CUDA(c, cudaMemsetAsync(c->post_bar, 0, sizeof(GridBar), c->stream));
-    MP_CUDA(c, launch_coop(form.func, form.grid, PB, &P, c->stream));
+    MP_CUDA(c, launch_coop(form.func, form.grid, form.threads, &P, c->stream));
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -552,7 +590,7 @@ int mp_plan_posterior(mp_group* G, int p, std::vector<GOp>& plan) {
     for (int i = 0; i < G->size(); ++i) {
         mp_ctx* c = G->ctx[i];
         tab.push_back(post_args(c, c->nbr_cur ^ p ^ 1));   // the list the merge of this step wrote
-        bpb.push_back(tab.back().nb);
+        bpb.push_back(grid_for(c->n, PB));
         max_iters = std::max(max_iters, tab.back().iters);
         max_K = std::max(max_K, tab.back().K);
     }

@@ -212,7 +212,7 @@ int alloc_particles(mp_ctx* c, int64_t n) {
     A_(c->nbr_ids[0], n * K); A_(c->nbr_ids[1], n * K); A_(c->nbr_k, n * K); A_(c->nbr_d, n * K * 6);
     A_(c->gn, (int64_t)MP_GN * n); A_(c->psi, 8 * n); A_(c->phi, 8 * n);
     if (c->p.svgd_precond) A_(c->pinv, 24 * n);
-    A_(c->red, 4 * (n / 256 + 2));
+    A_(c->red, 4 * (n / 128 + 2));
 #undef A_
     c->cap = n;
     c->cur = 0;
