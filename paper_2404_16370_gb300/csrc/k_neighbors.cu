@@ -462,8 +462,9 @@ __global__ void __launch_bounds__(256) k_visit_keys(const VisitKeyArgs A) { Visi
 // radix pass of the general path is three dependent launches, or three grid
 // barriers of a batch's persistent phase; here it is a few block barriers. The
 // order is the same: both sorts are stable. Measured (sort stage): 256 particles
-// 67 -> 10 us, 4096 91 -> 29, 16000 98 -> 94; 16384 fill an SM's shared memory
-// (210 KB), and the general path catches up there.
+// 67 -> 10 us, 4096 91 -> 30, 16000 98 -> 94; 16384 fill an SM's shared memory
+// (210 KB). A batch runs one such CTA per instance; a single instance has more
+// CTAs to itself from MS_MIN particles on (k_mid_sort).
 constexpr int SS_THREADS = 1024, SS_WARPS = SS_THREADS / 32, SS_MAX = 16384, SS_ROWS = SS_MAX / SS_THREADS;
 
 struct SmallSortSmem {
@@ -575,6 +576,140 @@ struct SmallSortOp {
 };
 
 __global__ void __launch_bounds__(SS_THREADS) k_small_sort(const SmallSortArgs A) { SmallSortOp::run(A, 0, 0); }
+
+// ---------------------------------------------------------------------------
+// the whole sort of a middling instance in one cooperative launch
+// ---------------------------------------------------------------------------
+// The general path's fourteen short launches wait for one another. Here a CTA per
+// tile of 1024 or 4096 particles, all resident, keeps its keys and ids in registers through a
+// pass: ranks within the tile, the tile's digit counts to memory, a grid barrier,
+// the offsets (every CTA sums the counts of all tiles itself), the scatter, a grid
+// barrier. The passes are stable, so the order is the general path's. Bound by the
+// chain of two barriers and three L2 round trips a pass, and by the sums over the
+// tiles' counts. Four elements a thread while that makes one CTA per SM (155648
+// particles), else sixteen and two CTAs (1245184). Measured (sort stage): against
+// one CTA 3072 particles 26 and 29 us, 4096 32 and 30, 16000 94 and 33; against the
+// launches 50021 138 and 41, 262144 172 and 74, 2^20 234 and 151.
+constexpr int MS_THREADS = 256, MS_MIN = 3584;
+static_assert(4 * MS_THREADS >= MP_COUNT_TILE, "room for the counts");
+
+struct MidSortArgs {
+    SortArgs s;           // counts: MP_RADIX a tile, tile-major
+    VisitKeyArgs v;
+    int32_t* visit;
+    GridBar* bar;
+    int32_t* err;
+    long long budget;
+};
+
+template <int MS_ITEMS>
+__global__ void __launch_bounds__(MS_THREADS) k_mid_sort(const __grid_constant__ MidSortArgs A) {
+    __shared__ uint32_t wcnt[MS_THREADS / 32][MP_RADIX];   // a warp's elements per digit, then their offset
+    __shared__ uint32_t base[MP_RADIX], wtot[MP_RADIX / 32];
+    static_assert(MS_THREADS == MP_RADIX, "a thread per digit");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = (int)A.s.n;
+    const unsigned lt = (1u << lane) - 1u;
+    const int e0 = (int)blockIdx.x * (MS_THREADS * MS_ITEMS) + w * (32 * MS_ITEMS) + lane;   // item it: e0 + 32 it
+    uint32_t key[MS_ITEMS];
+    int32_t id[MS_ITEMS];
+    unsigned target = 0;
+    auto sync = [&] {
+        const bool ok = grid_sync(A.bar, target, gridDim.x, A.budget);
+        if (!ok && threadIdx.x == 0) atomicOr(A.err, MP_ERR_WAIT);
+        return ok;
+    };
+    // a pass over the digit at shift; the ids go to iout, and the keys to kout (null: not needed)
+    auto pass = [&](int shift, uint32_t* kout, int32_t* iout) {
+        uint32_t loc[MS_ITEMS];
+        for (int d = threadIdx.x; d < MS_THREADS / 32 * MP_RADIX; d += MS_THREADS) (&wcnt[0][0])[d] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < MS_ITEMS; ++it) {
+            const bool ok = e0 + 32 * it < n;
+            const uint32_t dg = ok ? (key[it] >> shift) & (MP_RADIX - 1) : MP_RADIX;
+            const unsigned peers = __match_any_sync(0xffffffffu, dg);
+            const uint32_t before = ok ? wcnt[w][dg] : 0u;
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) wcnt[w][dg] = before + __popc(peers);
+            __syncwarp();
+            loc[it] = before + __popc(peers & lt);
+        }
+        __syncthreads();
+        uint32_t run = 0;
+#pragma unroll
+        for (int k = 0; k < MS_THREADS / 32; ++k) {
+            const uint32_t t = wcnt[k][threadIdx.x];
+            wcnt[k][threadIdx.x] = run;
+            run += t;
+        }
+        A.s.counts[blockIdx.x * MP_RADIX + threadIdx.x] = run;
+        if (!sync()) return false;
+        // this digit's elements in the tiles before, and in all
+        uint32_t before = 0, all = 0;
+#pragma unroll 16
+        for (int k = 0; k < (int)gridDim.x; ++k) {
+            const uint32_t t = __ldcg(A.s.counts + k * MP_RADIX + threadIdx.x);
+            before += k < (int)blockIdx.x ? t : 0u;
+            all += t;
+        }
+        uint32_t inc = all;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wtot[w] = inc;
+        __syncthreads();
+        uint32_t b = inc - all + before;
+        for (int k = 0; k < w; ++k) b += wtot[k];
+        base[threadIdx.x] = b;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < MS_ITEMS; ++it) {
+            if (e0 + 32 * it >= n) continue;
+            const uint32_t dg = (key[it] >> shift) & (MP_RADIX - 1), pos = base[dg] + wcnt[w][dg] + loc[it];
+            if (!MP_DCHECK(pos < (uint32_t)n, "mid sort position", pos)) continue;
+            if (kout) kout[pos] = key[it];
+            iout[pos] = id[it];
+        }
+        return true;
+    };
+    auto load = [&](int src) {
+#pragma unroll
+        for (int it = 0; it < MS_ITEMS; ++it) {
+            const int e = min(e0 + 32 * it, n - 1);
+            key[it] = __ldcg(A.s.keys[src] + e);
+            id[it] = __ldcg(A.s.ids[src] + e);
+        }
+    };
+#pragma unroll
+    for (int it = 0; it < MS_ITEMS; ++it) {
+        id[it] = min(e0 + 32 * it, n - 1);
+        key[it] = A.s.buckets[id[it]];
+    }
+    int src = 0;
+    for (int pss = 0; pss < A.s.passes; ++pss) {
+        src = pss & 1;
+        if (!pass(pss * MP_RADIX_BITS, A.s.keys[src], A.s.ids[src]) || !sync()) return;
+        load(src);
+    }
+    // sorted ids, ranks, [lo, hi) of every present bucket; then the visiting keys
+#pragma unroll
+    for (int it = 0; it < MS_ITEMS; ++it) {
+        const int p = e0 + 32 * it;
+        if (p >= n) continue;
+        const uint32_t b = key[it];
+        const int32_t i = id[it];
+        A.s.sorted_ids[p] = i;
+        A.s.rank[i] = p;
+        if (p == 0 || __ldcg(A.s.keys[src] + p - 1) != b) A.s.blo[b] = p;
+        if (p == n - 1 || __ldcg(A.s.keys[src] + p + 1) != b) A.s.bhi[b] = p + 1;
+        key[it] = visit_key(A.v, A.v.poses[2 * (int64_t)i + 1]);
+    }
+    if (!pass(0, A.s.keys[0], A.s.ids[0]) || !sync()) return;
+    load(0);
+    pass(MP_RADIX_BITS, nullptr, A.visit);
+}
 
 // ---------------------------------------------------------------------------
 // neighbour merge: one warp per particle, 64 candidate slots (2 per lane)
@@ -949,6 +1084,30 @@ cudaError_t small_sort_prepare(const void* func) {
     return cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSortSmem));
 }
 
+// Tiles that k_mid_sort<ITEMS> may have on the current device: `per_sm` CTAs an SM
+// at most, all resident
+template <int ITEMS>
+unsigned mid_sort_tiles(int per_sm) {
+    static int cap[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (!cap[dev]) {
+        int sms = 0, per = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_mid_sort<ITEMS>, MS_THREADS, 0) != cudaSuccess)
+            return 0;
+        cap[dev] = sms * std::min(per, per_sm);
+    }
+    return (unsigned)cap[dev];
+}
+
+// The tiles of n particles if they go to k_mid_sort<ITEMS>, else 0
+template <int ITEMS>
+unsigned mid_sort_grid(int64_t n, int per_sm) {
+    const unsigned tiles = grid_for(n, MS_THREADS * ITEMS);
+    return n > MS_MIN && tiles <= mid_sort_tiles<ITEMS>(per_sm) ? tiles : 0;
+}
+
 MergeArgs merge_args(mp_ctx* c, int cur) {
     MergeArgs A;
     A.poses = c->poses[c->cur];
@@ -978,6 +1137,16 @@ int mp_launch_lsh_keys(mp_ctx* c) {
 }
 
 int mp_launch_sort(mp_ctx* c) {
+    const unsigned t4 = mid_sort_grid<4>(c->n, 1), t16 = t4 ? 0 : mid_sort_grid<16>(c->n, 2);
+    if (t4 || t16) {
+        const SmallSortArgs S = small_sort_args(c);
+        MidSortArgs M = {S.s, S.v, S.visit, c->post_bar, c->dev_error, c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET};
+        MP_CUDA(c, cudaMemsetAsync(c->post_bar, 0, sizeof(GridBar), c->stream));
+        MP_CUDA(c, launch_coop(t4 ? (const void*)k_mid_sort<4> : (const void*)k_mid_sort<16>, t4 ? t4 : t16, MS_THREADS,
+                               &M, c->stream));
+        MP_LAUNCHED(c);
+        return MP_OK;
+    }
     if (c->n <= SS_MAX) {
         MP_CUDA(c, small_sort_prepare((const void*)k_small_sort));
         k_small_sort<<<1, SS_THREADS, sizeof(SmallSortSmem), c->stream>>>(small_sort_args(c));

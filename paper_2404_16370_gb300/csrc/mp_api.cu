@@ -206,7 +206,7 @@ int alloc_particles(mp_ctx* c, int64_t n) {
     A_(c->lk_ticket, n / 256 + 3);
     A_(c->seg, 2 * ((int64_t)1 << c->p.n_buckets_log2));
     A_(c->sort_keys[0], n); A_(c->sort_keys[1], n); A_(c->sort_ids[0], n); A_(c->sort_ids[1], n);
-    A_(c->radix_counts, MP_RADIX * nb);
+    A_(c->radix_counts, MP_RADIX * ((n + MP_COUNT_TILE - 1) / MP_COUNT_TILE));
     c->scan_tmp_cap = scan_need(MP_RADIX * nb) + 64;
     A_(c->scan_tmp, c->scan_tmp_cap);
     A_(c->nbr_ids[0], n * K); A_(c->nbr_ids[1], n * K); A_(c->nbr_k, n * K); A_(c->nbr_d, n * K * 6);

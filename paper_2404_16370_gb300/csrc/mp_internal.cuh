@@ -25,6 +25,7 @@
 #define MP_RADIX_BITS 8
 #define MP_RADIX 256
 #define MP_SORT_TILE 2048   // elements per radix-sort block (256 threads x 8)
+#define MP_COUNT_TILE 1024  // fewest elements of a block with digit counts of its own
 #define MP_SCAN_CHUNK 256   // scan points per staged chunk of the likelihood
 
 // Per-step values the kernels read from device memory rather than from

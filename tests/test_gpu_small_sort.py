@@ -1,6 +1,7 @@
-"""The one-CTA sort of instances of at most 16384 particles against the general
-one's definition: the stable bucket order, ranks and segments, and the visiting
-order, at the edges of its rows of 1024 and with one, two and four radix passes."""
+"""The sorts of an instance (one CTA, one cooperative launch of a CTA per 1024
+particles, radix passes as launches) against their definition: the stable bucket
+order, ranks and segments, and the visiting order, at the edges of their ranges
+and tiles and with one, two and four radix passes."""
 import numpy as np
 import pytest
 
@@ -10,7 +11,7 @@ from paper_2404_16370_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 1023, 1024, 1025, 4096, 15360, 16383, 16384, 16385])
+@pytest.mark.parametrize("n", [1, 2, 31, 1023, 1024, 1025, 3584, 3585, 5120, 16385, 100001, 155648, 155649, 400001, 1245185])
 @pytest.mark.parametrize("bits", [1, 8, 13, 26])
 def test_small_sort(n, bits):
     from paper_2404_16370_gb300 import mp
