@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(256) k_gemm(const float* __restrict__ A, const
 // batch: few rows, so what counts is latency and CTAs. A CTA of 128 threads takes
 // 16 x 32 outputs (4 a thread) and stages 128 of K at a time, whole slices in
 // flight at once. A 64 x 64 tile with 16 of K a step left 7 CTAs waiting for 16
-// loads in a row: 46 us for 4 x 416 x 256, 7 now; the six products and
-// four column sums and gates of a training step at batch 128 320 us, 44 now.
+// loads in a row: 46 us for 4 x 416 x 256, 7 now, of which 3 pass under the kernel before (head); the six products and
+// four column sums and gates of a training step at batch 128 320 us, 36 now.
 // N and the extents along which op(A) and op(B) are contiguous are multiples of
 // 4, the matrices 16-byte aligned. Each output is one chain of fmaf over k.
 enum : int { HEAD_BIAS = 1, HEAD_RELU = 2, HEAD_GATE = 4, HEAD_COLSUM = 8 };
@@ -159,20 +159,43 @@ constexpr int HM = 16, HN = 32, HK = 128;
 
 // aux: the bias [N] (HEAD_BIAS), or a matrix like C whose entries <= 0 zero the
 // output's (HEAD_GATE). colsum: column sums of op(B) (HEAD_COLSUM).
-template <bool TA, bool TB, int EPI>
-__global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const float* __restrict__ B,
-                                              float* __restrict__ C, const float* __restrict__ aux,
-                                              float* __restrict__ colsum, int M, int N, int K, int lda, int ldb,
-                                              int ldc) {
-    __shared__ __align__(16) float As[HM][HK + 4];
-    __shared__ __align__(16) float Bs[HK][HN + 4];
-    __shared__ float cs[4][HN];
+struct HeadArgs {
+    const float *A, *B;
+    float* C;
+    const float* aux;
+    float* colsum;
+    int M, N, K, lda, ldb, ldc;
+};
+struct HeadSmem {
+    __align__(16) float As[HM][HK + 4];
+    __align__(16) float Bs[HK][HN + 4];
+    float cs[4][HN];
+};
+
+// A dependent launch's wait for the kernels before it, and the word to one that
+// it may start. Without the launch attribute both do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// PDL: op(B) is a weight matrix, which the kernels just before do not write: its
+// first slice is asked for before the wait for them.
+template <bool TA, bool TB, int EPI, bool PDL = false>
+__device__ __forceinline__ void head_tile(const HeadArgs& H, HeadSmem& S, int bx, int by) {
+    const float* __restrict__ A = H.A;
+    const float* __restrict__ B = H.B;
+    const float* __restrict__ aux = H.aux;
+    float* __restrict__ C = H.C;
+    float* __restrict__ colsum = H.colsum;
+    const int M = H.M, N = H.N, K = H.K, lda = H.lda, ldb = H.ldb, ldc = H.ldc;
+    auto& As = S.As;
+    auto& Bs = S.Bs;
+    auto& cs = S.cs;
     const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
-    const int m0 = blockIdx.y * HM, n0 = blockIdx.x * HN;
+    const int m0 = by * HM, n0 = bx * HN;
     float acc[4] = {0.f, 0.f, 0.f, 0.f}, col = 0.f;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 ra[HM * HK / 512], rb[HN * HK / 512];
-    auto load = [&](int k0) {
+    auto load_a = [&](int k0) {
 #pragma unroll
         for (int e = 0; e < HM * HK / 512; ++e) {
             const int v = e * 128 + tid;
@@ -184,6 +207,8 @@ __global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const
                 ra[e] = k < K && m < M ? *reinterpret_cast<const float4*>(A + (int64_t)m * lda + k) : zero;
             }
         }
+    };
+    auto load_b = [&](int k0) {
 #pragma unroll
         for (int e = 0; e < HN * HK / 512; ++e) {
             const int v = e * 128 + tid;
@@ -196,7 +221,12 @@ __global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const
             }
         }
     };
-    load(0);
+    load_b(0);
+    if (PDL) {
+        pdl_wait();
+        pdl_trigger();
+    }
+    load_a(0);
     for (int k0 = 0; k0 < K; k0 += HK) {
         __syncthreads();
 #pragma unroll
@@ -220,7 +250,10 @@ __global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const
             }
         }
         __syncthreads();
-        if (k0 + HK < K) load(k0 + HK);
+        if (k0 + HK < K) {
+            load_a(k0 + HK);
+            load_b(k0 + HK);
+        }
         const int ke = min(HK, (K - k0 + 3) & ~3);   // beyond K both are 0
 #pragma unroll 4
         for (int k = 0; k < ke; k += 4) {
@@ -260,6 +293,22 @@ __global__ void __launch_bounds__(128) k_head(const float* __restrict__ A, const
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[j] = fmaxf(acc[j], 0.f);
     *reinterpret_cast<float4*>(C + (int64_t)m * ldc + n) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+}
+
+template <bool TA, bool TB, int EPI, bool PDL>
+__global__ void __launch_bounds__(128) k_head(const HeadArgs H) {
+    __shared__ HeadSmem S;
+    head_tile<TA, TB, EPI, PDL>(H, S, blockIdx.x, blockIdx.y);
+}
+
+// A layer's two gradients in one launch: the weights' (with the bias's, column
+// sums) by the first `tiles` CTAs and the input's, gated or not, by the others.
+template <int EPI>
+__global__ void __launch_bounds__(128) k_head_back(const HeadArgs W, const HeadArgs X, int tiles, int wx, int xx) {
+    __shared__ HeadSmem S;
+    const int t = blockIdx.x;
+    if (t < tiles) head_tile<true, false, HEAD_COLSUM>(W, S, t % wx, t / wx);
+    else head_tile<false, true, EPI>(X, S, (t - tiles) % xx, (t - tiles) / xx);
 }
 
 __global__ void k_scale_points(const float* __restrict__ x, int64_t n, float inv, float* __restrict__ y) {
@@ -626,13 +675,34 @@ void gemm(cudaStream_t s, const float* A, const float* B, float* C, const float*
     k_gemm<<<dim3((N + GT - 1) / GT, (M + GT - 1) / GT), 256, 0, s>>>(A, B, C, bias, M, N, K);
 }
 
-template <bool TA, bool TB, int EPI>
-void head(cudaStream_t s, const float* A, const float* B, float* C, const float* aux, float* colsum, int M, int N, int K,
-          int lda, int ldb, int ldc) {
-    static_assert(OB1 % 4 == 0 && OW4 % 4 == 0 && OB4 % 4 == 0 && OW5 % 4 == 0 && OB5 % 4 == 0 && NOUT % 4 == 0,
-                  "k_head's loads of four floats");
-    const dim3 grid((N + HN - 1) / HN, (M + HM - 1) / HM);
-    k_head<TA, TB, EPI><<<grid, 128, 0, s>>>(A, B, C, aux, colsum, M, N, K, lda, ldb, ldc);
+static_assert(OB1 % 4 == 0 && OW4 % 4 == 0 && OB4 % 4 == 0 && OW5 % 4 == 0 && OB5 % 4 == 0 && NOUT % 4 == 0,
+              "head_tile's loads of four floats");
+// A forward product of the head, started while the kernel before it ends.
+template <int EPI>
+cudaError_t head(cudaStream_t s, const float* X, const float* W, const float* bias, float* Y, int B, int K, int N) {
+    const HeadArgs H = {X, W, Y, bias, nullptr, B, N, K, K, N, N};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((N + HN - 1) / HN, (B + HM - 1) / HM);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_head<false, false, EPI, true>, H);
+}
+
+// Gradients of Y = X W + b from dY [B x N]: dW [K x N] = X^T dY, db, and dX = dY W^T,
+// with HEAD_GATE only where X > 0.
+template <int EPI>
+void head_back(cudaStream_t s, const float* X, const float* W, const float* dY, float* dW, float* db, float* dX, int B,
+               int K, int N) {
+    const HeadArgs w = {X, dY, dW, nullptr, db, K, N, B, K, N, N};
+    const HeadArgs x = {dY, W, dX, X, nullptr, B, K, N, N, N, K};
+    const int wx = (N + HN - 1) / HN, wt = wx * ((K + HM - 1) / HM), xx = (K + HN - 1) / HN;
+    const int64_t tiles = wt + (int64_t)xx * ((B + HM - 1) / HM);
+    k_head_back<EPI><<<(unsigned)tiles, 128, 0, s>>>(w, x, wt, wx, xx);
 }
 
 // BF16 image of the per-point weights, refreshed after every parameter update
@@ -659,8 +729,8 @@ int forward(mp_pn* net, const float* scans, int B, bool train) {
         gemm(s, net->h2, W + OW3, net->h3, W + OB3, (int)rows, C3, C2);
         k_maxpool<<<dim3(C3 / 128, B), 128, 0, s>>>(net->h3, B, net->P, net->g, net->gi);
     }
-    head<false, false, HEAD_BIAS | HEAD_RELU>(s, net->g, W + OW4, net->h4, W + OB4, nullptr, B, C4, C3, C3, C4, C4);
-    head<false, false, HEAD_BIAS>(s, net->h4, W + OW5, net->o, W + OB5, nullptr, B, NOUT, C4, C4, NOUT, NOUT);
+    PN_CUDA((head<HEAD_BIAS | HEAD_RELU>(s, net->g, W + OW4, W + OB4, net->h4, B, C3, C4)));
+    PN_CUDA((head<HEAD_BIAS>(s, net->h4, W + OW5, W + OB5, net->o, B, C4, NOUT)));
     PN_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -780,10 +850,8 @@ int mp_pn_loss_grad(mp_pn* net, const float* scans, const float* targets, int B,
     PN_CUDA(cudaMemsetAsync(loss_dev, 0, sizeof(float), s));
     k_mdn_loss<<<grid_for(B, 2), 64, 0, s>>>(net->o, targets, B, net->dO, loss_dev);
     // head
-    head<true, false, HEAD_COLSUM>(s, net->h4, net->dO, G + OW5, nullptr, G + OB5, C4, NOUT, B, C4, NOUT, NOUT);
-    head<false, true, HEAD_GATE>(s, net->dO, W + OW5, net->dh4, net->h4, nullptr, B, C4, NOUT, NOUT, NOUT, C4);
-    head<true, false, HEAD_COLSUM>(s, net->g, net->dh4, G + OW4, nullptr, G + OB4, C3, C4, B, C3, C4, C4);
-    head<false, true, 0>(s, net->dh4, W + OW4, net->dg, nullptr, nullptr, B, C3, C4, C4, C4, C3);
+    head_back<HEAD_GATE>(s, net->h4, W + OW5, net->dO, G + OW5, G + OB5, net->dh4, B, C4, NOUT);
+    head_back<0>(s, net->g, W + OW4, net->dh4, G + OW4, G + OB4, net->dg, B, C3, C4);
     // max-pool and the shared layers, on the pooled rows (c, b) only
     PoolArgs pa = {};
     pa.dg = net->dg; pa.g = net->g; pa.gi = net->gi;
