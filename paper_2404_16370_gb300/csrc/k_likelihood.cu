@@ -716,6 +716,8 @@ __device__ __forceinline__ void LkOp<WPP, V>::run(const LkArgs& A, unsigned bxi,
 
 template <int WPP, typename V>
 __global__ void __launch_bounds__(LK_THREADS, LK_MINB) k_likelihood(const LkArgs A) {
+    pdl_wait();
+    pdl_trigger();
     LkOp<WPP, V>::run(A, blockIdx.x, blockIdx.y);
 }
 
@@ -1341,8 +1343,7 @@ int launch_point_major(mp_ctx* c, LkArgs A) {
     const dim3 grid((unsigned)lk_blocks(A), (unsigned)A.split);
     const int segs = lk_segments(c->n_scan, A);
     for (A.seg = 0; A.seg < segs; ++A.seg) {
-        if (A.wpp > 1) k_likelihood<LK_WARPS, V><<<grid, LK_THREADS, 0, c->stream>>>(A);
-        else k_likelihood<1, V><<<grid, LK_THREADS, 0, c->stream>>>(A);
+        MP_CUDA(c, launch_next(A.wpp > 1 ? k_likelihood<LK_WARPS, V> : k_likelihood<1, V>, grid, LK_THREADS, 0, c->stream, A));
         MP_LAUNCHED(c);
     }
     return MP_OK;

@@ -543,11 +543,16 @@ __device__ __forceinline__ void scan_run(const ScanArgs2& A) {
     const ScanArgs& a = A.s[blockIdx.y];
     if (blockIdx.x * PTS < (unsigned)a.n) Op::run(a, blockIdx.x, 0);
 }
-__global__ void __launch_bounds__(256) k_scan_to_float4(const __grid_constant__ ScanArgs2 A) { scan_run<ScanF4Op, 256>(A); }
+__global__ void __launch_bounds__(256) k_scan_to_float4(const __grid_constant__ ScanArgs2 A) {
+    pdl_trigger();
+    scan_run<ScanF4Op, 256>(A);
+}
 __global__ void __launch_bounds__(NRM_CTA) k_scan_normals(const __grid_constant__ ScanArgs2 A) {
+    pdl_wait();   // (no trigger: the sort's waiting CTAs took 11 us from 4999 points' normals)
     scan_run<ScanNormalsOp, NRM_PTS>(A);
 }
 __global__ void __launch_bounds__(SCAN_CTA) k_scan_sort(const __grid_constant__ ScanArgs2 A) {
+    pdl_wait();
     scan_run<ScanSortOp, SCAN_PTS>(A);
 }
 
@@ -813,9 +818,9 @@ static int launch_scans(mp_ctx* c, const ScanArgs2& A, int m, cudaStream_t s) {
     const int n = m > 1 ? std::max(A.s[0].n, A.s[1].n) : A.s[0].n;
     k_scan_to_float4<<<dim3(grid_for(n, 256), m), 256, 0, s>>>(A);
     MP_LAUNCHED(c);
-    k_scan_normals<<<dim3(grid_for(n, NRM_PTS), m), NRM_CTA, 0, s>>>(A);
+    MP_CUDA(c, launch_next(k_scan_normals, dim3(grid_for(n, NRM_PTS), m), NRM_CTA, 0, s, A));
     MP_LAUNCHED(c);
-    k_scan_sort<<<dim3(grid_for(n, SCAN_PTS), m), SCAN_CTA, 0, s>>>(A);
+    MP_CUDA(c, launch_next(k_scan_sort, dim3(grid_for(n, SCAN_PTS), m), SCAN_CTA, 0, s, A));
     MP_LAUNCHED(c);
     return MP_OK;
 }

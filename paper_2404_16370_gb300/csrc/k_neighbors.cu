@@ -160,7 +160,11 @@ __device__ __forceinline__ void LshOp::run(const LshArgs& A, unsigned bx, unsign
     A.buckets[i] = key & A.mask;
 }
 
-__global__ void __launch_bounds__(256) k_lsh_keys(const LshArgs A) { LshOp::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(256) k_lsh_keys(const LshArgs A) {
+    pdl_wait();
+    pdl_trigger();
+    LshOp::run(A, blockIdx.x, 0);
+}
 
 // ---------------------------------------------------------------------------
 // stable LSD radix sort of (bucket, id), 8-bit digits, 2048 elements per block
@@ -575,7 +579,11 @@ struct SmallSortOp {
     }
 };
 
-__global__ void __launch_bounds__(SS_THREADS) k_small_sort(const SmallSortArgs A) { SmallSortOp::run(A, 0, 0); }
+__global__ void __launch_bounds__(SS_THREADS) k_small_sort(const SmallSortArgs A) {
+    pdl_wait();
+    pdl_trigger();
+    SmallSortOp::run(A, 0, 0);
+}
 
 // ---------------------------------------------------------------------------
 // the whole sort of a middling instance in one cooperative launch
@@ -889,7 +897,10 @@ __device__ __forceinline__ void MergeOp::run(const MergeArgs& args, unsigned bx,
     }
 }
 
-__global__ void __launch_bounds__(256) k_merge(const MergeArgs A) { MergeOp::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(256) k_merge(const MergeArgs A) {
+    pdl_wait();
+    MergeOp::run(A, blockIdx.x, 0);
+}
 
 // ---------------------------------------------------------------------------
 // the LSH / sort / visiting-order phase of a batch as one persistent kernel
@@ -1131,7 +1142,7 @@ MergeArgs merge_args(mp_ctx* c, int cur) {
 }  // namespace
 
 int mp_launch_lsh_keys(mp_ctx* c) {
-    k_lsh_keys<<<grid_for(c->n, 256), 256, 0, c->stream>>>(lsh_args(c, c->step_dev));
+    MP_CUDA(c, launch_next(k_lsh_keys, grid_for(c->n, 256), 256, 0, c->stream, lsh_args(c, c->step_dev)));
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -1149,7 +1160,7 @@ int mp_launch_sort(mp_ctx* c) {
     }
     if (c->n <= SS_MAX) {
         MP_CUDA(c, small_sort_prepare((const void*)k_small_sort));
-        k_small_sort<<<1, SS_THREADS, sizeof(SmallSortSmem), c->stream>>>(small_sort_args(c));
+        MP_CUDA(c, launch_next(k_small_sort, 1, SS_THREADS, sizeof(SmallSortSmem), c->stream, small_sort_args(c)));
         MP_LAUNCHED(c);
         return MP_OK;
     }
@@ -1195,7 +1206,7 @@ int mp_launch_sort(mp_ctx* c) {
 }
 
 int mp_launch_merge(mp_ctx* c) {
-    k_merge<<<grid_for(c->n * 32, 256), 256, 0, c->stream>>>(merge_args(c, c->nbr_cur));
+    MP_CUDA(c, launch_next(k_merge, grid_for(c->n * 32, 256), 256, 0, c->stream, merge_args(c, c->nbr_cur)));
     MP_LAUNCHED(c);
     c->nbr_cur ^= 1;
     return MP_OK;

@@ -245,8 +245,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_pn_mlp_tc(const MlpArgs A) {
     const uint32_t off_h1 = OFF_H + (uint32_t)group * 3u * SW_BLOCK, off_h2 = off_h1 + SW_BLOCK;
     uint64_t* const bar = bars + 2 * group;         // bar[1], bar[2]: this group's
 
-    // a dependent launch (the head) may take its place: it waits for this kernel's end
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_trigger();
     for (int e = threadIdx.x; e < 3 * 64; e += TC_THREADS) sW1[e] = A.W1[e];
     for (int e = threadIdx.x; e < 64; e += TC_THREADS) sb1[e] = A.b1[e];
     for (int e = threadIdx.x; e < 128; e += TC_THREADS) sb2[e] = A.b2[e];

@@ -150,8 +150,9 @@ __global__ void __launch_bounds__(256) k_gemm(const float* __restrict__ A, const
 // batch: few rows, so what counts is latency and CTAs. A CTA of 128 threads takes
 // 16 x 32 outputs (4 a thread) and stages 128 of K at a time, whole slices in
 // flight at once. A 64 x 64 tile with 16 of K a step left 7 CTAs waiting for 16
-// loads in a row: 46 us for 4 x 416 x 256, 7 now, of which 3 pass under the kernel before (head); the six products and
-// four column sums and gates of a training step at batch 128 320 us, 36 now.
+// loads in a row: 46 us for 4 x 416 x 256, 7 now, of which 3 pass under the kernel before
+// (head); the six products and four column sums and gates of a training step at
+// batch 128 320 us, 36 now.
 // N and the extents along which op(A) and op(B) are contiguous are multiples of
 // 4, the matrices 16-byte aligned. Each output is one chain of fmaf over k.
 enum : int { HEAD_BIAS = 1, HEAD_RELU = 2, HEAD_GATE = 4, HEAD_COLSUM = 8 };
@@ -171,11 +172,6 @@ struct HeadSmem {
     __align__(16) float Bs[HK][HN + 4];
     float cs[4][HN];
 };
-
-// A dependent launch's wait for the kernels before it, and the word to one that
-// it may start. Without the launch attribute both do nothing.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // PDL: op(B) is a weight matrix, which the kernels just before do not write: its
 // first slice is asked for before the wait for them.
@@ -681,16 +677,7 @@ static_assert(OB1 % 4 == 0 && OW4 % 4 == 0 && OB4 % 4 == 0 && OW5 % 4 == 0 && OB
 template <int EPI>
 cudaError_t head(cudaStream_t s, const float* X, const float* W, const float* bias, float* Y, int B, int K, int N) {
     const HeadArgs H = {X, W, Y, bias, nullptr, B, N, K, K, N, N};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((N + HN - 1) / HN, (B + HM - 1) / HM);
-    cfg.blockDim = dim3(128);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_head<false, false, EPI, true>, H);
+    return launch_next(k_head<false, false, EPI, true>, dim3((N + HN - 1) / HN, (B + HM - 1) / HM), 128, 0, s, H);
 }
 
 // Gradients of Y = X W + b from dY [B x N]: dW [K x N] = X^T dY, db, and dX = dY W^T,

@@ -71,7 +71,10 @@ __device__ __forceinline__ void PredOp::run(const PredArgs& A, unsigned bx, unsi
     store_pose(A.poses, i, q, t);
 }
 
-__global__ void __launch_bounds__(256) k_predict(const PredArgs A) { PredOp::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(256) k_predict(const PredArgs A) {
+    pdl_trigger();
+    PredOp::run(A, blockIdx.x, 0);
+}
 
 struct SolveArgs {
     const float* gn;
@@ -198,7 +201,11 @@ __device__ __forceinline__ void SolveOp::run(const SolveArgs& args, unsigned bx,
     n_in[i] = cnt;
 }
 
-__global__ void __launch_bounds__(128) k_solve(const SolveArgs A) { SolveOp::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(128) k_solve(const SolveArgs A) {
+    pdl_wait();
+    pdl_trigger();
+    SolveOp::run(A, blockIdx.x, 0);
+}
 
 struct SvgdArgs {
     float4* poses;
@@ -301,7 +308,10 @@ __device__ __forceinline__ void SvgdOp<G, PRE>::run(const SvgdArgs& A, unsigned 
 }
 
 template <int G, bool PRE>
-__global__ void __launch_bounds__(256) k_svgd(const SvgdArgs A) { SvgdOp<G, PRE>::run(A, blockIdx.x, 0); }
+__global__ void __launch_bounds__(256) k_svgd(const SvgdArgs A) {
+    pdl_wait();
+    SvgdOp<G, PRE>::run(A, blockIdx.x, 0);
+}
 
 struct InitArgs {
     float4* poses;
@@ -455,8 +465,8 @@ int svgd_lanes(int K) {
 template <int G>
 int launch_svgd_g(mp_ctx* c) {
     const unsigned grid = grid_for(c->n * G, 256);
-    if (c->p.svgd_precond) k_svgd<G, true><<<grid, 256, 0, c->stream>>>(svgd_args(c, c->nbr_cur));
-    else k_svgd<G, false><<<grid, 256, 0, c->stream>>>(svgd_args(c, c->nbr_cur));
+    MP_CUDA(c, launch_next(c->p.svgd_precond ? k_svgd<G, true> : k_svgd<G, false>, grid, 256, 0, c->stream,
+                           svgd_args(c, c->nbr_cur)));
     MP_LAUNCHED(c);
     return MP_OK;
 }
@@ -489,7 +499,7 @@ int mp_launch_predict(mp_ctx* c) {
 }
 
 int mp_launch_solve(mp_ctx* c) {
-    k_solve<<<grid_for(c->n, 128), 128, 0, c->stream>>>(solve_args(c));
+    MP_CUDA(c, launch_next(k_solve, grid_for(c->n, 128), 128, 0, c->stream, solve_args(c)));
     MP_LAUNCHED(c);
     return MP_OK;
 }

@@ -430,6 +430,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 #define MP_WAIT_BUDGET (4000000000LL)   // ~2 s at 2 GHz
 #define MP_ERR_WAIT 1
 
+// A kernel launched by launch_next may start while the kernel before it on the
+// stream ends, once every CTA of that one has called pdl_trigger() or is done.
+// pdl_wait() then waits for that kernel's end and makes its writes (and those of
+// the kernels it waited for) visible: it comes before the first access to memory
+// that any of them touches. Launched in another way, the two calls do nothing.
+// What this saves is the launch, 1 to 3 us a kernel.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Grid-wide barrier of a cooperative (persistent) launch, whose CTAs are all
 // resident at once. Thread 0 of each CTA arrives on a counter that only grows
 // and spins until it reaches this barrier's target, the arrivals of all
@@ -697,6 +706,20 @@ inline void plan_coop(std::vector<GOp>& plan, const void* func, unsigned grid, u
     plan.push_back(o);
 }
 // A cooperative launch on a stream (also inside a stream capture).
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 inline cudaError_t launch_coop(const void* func, unsigned grid, unsigned block, void* arg, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
