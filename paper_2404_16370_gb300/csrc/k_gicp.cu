@@ -2,8 +2,8 @@
 // ~ T_{t-1}^-1 T_t from the current scan (source) and the previous one
 // (target), and Sigma^DeltaT from the Gauss-Newton Hessian at the result.
 //
-// One cooperative kernel runs all iterations on the sorted valid points of both
-// scans. For the current estimate T = (R, t) (FP64, in shared memory):
+// One cooperative kernel runs all iterations on the sorted points of both scans
+// (those without a normal at 1e18 m: out of reach as targets, skipped as sources). For the current estimate T = (R, t) (FP64, in shared memory):
 //  * decisions in FP32 on T's rounding to float (R from the unit quaternion,
 //    q = R mu + t by the fixed sequence, squared distances un-fused); the
 //    correspondence is the target point of smallest squared distance, ties to
@@ -21,10 +21,10 @@
 //    Sigma^DeltaT = H^-1 is taken on the host.
 // Bound by latency: at two scans of 8192 points 37 us an iteration, 13 of them
 // the barrier and the FP64 step (28 with its instructions on one thread) and the
-// rest the search (75 us without the last correspondence as a bound); the point
-// Gaussians before it, 170 us, are the larger part. mp_gicp at 8192 points and
+// rest the search (75 us without the last correspondence as a bound), before it
+// 57 us for the scans' order and 89 for their normals. mp_gicp at 8192 points and
 // six iterations: 3930 us with all pairs of points tested and two launches an
-// iteration, 540 now.
+// iteration, 458 now.
 #include "mp_internal.cuh"
 
 #include <algorithm>
@@ -35,8 +35,8 @@ struct GicpBufs {
     int cap;
     float *src_raw, *tgt_raw, *src_n, *tgt_n;
     uint8_t *src_v, *tgt_v;
-    float *src_soa, *tgt_soa;      // the valid points, sorted (scan_word)
-    int32_t *tgt_idx, *counts;     // their original indices; valid points of src and tgt, error bits
+    float *sorted, *src_soa, *tgt_soa;   // the points, sorted (scan_word): two scans' points; with their normals
+    int32_t *idx, *tgt_idx, *counts;     // their original indices; points of src and tgt, error bits
     float4* tmp4;
     float* box;         // target tiles' bounding boxes
     int32_t* corr;      // correspondences
@@ -59,12 +59,12 @@ constexpr int GTILE = 64;      // target points per tile
 constexpr int NPART = 32;      // floats per partial: 27 sums + count (+ pad)
 constexpr int ST_Q = 0, ST_T = 4, ST_H = 7, ST_DONE = 28, ST_IT = 29, ST_NC = 30, ST_N = 32;
 
-// One registration. Scans: sorted valid points in chunks of six planes
-// (scan_word), their original indices, and their number in device memory.
+// One registration. Scans: sorted points and normals in chunks of six planes
+// (scan_word), invalid points at 1e18 m, and the points' original indices.
 struct GicpArgs {
     const float *src, *tgt;
-    const int32_t *tgt_idx, *n_src, *n_tgt;
-    int cap_src, cap_tgt;    // points the host gave (bounds of the counts)
+    const int32_t* tgt_idx;
+    int n_src, n_tgt;
     float* box;              // 6 per target tile: lower and upper corner
     int32_t* corr;           // a source point's correspondence in the last iteration
     double* state;
@@ -78,6 +78,8 @@ struct GicpArgs {
 };
 
 __device__ __forceinline__ float gicp_word(const float* s, int i, int k) { return __ldg(s + scan_word(i, k)); }
+
+__device__ __forceinline__ bool gicp_valid(const float* s, int i) { return gicp_word(s, i, 0) < 1e17f; }
 
 // Nearest target point (squared distance by the decision sequence, ties to the
 // smaller original index) of this thread's source point, over the tiles whose
@@ -397,7 +399,7 @@ __global__ void __launch_bounds__(GB) k_gicp(const GicpArgs A) {
     __shared__ double part_s[GB / 32][NPART], S[NPART], st[ST_N], M[6][7], T[27];
     __shared__ GicpPose P;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int ns = min(max(*A.n_src, 0), A.cap_src), nt = min(max(*A.n_tgt, 0), A.cap_tgt);
+    const int ns = A.n_src, nt = A.n_tgt;
     if (threadIdx.x < ST_N) st[threadIdx.x] = A.state[threadIdx.x];
     __syncthreads();
     // the target tiles' boxes
@@ -406,10 +408,11 @@ __global__ void __launch_bounds__(GB) k_gicp(const GicpArgs A) {
         float lo[3], hi[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const int j0 = min(t * GTILE + lane, nt - 1), j1 = min(t * GTILE + 32 + lane, nt - 1);
-            const float u = gicp_word(A.tgt, j0, a), v = gicp_word(A.tgt, j1, a);
-            lo[a] = fminf(u, v);
-            hi[a] = fmaxf(u, v);
+            const int j0 = t * GTILE + lane, j1 = j0 + 32;
+            const bool in0 = j0 < nt && gicp_valid(A.tgt, j0), in1 = j1 < nt && gicp_valid(A.tgt, j1);
+            const float u = in0 ? gicp_word(A.tgt, j0, a) : 0.f, v = in1 ? gicp_word(A.tgt, j1, a) : 0.f;
+            lo[a] = fminf(in0 ? u : INFINITY, in1 ? v : INFINITY);
+            hi[a] = fmaxf(in0 ? u : -INFINITY, in1 ? v : -INFINITY);   // (none: no point is near the box)
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
@@ -447,9 +450,9 @@ __global__ void __launch_bounds__(GB) k_gicp(const GicpArgs A) {
         for (int a = 0; a < NPART; ++a) acc[a] = 0.f;
         for (int k0 = blockIdx.x * GPTS; k0 < ns; k0 += gridDim.x * GPTS) {
             const int k = k0 + threadIdx.x / GPARTS;
-            const bool have = k < ns;
+            const bool have = k < ns && gicp_valid(A.src, k);
             // transformed source point by the decision sequence
-            const int kk = have ? k : ns - 1;
+            const int kk = min(k, ns - 1);
             const float m[3] = {gicp_word(A.src, kk, 0), gicp_word(A.src, kk, 1), gicp_word(A.src, kk, 2)};
             float qt[3], q[3];
 #pragma unroll
@@ -505,7 +508,7 @@ int gicp_alloc(mp_ctx* c) {
     A(&g->src_raw, 3 * (size_t)cap); A(&g->tgt_raw, 3 * (size_t)cap); A(&g->src_n, 3 * (size_t)cap);
     A(&g->tgt_n, 3 * (size_t)cap); A(&g->src_v, cap); A(&g->tgt_v, cap); A(&g->tmp4, 2 * (size_t)cap);
     const size_t soa = scan_word((cap + MP_SCAN_CHUNK - 1) / MP_SCAN_CHUNK * MP_SCAN_CHUNK, 0);
-    A(&g->src_soa, soa); A(&g->tgt_soa, soa); A(&g->tgt_idx, cap); A(&g->counts, 3);
+    A(&g->sorted, 2 * soa); A(&g->src_soa, soa); A(&g->tgt_soa, soa); A(&g->idx, cap); A(&g->tgt_idx, cap); A(&g->counts, 3);
     A(&g->box, 6 * (size_t)((cap + GTILE - 1) / GTILE)); A(&g->corr, cap); A(&g->bar, 1);
     int dev = 0, sms = 0, per = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -550,8 +553,8 @@ bool inv6(const double H[36], double I[36]) {
 void mp_gicp_free(mp_ctx* c) {
     GicpBufs* g = c->gicp;
     if (!g) return;
-    void* bufs[] = {g->src_raw, g->tgt_raw, g->src_n, g->tgt_n, g->src_v, g->tgt_v, g->src_soa,
-                    g->tgt_soa, g->tgt_idx, g->counts, g->tmp4, g->box, g->corr, g->bar, g->partial, g->state, g->prev};
+    void* bufs[] = {g->src_raw, g->tgt_raw, g->src_n, g->tgt_n, g->src_v, g->tgt_v, g->sorted,
+                    g->src_soa, g->tgt_soa, g->idx, g->tgt_idx, g->counts, g->tmp4, g->box, g->corr, g->bar, g->partial, g->state, g->prev};
     for (void* p : bufs)
         if (p) cudaFree(p);
     delete g;
@@ -571,9 +574,10 @@ int mp_gicp(mp_ctx* c, const float* src, int32_t n_src, const float* tgt, int32_
     GicpBufs* g = c->gicp;
     MP_CUDA(c, cudaMemcpyAsync(g->src_raw, src, sizeof(float) * 3 * (size_t)n_src, cudaMemcpyDefault, c->stream));
     MP_CUDA(c, cudaMemcpyAsync(g->tgt_raw, tgt, sizeof(float) * 3 * (size_t)n_tgt, cudaMemcpyDefault, c->stream));
+    float* sorted = g->sorted + scan_word((g->cap + MP_SCAN_CHUNK - 1) / MP_SCAN_CHUNK * MP_SCAN_CHUNK, 0);
     const PointScan scans[2] = {
-        {g->src_raw, n_src, g->tmp4, g->src_n, g->src_v, g->src_soa, nullptr, g->counts},
-        {g->tgt_raw, n_tgt, g->tmp4 + g->cap, g->tgt_n, g->tgt_v, g->tgt_soa, g->tgt_idx, g->counts + 1}};
+        {g->src_raw, n_src, g->tmp4, g->src_n, g->src_v, g->sorted, g->src_soa, g->idx, g->counts},
+        {g->tgt_raw, n_tgt, g->tmp4 + g->cap, g->tgt_n, g->tgt_v, sorted, g->tgt_soa, g->tgt_idx, g->counts + 1}};
     if ((rc = mp_launch_point_gaussians(c, scans, 2))) return rc;
     // initial state from init_T (identity when NULL)
     double st[ST_N];
@@ -588,10 +592,8 @@ int mp_gicp(mp_ctx* c, const float* src, int32_t n_src, const float* tgt, int32_
     A.src = g->src_soa;
     A.tgt = g->tgt_soa;
     A.tgt_idx = g->tgt_idx;
-    A.n_src = g->counts;
-    A.n_tgt = g->counts + 1;
-    A.cap_src = n_src;
-    A.cap_tgt = n_tgt;
+    A.n_src = n_src;
+    A.n_tgt = n_tgt;
     A.box = g->box;
     A.corr = g->corr;
     A.state = g->state;

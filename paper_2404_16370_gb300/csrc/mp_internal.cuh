@@ -573,10 +573,10 @@ struct PointScan {      // n x 3 points, and what is made of them
     const float* raw;
     int n;
     float4* tmp4;
-    float* normals;
+    float* normals;      // n x 3, which the sort copies along without need
     uint8_t* valid;
-    float* soa;
-    int32_t *idx, *nvalid;
+    float *sorted, *out;   // sorted points; with their normals, invalid ones at 1e18 m (scan_word)
+    int32_t *idx, *count;  // sorted points' indices, their number
 };
 int mp_launch_point_gaussians(mp_ctx* c, const PointScan* in, int m);
 int mp_launch_nnf_query(mp_ctx* c, const int32_t* vox_dev, int64_t m, int32_t* out_dev);
