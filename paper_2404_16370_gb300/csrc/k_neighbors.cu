@@ -122,15 +122,16 @@ __device__ __forceinline__ void log_se3_d(double qx, double qy, double qz, doubl
 struct LshOp {
     using Args = LshArgs;
     static constexpr int THREADS = 256, MINB = 1;
-    static __device__ __forceinline__ void run(const LshArgs& A, unsigned bx, unsigned);
+    static __device__ __forceinline__ void key(const LshArgs& A, int64_t i);   // of particle i
+    static __device__ __forceinline__ void run(const LshArgs& A, unsigned bx, unsigned) {
+        key(A, (int64_t)bx * THREADS + threadIdx.x);
+    }
 };
 
-__device__ __forceinline__ void LshOp::run(const LshArgs& A, unsigned bx, unsigned) {
+__device__ __forceinline__ void LshOp::key(const LshArgs& A, int64_t i) {
     const float4* __restrict__ poses = A.poses;
     const StepDev* __restrict__ sd = A.sd;
-    const int64_t n = A.n;
-    int64_t i = (int64_t)bx * THREADS + threadIdx.x;
-    if (i >= n) return;
+    if (i >= A.n) return;
     float4 a = poses[2 * i], b = poses[2 * i + 1];
     double qx = a.x, qy = a.y, qz = a.z, qw = a.w;
     double nrm = rsqrt(fma(qw, qw, fma(qz, qz, fma(qy, qy, qx * qx))));
@@ -149,21 +150,25 @@ __device__ __forceinline__ void LshOp::run(const LshArgs& A, unsigned bx, unsign
     double xi[6];
     log_se3_d(rx, ry, rz, rw, t, xi);
     const uint32_t P[6] = {73856093u, 19349663u, 83492791u, 2654435761u, 805459861u, 3674653429u};
-    uint32_t key = 0;
+    uint32_t h = 0;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         double z = fma(A.scale[k], xi[k], sd->lsh_delta[k]);
         int cell = (int)floor(z);
-        key ^= (uint32_t)cell * P[k];
+        h ^= (uint32_t)cell * P[k];
     }
-    A.keys[i] = key;
-    A.buckets[i] = key & A.mask;
+    A.keys[i] = h;
+    A.buckets[i] = h & A.mask;
 }
 
-__global__ void __launch_bounds__(256) k_lsh_keys(const LshArgs A) {
+// (a warp on each quarter of an SM: an FP64 instruction holds the quarter for 64
+// cycles, so the second warp there of a 256-thread CTA waited: up to 19456 particles
+// 16.3 -> 11.8 us, 50021 29 -> 22)
+constexpr int LSH_THREADS = 128;
+__global__ void __launch_bounds__(LSH_THREADS) k_lsh_keys(const LshArgs A) {
     pdl_wait();
     pdl_trigger();
-    LshOp::run(A, blockIdx.x, 0);
+    LshOp::key(A, (int64_t)blockIdx.x * LSH_THREADS + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1142,7 +1147,7 @@ MergeArgs merge_args(mp_ctx* c, int cur) {
 }  // namespace
 
 int mp_launch_lsh_keys(mp_ctx* c) {
-    MP_CUDA(c, launch_next(k_lsh_keys, grid_for(c->n, 256), 256, 0, c->stream, lsh_args(c, c->step_dev)));
+    MP_CUDA(c, launch_next(k_lsh_keys, grid_for(c->n, LSH_THREADS), LSH_THREADS, 0, c->stream, lsh_args(c, c->step_dev)));
     MP_LAUNCHED(c);
     return MP_OK;
 }
