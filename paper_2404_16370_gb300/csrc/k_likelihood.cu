@@ -41,7 +41,8 @@
 // 55 to 72%). Measured on one GB300, likelihood stage, every size
 // particle-major before -> now: 256 x 128 points 29 -> 8.2 us, 4096 x 512 147
 // -> 26.7 us, 10000 x 2048 688 -> 178 us, 16000 x 1021 in BF16 593 -> 147 us,
-// 50021 x 4999 (outdoor) 3.53 -> 1.83 ms; particle-major in parts, 2^17 x 512
+// 50021 x 4999 (outdoor, one particle a thread) 3.53 -> 2.07 ms; particle-major in
+// parts, 2^17 x 512
 // 426 -> 392 us, 2^17 x 8192 10.4 -> 8.2 ms, 2^18 x 8192 around the sensor 17.7
 // -> 16.7 ms, 2^20 x 8192 52.8 -> 52.4 ms.
 #include "mp_internal.cuh"
@@ -65,12 +66,15 @@ constexpr int LK_CHUNK_BYTES = 6 * LK_CHUNK * 4;
 constexpr int LK_QCAP = LK_CHUNK + 64;           // entries of a warp's queue
 
 constexpr int64_t LK_PM_MIN = 80 << 10;          // lk_particle_major()
+constexpr int LK_WIDE = 512;                     // (voxels across a map)
+constexpr int64_t LK_PM1_MAX = 112 << 10;        // of a wide map: one particle per thread
 
 constexpr int PM_THREADS = 128;                  // particle-major form: two particles per thread
 constexpr int PM_PER_CTA = 2 * PM_THREADS;
 constexpr int PM_CHUNK = 128;   // points per stage: 128 x 48 B = 6 KB (smaller stages leave L1 more room
                                 // for the gathers: 3% faster with converged particles than 256)
 constexpr int PM_MINB = 3;      // 163 registers
+constexpr int PM1_MINB = 3;     // one particle per thread, gathers in groups of four: 139 registers
 constexpr int PMH_MINB = 4;     // its 16-bit forms: their per-pair values take half the registers, so a
                                 // fourth CTA (16 warps per SM) fits in 128 registers
 
@@ -119,11 +123,32 @@ __device__ __forceinline__ float2 neg2(float2 v) {
                        __uint_as_float(__float_as_uint(v.y) ^ 0x80000000u));
 }
 
-struct Lk2Acc {
-    float2 Hww[6], Hwv[9], Hvv[6], bw[3], nbv[3];   // nbv = -bv
-    float2 lc;    // sum of the inlier costs
-    float2 cnt;   // inlier count
+// The same operations on one value: a P is a pair (float2) or one (float).
+__device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul2(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float neg2(float v) { return __uint_as_float(__float_as_uint(v) ^ 0x80000000u); }
+__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) { return __fadd2_rd(a, b); }
+__device__ __forceinline__ float add2_rd(float a, float b) { return __fadd_rd(a, b); }
+__device__ __forceinline__ float first(float2 v) { return v.x; }
+__device__ __forceinline__ float first(float v) { return v; }
+__device__ __forceinline__ float second(float2 v) { return v.y; }
+__device__ __forceinline__ float second(float v) { return v; }
+template <typename P>
+__device__ __forceinline__ P pk(float a, float b) {
+    if constexpr (sizeof(P) == sizeof(float2)) return make_float2(a, b);
+    else return a;
+}
+template <typename P>
+__device__ __forceinline__ P pk(float2 both) { return pk<P>(both.x, both.y); }
+
+template <typename P>
+struct LkSums {
+    P Hww[6], Hwv[9], Hvv[6], bw[3], nbv[3];   // nbv = -bv
+    P lc;    // sum of the inlier costs
+    P cnt;   // inlier count
 };
+using Lk2Acc = LkSums<float2>;
 
 // 1 / x to one ulp in one instruction (x is the product of two positive
 // information-matrix scalars, of the order of 4 eps_cov to 2)
@@ -230,9 +255,9 @@ struct LkRec {
     float2 a1, b1;
 };
 // What a pair keeps of its records: lever arm, residual, u + w' and u - w'.
-template <typename V>
+template <typename V, typename Q = float2>
 struct LkPair {
-    float2 qt[3];
+    Q qt[3];
     V e[3], s[3], d[3];
 };
 
@@ -243,25 +268,36 @@ __device__ __forceinline__ void lk_record(const LkArgs& A, int mm, float4& r0, f
 
 
 // The pair's residuals and normals from q, the scan normals nn and the records.
-__device__ __forceinline__ void lk_geometry(const LkArgs& A, const float2 R[9], const float2 q[3], const float2 nn[3],
-                                            const LkRec& r, LkPair<float2>& o) {
+template <typename P>
+__device__ __forceinline__ void lk_geometry_f(const LkArgs& A, const P R[9], const P q[3], const P nn[3], const LkRec& r,
+                                              LkPair<P, P>& o) {
+    const P m1 = pk<P>(A.m1);
     // residual e = mu^M - q
-    o.e[0] = make_float2(r.a0.x - q[0].x, r.b0.x - q[0].y);
-    o.e[1] = make_float2(r.a0.y - q[1].x, r.b0.y - q[1].y);
-    o.e[2] = make_float2(r.a0.z - q[2].x, r.b0.z - q[2].y);
+    o.e[0] = pk<P>(r.a0.x - first(q[0]), r.b0.x - second(q[0]));
+    o.e[1] = pk<P>(r.a0.y - first(q[1]), r.b0.y - second(q[1]));
+    o.e[2] = pk<P>(r.a0.z - first(q[2]), r.b0.z - second(q[2]));
     // u = R n (scan normal in the map frame), w = map normal
-    const float2 ux = fma2(R[2], nn[2], fma2(R[1], nn[1], mul2(R[0], nn[0])));
-    const float2 uy = fma2(R[5], nn[2], fma2(R[4], nn[1], mul2(R[3], nn[0])));
-    const float2 uz = fma2(R[8], nn[2], fma2(R[7], nn[1], mul2(R[6], nn[0])));
+    const P ux = fma2(R[2], nn[2], fma2(R[1], nn[1], mul2(R[0], nn[0])));
+    const P uy = fma2(R[5], nn[2], fma2(R[4], nn[1], mul2(R[3], nn[0])));
+    const P uz = fma2(R[8], nn[2], fma2(R[7], nn[1], mul2(R[6], nn[0])));
     // sign of u.w as an explicit fma chain (every instantiation rounds it the
     // same way)
-    const float sga = copysignf(1.f, fmaf(uz.x, r.a1.y, fmaf(uy.x, r.a1.x, ux.x * r.a0.w)));
-    const float sgb = copysignf(1.f, fmaf(uz.y, r.b1.y, fmaf(uy.y, r.b1.x, ux.y * r.b0.w)));
-    const float2 swx = make_float2(sga * r.a0.w, sgb * r.b0.w);
-    const float2 swy = make_float2(sga * r.a1.x, sgb * r.b1.x);
-    const float2 swz = make_float2(sga * r.a1.y, sgb * r.b1.y);
+    const float sga = copysignf(1.f, fmaf(first(uz), r.a1.y, fmaf(first(uy), r.a1.x, first(ux) * r.a0.w)));
+    const float sgb = copysignf(1.f, fmaf(second(uz), r.b1.y, fmaf(second(uy), r.b1.x, second(ux) * r.b0.w)));
+    const P swx = pk<P>(sga * r.a0.w, sgb * r.b0.w);
+    const P swy = pk<P>(sga * r.a1.x, sgb * r.b1.x);
+    const P swz = pk<P>(sga * r.a1.y, sgb * r.b1.y);
     o.s[0] = add2(ux, swx); o.s[1] = add2(uy, swy); o.s[2] = add2(uz, swz);
-    o.d[0] = fma2(A.m1, swx, ux); o.d[1] = fma2(A.m1, swy, uy); o.d[2] = fma2(A.m1, swz, uz);
+    o.d[0] = fma2(m1, swx, ux); o.d[1] = fma2(m1, swy, uy); o.d[2] = fma2(m1, swz, uz);
+}
+
+__device__ __forceinline__ void lk_geometry(const LkArgs& A, const float2 R[9], const float2 q[3], const float2 nn[3],
+                                            const LkRec& r, LkPair<float2>& o) {
+    lk_geometry_f<float2>(A, R, q, nn, r, o);
+}
+__device__ __forceinline__ void lk_geometry(const LkArgs& A, const float R[9], const float q[3], const float nn[3],
+                                            const LkRec& r, LkPair<float, float>& o) {
+    lk_geometry_f<float>(A, R, q, nn, r, o);
 }
 
 __device__ __forceinline__ void lk_pair(const LkArgs& A, const float2 R[9], const float2 t[3], const float* scan,
@@ -277,45 +313,48 @@ __device__ __forceinline__ void lk_pair(const LkArgs& A, const float2 R[9], cons
 }
 
 // va, vb: whether the pair's points count at all.
-__device__ __forceinline__ void lk_accumulate(const LkArgs& A, Lk2Acc& S, const LkPair<float2>& o, bool va, bool vb) {
-    const float2 qtx = o.qt[0], qty = o.qt[1], qtz = o.qt[2];
-    const float2 ex = o.e[0], ey = o.e[1], ez = o.e[2];
-    const float2 sx = o.s[0], sy = o.s[1], sz = o.s[2], dx = o.d[0], dy = o.d[1], dz = o.d[2];
-    const float2 nqx = neg2(qtx), nqy = neg2(qty), nqz = neg2(qtz);
+template <typename P>
+__device__ __forceinline__ void lk_accumulate_f(const LkArgs& A, LkSums<P>& S, const LkPair<P, P>& o, bool va, bool vb) {
+    const P half2 = pk<P>(A.half2), half_a2 = pk<P>(A.half_a2), nhalf_a2 = pk<P>(A.nhalf_a2), two_eps2 = pk<P>(A.two_eps2);
+    const P two2 = pk<P>(A.two2), quarter_a2 = pk<P>(A.quarter_a2);
+    const P qtx = o.qt[0], qty = o.qt[1], qtz = o.qt[2];
+    const P ex = o.e[0], ey = o.e[1], ez = o.e[2];
+    const P sx = o.s[0], sy = o.s[1], sz = o.s[2], dx = o.d[0], dy = o.d[1], dz = o.d[2];
+    const P nqx = neg2(qtx), nqy = neg2(qty), nqz = neg2(qtz);
     // closed-form Omega = I/2 + as s s^T + ad d d^T
-    const float2 dd = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-    const float2 ls = fma2(A.half_a2, dd, A.two_eps2);
-    const float2 ld = fma2(A.nhalf_a2, dd, A.two2);
-    const float2 pr = mul2(ls, ld);
-    const float2 rr = mul2(A.quarter_a2, make_float2(rcp1(pr.x), rcp1(pr.y)));
-    const float2 as = mul2(ld, rr), ad = mul2(ls, rr);
-    const float2 se = fma2(sz, ez, fma2(sy, ey, mul2(sx, ex)));
-    const float2 de = fma2(dz, ez, fma2(dy, ey, mul2(dx, ex)));
-    const float2 ee = fma2(ez, ez, fma2(ey, ey, mul2(ex, ex)));
-    const float2 cost = fma2(A.half2, ee, fma2(mul2(as, se), se, mul2(mul2(ad, de), de)));
-    const bool ia = va && (cost.x <= A.c_max);
-    const bool ib = vb && (cost.y <= A.c_max);
-    const float2 inl = make_float2(ia ? 1.f : 0.f, ib ? 1.f : 0.f);
+    const P dd = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+    const P ls = fma2(half_a2, dd, two_eps2);
+    const P ld = fma2(nhalf_a2, dd, two2);
+    const P pr = mul2(ls, ld);
+    const P rr = mul2(quarter_a2, pk<P>(rcp1(first(pr)), rcp1(second(pr))));
+    const P as = mul2(ld, rr), ad = mul2(ls, rr);
+    const P se = fma2(sz, ez, fma2(sy, ey, mul2(sx, ex)));
+    const P de = fma2(dz, ez, fma2(dy, ey, mul2(dx, ex)));
+    const P ee = fma2(ez, ez, fma2(ey, ey, mul2(ex, ex)));
+    const P cost = fma2(half2, ee, fma2(mul2(as, se), se, mul2(mul2(ad, de), de)));
+    const bool ia = va && (first(cost) <= A.c_max);
+    const bool ib = vb && (second(cost) <= A.c_max);
+    const P inl = pk<P>(ia ? 1.f : 0.f, ib ? 1.f : 0.f);
     S.lc = fma2(inl, cost, S.lc);
     S.cnt = add2(S.cnt, inl);
-    const float2 h = mul2(A.half2, inl), Pw = mul2(as, inl), Qw = mul2(ad, inl);
-    const float2 Psx = mul2(Pw, sx), Psy = mul2(Pw, sy), Psz = mul2(Pw, sz);
-    const float2 Qdx = mul2(Qw, dx), Qdy = mul2(Qw, dy), Qdz = mul2(Qw, dz);
-    const float2 Oxx = fma2(Psx, sx, fma2(Qdx, dx, h));
-    const float2 Oyy = fma2(Psy, sy, fma2(Qdy, dy, h));
-    const float2 Ozz = fma2(Psz, sz, fma2(Qdz, dz, h));
-    const float2 Oxy = fma2(Psx, sy, mul2(Qdx, dy));
-    const float2 Oxz = fma2(Psx, sz, mul2(Qdx, dz));
-    const float2 Oyz = fma2(Psy, sz, mul2(Qdy, dz));
-    const float2 gx = fma2(Oxz, ez, fma2(Oxy, ey, mul2(Oxx, ex)));
-    const float2 gy = fma2(Oyz, ez, fma2(Oyy, ey, mul2(Oxy, ex)));
-    const float2 gz = fma2(Ozz, ez, fma2(Oyz, ey, mul2(Oxz, ex)));
+    const P h = mul2(half2, inl), Pw = mul2(as, inl), Qw = mul2(ad, inl);
+    const P Psx = mul2(Pw, sx), Psy = mul2(Pw, sy), Psz = mul2(Pw, sz);
+    const P Qdx = mul2(Qw, dx), Qdy = mul2(Qw, dy), Qdz = mul2(Qw, dz);
+    const P Oxx = fma2(Psx, sx, fma2(Qdx, dx, h));
+    const P Oyy = fma2(Psy, sy, fma2(Qdy, dy, h));
+    const P Ozz = fma2(Psz, sz, fma2(Qdz, dz, h));
+    const P Oxy = fma2(Psx, sy, mul2(Qdx, dy));
+    const P Oxz = fma2(Psx, sz, mul2(Qdx, dz));
+    const P Oyz = fma2(Psy, sz, mul2(Qdy, dz));
+    const P gx = fma2(Oxz, ez, fma2(Oxy, ey, mul2(Oxx, ex)));
+    const P gy = fma2(Oyz, ez, fma2(Oyy, ey, mul2(Oxy, ex)));
+    const P gz = fma2(Ozz, ez, fma2(Oyz, ey, mul2(Oxz, ex)));
     // Pm = [q~]x Omega (nq = -q~ carries the minus signs)
-    const float2 P00 = fma2(qty, Oxz, mul2(nqz, Oxy)), P01 = fma2(qty, Oyz, mul2(nqz, Oyy)),
+    const P P00 = fma2(qty, Oxz, mul2(nqz, Oxy)), P01 = fma2(qty, Oyz, mul2(nqz, Oyy)),
                  P02 = fma2(qty, Ozz, mul2(nqz, Oyz));
-    const float2 P10 = fma2(qtz, Oxx, mul2(nqx, Oxz)), P11 = fma2(qtz, Oxy, mul2(nqx, Oyz)),
+    const P P10 = fma2(qtz, Oxx, mul2(nqx, Oxz)), P11 = fma2(qtz, Oxy, mul2(nqx, Oyz)),
                  P12 = fma2(qtz, Oxz, mul2(nqx, Ozz));
-    const float2 P20 = fma2(qtx, Oxy, mul2(nqy, Oxx)), P21 = fma2(qtx, Oyy, mul2(nqy, Oxy)),
+    const P P20 = fma2(qtx, Oxy, mul2(nqy, Oxx)), P21 = fma2(qtx, Oyy, mul2(nqy, Oxy)),
                  P22 = fma2(qtx, Oyz, mul2(nqy, Oxz));
     // H~_ww += Pm [q~]x^T ; H~_wv += Pm ; H~_vv += Omega
     S.Hww[0] = fma2(qty, P02, fma2(nqz, P01, S.Hww[0]));
@@ -334,6 +373,14 @@ __device__ __forceinline__ void lk_accumulate(const LkArgs& A, Lk2Acc& S, const 
     S.bw[1] = fma2(gz, qtx, fma2(gx, nqz, S.bw[1]));
     S.bw[2] = fma2(gx, qty, fma2(gy, nqx, S.bw[2]));
     S.nbv[0] = add2(S.nbv[0], gx); S.nbv[1] = add2(S.nbv[1], gy); S.nbv[2] = add2(S.nbv[2], gz);
+}
+
+__device__ __forceinline__ void lk_accumulate(const LkArgs& A, Lk2Acc& S, const LkPair<float2>& o, bool va, bool vb) {
+    lk_accumulate_f<float2>(A, S, o, va, vb);
+}
+__device__ __forceinline__ void lk_accumulate(const LkArgs& A, LkSums<float>& S, const LkPair<float, float>& o, bool va,
+                                              bool vb) {
+    lk_accumulate_f<float>(A, S, o, va, vb);
 }
 
 template <typename H2>
@@ -790,41 +837,54 @@ __device__ __forceinline__ void lk_store(const LkArgs& A, const float R[9], cons
     for (int f = 0; f < MP_GN; ++f) A.gn[(int64_t)f * A.stride + p] = out[f];
 }
 
-struct Lk2Look {
+// (P = float: particle a alone, and mb = -1)
+template <typename P>
+struct LkLook {
     int ma, mb;
-    float2 qx, qy, qz;
+    P qx, qy, qz;
 };
+using Lk2Look = LkLook<float2>;
 
-__device__ __forceinline__ Lk2Look lk2_lookup(const LkArgs& A, const float2 R[9], float2 tx, float2 ty, float2 tz,
-                                              const float4* Pp) {
+// A staged point of the particle (pair): q alone.
+template <typename P>
+__device__ __forceinline__ LkLook<P> lk2_point(const P R[9], P tx, P ty, P tz, const float4* Pp) {
     const float4 p0 = Pp[0], p1 = Pp[1];
-    const float2 mx = make_float2(p0.x, p0.y), my = make_float2(p0.z, p0.w), mz = make_float2(p1.x, p1.y);
-    Lk2Look L;
+    const P mx = pk<P>(p0.x, p0.y), my = pk<P>(p0.z, p0.w), mz = pk<P>(p1.x, p1.y);
+    LkLook<P> L;
     // decision sequence: q~ = fma(R_a2, mz, fma(R_a1, my, R_a0 mx)), q = q~ + t
     L.qx = add2(fma2(R[2], mz, fma2(R[1], my, mul2(R[0], mx))), tx);
     L.qy = add2(fma2(R[5], mz, fma2(R[4], my, mul2(R[3], mx))), ty);
     L.qz = add2(fma2(R[8], mz, fma2(R[7], my, mul2(R[6], mx))), tz);
+    return L;
+}
+
+// And its map indices.
+template <typename P>
+__device__ __forceinline__ LkLook<P> lk2_lookup(const LkArgs& A, const P R[9], P tx, P ty, P tz, const float4* Pp) {
+    constexpr bool PAIR = sizeof(P) == sizeof(float2);
+    LkLook<P> L = lk2_point<P>(R, tx, ty, tz, Pp);
     // voxel = floor(fma(q, 1/res, off)): round-down add of 1.5 * 2^23
-    const float2 fx = __fadd2_rd(fma2(L.qx, A.inv2, A.offx2), A.magic2);
-    const float2 fy = __fadd2_rd(fma2(L.qy, A.inv2, A.offy2), A.magic2);
-    const float2 fz = __fadd2_rd(fma2(L.qz, A.inv2, A.offz2), A.magic2);
+    const P fx = add2_rd(fma2(L.qx, pk<P>(A.inv2), pk<P>(A.offx2)), pk<P>(A.magic2));
+    const P fy = add2_rd(fma2(L.qy, pk<P>(A.inv2), pk<P>(A.offy2)), pk<P>(A.magic2));
+    const P fz = add2_rd(fma2(L.qz, pk<P>(A.inv2), pk<P>(A.offz2)), pk<P>(A.magic2));
     // unsigned arithmetic: an out-of-range voxel wraps to a large value
-    const unsigned vxa = __float_as_uint(fx.x) - 0x4B400000u, vxb = __float_as_uint(fx.y) - 0x4B400000u;
-    const unsigned vya = __float_as_uint(fy.x) - 0x4B400000u, vyb = __float_as_uint(fy.y) - 0x4B400000u;
-    const unsigned vza = __float_as_uint(fz.x) - 0x4B400000u, vzb = __float_as_uint(fz.y) - 0x4B400000u;
+    const unsigned vxa = __float_as_uint(first(fx)) - 0x4B400000u, vxb = __float_as_uint(second(fx)) - 0x4B400000u;
+    const unsigned vya = __float_as_uint(first(fy)) - 0x4B400000u, vyb = __float_as_uint(second(fy)) - 0x4B400000u;
+    const unsigned vza = __float_as_uint(first(fz)) - 0x4B400000u, vzb = __float_as_uint(second(fz)) - 0x4B400000u;
     const bool ina = vxa < (unsigned)A.nx && vya < (unsigned)A.ny && vza < (unsigned)A.nz;
     const bool inb = vxb < (unsigned)A.nx && vyb < (unsigned)A.ny && vzb < (unsigned)A.nz;
     L.ma = -1;
     L.mb = -1;
     if (ina) L.ma = __ldg(A.nnf + (((int)vza * A.ny + (int)vya) * A.nx + (int)vxa));
-    if (inb) L.mb = __ldg(A.nnf + (((int)vzb * A.ny + (int)vyb) * A.nx + (int)vxb));
+    if (PAIR && inb) L.mb = __ldg(A.nnf + (((int)vzb * A.ny + (int)vyb) * A.nx + (int)vxb));
     return L;
 }
 
-__device__ __forceinline__ Lk2Look lk2_none() {
-    Lk2Look L;
+template <typename P>
+__device__ __forceinline__ LkLook<P> lk2_none() {
+    LkLook<P> L;
     L.ma = L.mb = -1;
-    L.qx = L.qy = L.qz = make_float2(0.f, 0.f);
+    L.qx = L.qy = L.qz = pk<P>(0.f, 0.f);
     return L;
 }
 
@@ -837,37 +897,39 @@ __device__ __forceinline__ void lk2_record(const LkArgs& A, int mm, float4& r0, 
 
 // The pair's sums: its lever arm q~ = q - t, its geometry, and the shared
 // accumulation.
-template <typename V>
-__device__ __forceinline__ void lk2_accumulate(const LkArgs& A, Lk2Acc& S, const V R[9], float2 tx, float2 ty, float2 tz,
-                                               const V nn[3], const Lk2Look& L, const float4& ra0, const float2& ra1,
+template <typename V, typename P>
+__device__ __forceinline__ void lk2_accumulate(const LkArgs& A, LkSums<P>& S, const V R[9], P tx, P ty, P tz,
+                                               const V nn[3], const LkLook<P>& L, const float4& ra0, const float2& ra1,
                                                const float4& rb0, const float2& rb1) {
-    const float2 q[3] = {L.qx, L.qy, L.qz};
-    LkPair<V> o;
-    o.qt[0] = fma2(A.m1, tx, L.qx);
-    o.qt[1] = fma2(A.m1, ty, L.qy);
-    o.qt[2] = fma2(A.m1, tz, L.qz);
+    const P q[3] = {L.qx, L.qy, L.qz}, m1 = pk<P>(A.m1);
+    LkPair<V, P> o;
+    o.qt[0] = fma2(m1, tx, L.qx);
+    o.qt[1] = fma2(m1, ty, L.qy);
+    o.qt[2] = fma2(m1, tz, L.qz);
     lk_geometry(A, R, q, nn, LkRec{ra0, rb0, ra1, rb1}, o);
     lk_accumulate(A, S, o, L.ma >= 0, L.mb >= 0);
 }
 
 // The scan normal of a staged point (broadcast pairs).
-__device__ __forceinline__ void lk2_normal(const float4* P, float2 nn[3]) {
-    nn[0] = make_float2(P[1].z, P[1].w);
-    nn[1] = make_float2(P[2].x, P[2].y);
-    nn[2] = make_float2(P[2].z, P[2].w);
+template <typename P>
+__device__ __forceinline__ void lk2_normal(const float4* p, P nn[3]) {
+    nn[0] = pk<P>(p[1].z, p[1].w);
+    nn[1] = pk<P>(p[2].x, p[2].y);
+    nn[2] = pk<P>(p[2].z, p[2].w);
 }
 
 // One half (particle a: h = 0, b: h = 1) of the packed sums as scalar sums.
-__device__ __forceinline__ LkAcc lk2_half(const LkArgs& A, const Lk2Acc& S, int h, int nv) {
+template <typename P>
+__device__ __forceinline__ LkAcc lk2_half(const LkArgs& A, const LkSums<P>& S, int h, int nv) {
     LkAcc o;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) { o.Hww[k] = h ? S.Hww[k].y : S.Hww[k].x; o.Hvv[k] = h ? S.Hvv[k].y : S.Hvv[k].x; }
+    for (int k = 0; k < 6; ++k) { o.Hww[k] = h ? second(S.Hww[k]) : first(S.Hww[k]); o.Hvv[k] = h ? second(S.Hvv[k]) : first(S.Hvv[k]); }
 #pragma unroll
-    for (int k = 0; k < 9; ++k) o.Hwv[k] = h ? S.Hwv[k].y : S.Hwv[k].x;
+    for (int k = 0; k < 9; ++k) o.Hwv[k] = h ? second(S.Hwv[k]) : first(S.Hwv[k]);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) { o.bw[k] = h ? S.bw[k].y : S.bw[k].x; o.bv[k] = -(h ? S.nbv[k].y : S.nbv[k].x); }
-    const float lc = h ? S.lc.y : S.lc.x;
-    const float cnt = h ? S.cnt.y : S.cnt.x;
+    for (int k = 0; k < 3; ++k) { o.bw[k] = h ? second(S.bw[k]) : first(S.bw[k]); o.bv[k] = -(h ? second(S.nbv[k]) : first(S.nbv[k])); }
+    const float lc = h ? second(S.lc) : first(S.lc);
+    const float cnt = h ? second(S.cnt) : first(S.cnt);
     // log p = -(sum of inlier costs) - c_max * (points that are not inliers)
     o.ll = fmaf(-A.c_max, (float)(nv - (int)cnt), -lc);
     o.cnt = (int)cnt;
@@ -881,22 +943,71 @@ struct LkPmStage {
     uint64_t bar[2];
 };
 
+// One particle's sums over the m points of a staged chunk. With few warps a
+// scheduler nothing hides a gather but the thread's own work, so the gathers run
+// in groups of four points: while a group is accumulated, the records of the next
+// and the NNF entries of the one after are in flight.
+__device__ __forceinline__ void lk_pm1_chunk(const LkArgs& A, LkSums<float>& S, const float R[9], float tx, float ty, float tz,
+                                             const float4* pts, int m) {
+    constexpr int G = 4;   // (8: 198 registers, 2218 against 1926 us at 1024 particles x 8192 points)
+    struct Group {
+        float4 r0[G];
+        float2 r1[G];
+        bool hit[G];
+    } u, v;
+    int mm[G];
+    auto look = [&](int k0) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) mm[g] = k0 + g < m ? lk2_lookup<float>(A, R, tx, ty, tz, pts + 3 * (k0 + g)).ma : -1;
+    };
+    auto records = [&](Group& r) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            r.hit[g] = mm[g] >= 0;
+            lk2_record(A, mm[g], r.r0[g], r.r1[g]);
+        }
+    };
+    auto accumulate = [&](const Group& r, int k0) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            if (k0 + g >= m) break;
+            LkLook<float> L = lk2_point<float>(R, tx, ty, tz, pts + 3 * (k0 + g));
+            L.ma = r.hit[g] ? 0 : -1;
+            float nn[3];
+            lk2_normal<float>(pts + 3 * (k0 + g), nn);
+            lk2_accumulate(A, S, R, tx, ty, tz, nn, L, r.r0[g], r.r1[g], r.r0[g], r.r1[g]);
+        }
+    };
+    look(0);
+    records(u);
+    look(G);
+    for (int k0 = 0; k0 < m; k0 += 2 * G) {
+        records(v);
+        look(k0 + 2 * G);
+        accumulate(u, k0);
+        records(u);
+        look(k0 + 3 * G);
+        accumulate(v, k0 + G);
+    }
+}
+
 // The sums of particle block bxi over chunks [c0, c1) of the scan, whose
 // sequence numbers start at q; returns false when a wait gave up. PART: the
 // block's sums so far are read from (c0 > 0) and left in (c1 < all) its columns
 // of the Gauss-Newton sums, in FP32 as they are.
-template <bool PART>
+template <bool PART, typename P>
 __device__ __forceinline__ bool lk_pm_block(const LkArgs& A, LkPmStage& st, int64_t bxi, int nv, int c0, int c1, int q) {
     // particles a and b of this thread sit PM_THREADS apart in sorted order,
     // so each half of a warp covers 32 consecutive sorted particles
-    const int64_t pa = (int64_t)bxi * PM_PER_CTA + threadIdx.x;
+    constexpr bool PAIR = sizeof(P) == sizeof(float2);
+    const int64_t pa = (int64_t)bxi * (PAIR ? PM_PER_CTA : PM_THREADS) + threadIdx.x;
     const int64_t pb = pa + PM_THREADS;
-    const bool acta = pa < A.n, actb = pb < A.n;
+    const bool acta = pa < A.n, actb = PAIR && pb < A.n;
     int64_t ia = acta ? A.order[pa] : 0, ib = actb ? A.order[pb] : 0;
     if (!MP_DCHECK(ia >= 0 && ia < A.n, "particle order entry", ia)) ia = 0;
     if (!MP_DCHECK(ib >= 0 && ib < A.n, "particle order entry", ib)) ib = 0;
-    float2 R[9];
-    float2 tx, ty, tz;
+    P R[9];
+    P tx, ty, tz;
     {
         Quat qa, qb;
         float ta[3], tb[3], Ra[9], Rb[9];
@@ -905,10 +1016,10 @@ __device__ __forceinline__ bool lk_pm_block(const LkArgs& A, LkPmStage& st, int6
         quat_rot_exact(qa, Ra);
         quat_rot_exact(qb, Rb);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) R[k] = make_float2(Ra[k], Rb[k]);
-        tx = make_float2(ta[0], tb[0]);
-        ty = make_float2(ta[1], tb[1]);
-        tz = make_float2(ta[2], tb[2]);
+        for (int k = 0; k < 9; ++k) R[k] = pk<P>(Ra[k], Rb[k]);
+        tx = pk<P>(ta[0], tb[0]);
+        ty = pk<P>(ta[1], tb[1]);
+        tz = pk<P>(ta[2], tb[2]);
     }
 
     const int nchunks = (nv + PM_CHUNK - 1) / PM_CHUNK;
@@ -928,18 +1039,16 @@ __device__ __forceinline__ bool lk_pm_block(const LkArgs& A, LkPmStage& st, int6
         if (c0 + 1 < c1) issue(c0 + 1);
     }
 
-    Lk2Acc S;
-    float2* const sum = reinterpret_cast<float2*>(&S);   // LK_SUMS pairs
-    constexpr int LK_SUMS = sizeof(Lk2Acc) / sizeof(float2);
+    LkSums<P> S;
+    P* const sum = reinterpret_cast<P*>(&S);   // LK_SUMS of them
+    constexpr int LK_SUMS = sizeof(S) / sizeof(P);
     static_assert(LK_SUMS == MP_GN, "one column of the Gauss-Newton sums each");
 #pragma unroll
     for (int k = 0; k < LK_SUMS; ++k) {
-        sum[k] = make_float2(0.f, 0.f);
-        if (PART && c0 > 0) {
-            // (through L2: another SM may have stored them in this launch)
-            if (acta) sum[k].x = __ldcg(A.gn + (int64_t)k * A.stride + pa);
-            if (actb) sum[k].y = __ldcg(A.gn + (int64_t)k * A.stride + pb);
-        }
+        sum[k] = pk<P>(0.f, 0.f);
+        if (PART && c0 > 0)   // (through L2: another SM may have stored them in this launch)
+            sum[k] = pk<P>(acta ? __ldcg(A.gn + (int64_t)k * A.stride + pa) : 0.f,
+                           actb ? __ldcg(A.gn + (int64_t)k * A.stride + pb) : 0.f);
     }
 
     const bool active = acta;   // acta is false only if actb is false too
@@ -951,27 +1060,29 @@ __device__ __forceinline__ bool lk_pm_block(const LkArgs& A, LkPmStage& st, int6
         bool got = mbar_wait_bounded(&st.bar[b], parity, A.budget);
         if (__syncthreads_or(!got)) { failed = true; break; }
         const int m = min(PM_CHUNK, nv - c * PM_CHUNK);
-        if (active) {
-            const float4* P = st.buf[b];
+        if constexpr (!PAIR) {
+            if (active) lk_pm1_chunk(A, S, R, tx, ty, tz, st.buf[b], m);
+        } else if (active) {
+            const float4* pts = st.buf[b];
             // software pipeline over the two dependent gathers: every
             // iteration issues the NNF loads of point k+2 and the record loads
             // of point k+1 before the arithmetic of point k. Invariant at the
             // loop head: sc = point k (records loaded), sb = point k+1 (map
             // indices loaded).
-            Lk2Look sb = lk2_none(), sc = lk2_lookup(A, R, tx, ty, tz, P);
+            LkLook<P> sb = lk2_none<P>(), sc = lk2_lookup<P>(A, R, tx, ty, tz, pts);
             float4 ra0, rb0;
             float2 ra1, rb1;
             lk2_record(A, sc.ma, ra0, ra1);
             lk2_record(A, sc.mb, rb0, rb1);
-            if (m > 1) sb = lk2_lookup(A, R, tx, ty, tz, P + 3);
+            if (m > 1) sb = lk2_lookup<P>(A, R, tx, ty, tz, pts + 3);
             for (int k = 0; k < m; ++k) {
-                const Lk2Look nb = (k + 2 < m) ? lk2_lookup(A, R, tx, ty, tz, P + 3 * (k + 2)) : lk2_none();
+                const LkLook<P> nb = (k + 2 < m) ? lk2_lookup<P>(A, R, tx, ty, tz, pts + 3 * (k + 2)) : lk2_none<P>();
                 float4 na0, nb0;
                 float2 na1, nb1;
                 lk2_record(A, sb.ma, na0, na1);
                 lk2_record(A, sb.mb, nb0, nb1);
-                float2 nn[3];
-                lk2_normal(P + 3 * k, nn);
+                P nn[3];
+                lk2_normal<P>(pts + 3 * k, nn);
                 lk2_accumulate(A, S, R, tx, ty, tz, nn, sc, ra0, ra1, rb0, rb1);
                 sc = sb;
                 sb = nb;
@@ -992,20 +1103,20 @@ __device__ __forceinline__ bool lk_pm_block(const LkArgs& A, LkPmStage& st, int6
     if (PART && c1 < nchunks) {
 #pragma unroll
         for (int k = 0; k < LK_SUMS; ++k) {
-            if (acta) A.gn[(int64_t)k * A.stride + pa] = sum[k].x;
-            if (actb) A.gn[(int64_t)k * A.stride + pb] = sum[k].y;
+            if (acta) A.gn[(int64_t)k * A.stride + pa] = first(sum[k]);
+            if (actb) A.gn[(int64_t)k * A.stride + pb] = second(sum[k]);
         }
         return true;
     }
     float Rs[9];
     if (acta) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Rs[k] = R[k].x;
+        for (int k = 0; k < 9; ++k) Rs[k] = first(R[k]);
         lk_store(A, Rs, lk2_half(A, S, 0, nv), pa);
     }
     if (actb) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) Rs[k] = R[k].y;
+        for (int k = 0; k < 9; ++k) Rs[k] = second(R[k]);
         lk_store(A, Rs, lk2_half(A, S, 1, nv), pb);
     }
     return true;
@@ -1031,12 +1142,24 @@ struct LkPmOp {
     static __device__ __forceinline__ void run(const LkArgs& A, unsigned bxi, unsigned) {
         __shared__ __align__(128) LkPmStage st;
         const int nv = lk_pm_begin(A, st, bxi);
-        lk_pm_block<false>(A, st, bxi, nv, 0, (nv + PM_CHUNK - 1) / PM_CHUNK, 0);
+        lk_pm_block<false, float2>(A, st, bxi, nv, 0, (nv + PM_CHUNK - 1) / PM_CHUNK, 0);
     }
 };
 
 __global__ void __launch_bounds__(PM_THREADS, PM_MINB) k_likelihood_pm(const LkArgs A) {
     LkPmOp::run(A, blockIdx.x, 0);
+}
+
+// One particle a thread, for fewer particles than pairs of them would keep the
+// SMs' schedulers busy with: twice the warps, and gathers four points deep where
+// a lone warp waited 1200 cycles a point (outdoors, likelihood stage, packed ->
+// now: 1024 particles x 8192 points 6.2 -> 1.9 ms, 8192 5.7 -> 1.9, 32768 5.5 ->
+// 2.6, 65536 6.2 -> 5.0, 98304 7.2 -> 6.7; 131072 8.15 and 8.19; 50021 x 4999 3.59
+// -> 2.07). The sums are the packed form's, bit for bit.
+__global__ void __launch_bounds__(PM_THREADS, PM1_MINB) k_likelihood_pm1(const LkArgs A) {
+    __shared__ __align__(128) LkPmStage st;
+    const int nv = lk_pm_begin(A, st, blockIdx.x);
+    lk_pm_block<false, float>(A, st, blockIdx.x, nv, 0, (nv + PM_CHUNK - 1) / PM_CHUNK, 0);
 }
 
 // The same over parts of the scan: item t of A.items x blocks is part t /
@@ -1080,7 +1203,7 @@ __global__ void __launch_bounds__(PM_THREADS, PM_MINB) k_likelihood_pm_parts(con
         if (t >= parts * blocks) return;
         const int part = t / blocks, blk = t - part * blocks;
         const int c0 = part * len, c1 = min(nchunks, c0 + len);
-        if (!lk_pm_block<true>(A, st, blk, nv, c0, c1, q)) return;
+        if (!lk_pm_block<true, float2>(A, st, blk, nv, c0, c1, q)) return;
         q += c1 - c0;
         __threadfence();      // the stored sums before the count
         __syncthreads();
@@ -1201,14 +1324,14 @@ __global__ void __launch_bounds__(PM_THREADS, MINB) k_likelihood_pm_h(const LkAr
         if (acta) {
             const uint4* P = buf[b];
             // the same two-gather software pipeline as the FP32 form
-            Lk2Look sb = lk2_none(), sc = lkh_lookup<H2>(A, R, tx, ty, tz, P);
+            Lk2Look sb = lk2_none<float2>(), sc = lkh_lookup<H2>(A, R, tx, ty, tz, P);
             float4 ra0, rb0;
             float2 ra1, rb1;
             lk2_record(A, sc.ma, ra0, ra1);
             lk2_record(A, sc.mb, rb0, rb1);
             if (m > 1) sb = lkh_lookup<H2>(A, R, tx, ty, tz, P + 2);
             for (int k = 0; k < m; ++k) {
-                const Lk2Look nb = (k + 2 < m) ? lkh_lookup<H2>(A, R, tx, ty, tz, P + 2 * (k + 2)) : lk2_none();
+                const Lk2Look nb = (k + 2 < m) ? lkh_lookup<H2>(A, R, tx, ty, tz, P + 2 * (k + 2)) : lk2_none<float2>();
                 float4 na0, nb0;
                 float2 na1, nb1;
                 lk2_record(A, sb.ma, na0, na1);
@@ -1276,7 +1399,16 @@ int lk_segments(int n_scan, LkArgs& A) {
     return segs;
 }
 
-// Whether a launch takes the particle-major form: from 80k particles on, which
+// A map of more than LK_WIDE voxels across. Its sums keep one order, the scan's,
+// in every form: a lever arm of hundreds of voxels turns the last bits of a
+// particle's step into other voxels for some of its points in the next, and with
+// the particles close around the sensor the log posterior of two orders differed
+// by 0.04 of its norm after a second step (box rooms of 100 voxels: 1e-6).
+bool lk_wide(const mp_ctx* c) {
+    return std::max(c->nnf_dims[0], std::max(c->nnf_dims[1], c->nnf_dims[2])) > LK_WIDE;
+}
+
+// Whether a launch takes the particle-major form: on wide maps, and from 80k particles on, which
 // are 320 of the 456 CTAs the GPU holds. Measured, box room x 1024 points,
 // particle-major / point-major: 32k particles 326 / 252 us, 64k 491 / 487, 96k
 // 670 / 730, 128k 818 / 953, 256k 1511 / 1815, and 512k x 512 1405 / 2007 (the
@@ -1288,7 +1420,7 @@ int lk_segments(int n_scan, LkArgs& A) {
 // / 577 us, 128k 1041 / 1142. The particle-major sums are added in scan order,
 // point by point, whatever the launch. A scan split is the point-major form's.
 bool lk_particle_major(const mp_ctx* c, int split) {
-    return split == 1 && c->n >= LK_PM_MIN;
+    return split == 1 && (c->n >= LK_PM_MIN || lk_wide(c));
 }
 
 LkArgs lk_args(mp_ctx* c) {
@@ -1374,7 +1506,9 @@ int mp_launch_likelihood(mp_ctx* c) {
     if (!pm) return launch_point_major<float2>(c, A);
     const int64_t blocks = (c->n + PM_PER_CTA - 1) / PM_PER_CTA;
     const int64_t slots = 152 * PM_MINB;
-    if (blocks <= slots || c->n_scan <= PM_CHUNK) {
+    if (lk_wide(c) && c->n <= LK_PM1_MAX) {
+        k_likelihood_pm1<<<grid_for(c->n, PM_THREADS), PM_THREADS, 0, c->stream>>>(A);
+    } else if (blocks <= slots || c->n_scan <= PM_CHUNK) {
         k_likelihood_pm<<<(unsigned)blocks, PM_THREADS, 0, c->stream>>>(A);
     } else {
         MP_CUDA(c, cudaMemsetAsync(c->lk_ticket, 0, sizeof(int) * (size_t)(blocks + 1), c->stream));

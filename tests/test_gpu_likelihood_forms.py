@@ -76,3 +76,39 @@ def test_particle_major_equals_point_major(room, precision, n, m):
     assert np.all(np.abs(pm[:1500] - pt) <= 2e-5 * (np.abs(pt).max(axis=0, keepdims=True) + 1e-6))
     assert np.array_equal(pm[:8192], pm[8192:16384])        # the same poses in other slots, to the last particle
     assert np.array_equal(pm[n - 1], pm[(n - 1) % 8192])
+
+
+@pytest.fixture(scope="module")
+def wide(room, oracle):
+    """The room on a map of more than 512 voxels across (two far patches)."""
+    y, z = np.meshgrid(0.1 * np.arange(5), 0.1 * np.arange(5))
+    far = [np.c_[np.full(25, x), y.ravel(), z.ravel()] for x in (-30.0, 30.0)]
+    pts = np.concatenate([room["w"].map_points, *far]).astype(np.float32)
+    return dict(room, w=type("W", (), dict(map_points=pts, particles=room["w"].particles)),
+                om=oracle.OracleMap(pts, room["P"]))
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 1025])
+@pytest.mark.parametrize("m", [40, 41, 127, 128, 129, 133, 700])
+def test_wide_map_one_particle_a_thread(wide, oracle, n, m):
+    # the densest part of the scan: m points are m staged points, in groups of four and chunks of 128
+    order = np.argsort(np.linalg.norm(wide["scan"], axis=1), kind="stable")
+    sc = np.ascontiguousarray(wide["scan"][order][:m])
+    gn, valid = sums(wide, wide["w"].particles[:n], sc)
+    P = wide["P"]
+    sn, sv, _, _ = oracle.point_normals(sc, P.r_cov, P.cov_k, P.cov_min)
+    assert np.array_equal(valid.astype(bool), sv.astype(bool))
+    ref = oracle.likelihood(wide["om"], wide["w"].particles[:n], sc, sn, sv, P, amb_tol=1e-4)
+    msg = check_sums(gn, ref)
+    assert not msg, msg
+
+
+def test_wide_map_sums_keep_their_bits(wide):
+    """One particle a thread (up to 114688), pairs, and parts of the scan: the
+    same sums, bit for bit."""
+    poses = np.tile(wide["w"].particles, (16, 1))
+    sc = np.ascontiguousarray(wide["scan"][:700])
+    one, _ = sums(wide, poses[:8192], sc)
+    for n in (114688, 114689, 131072):
+        many, _ = sums(wide, poses[:n], sc)
+        assert np.array_equal(many[:8192], one) and np.array_equal(many[n - 1], one[(n - 1) % 8192])
