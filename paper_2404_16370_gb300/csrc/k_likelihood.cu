@@ -29,7 +29,9 @@
 //    stage sorts them) read neighbouring NNF lines.
 //  * particle-major (k_likelihood_pm): a thread takes two particles and walks
 //    the scan, which it reads by broadcast. Fewer instructions a pair, but it
-//    needs 152 SMs x 768 particles to fill the GPU, and a full last wave.
+//    needs 152 SMs x 768 particles to fill the GPU, and a full last wave. With
+//    fewer on a wide map a thread takes one (k_likelihood_pm1), unpacked, to the
+//    same bits.
 //
 // lk_particle_major() chooses. What bounds both is the same: a gather of 32
 // different lines that miss L1 takes 32 cycles of its SM (one line a cycle,
@@ -42,9 +44,8 @@
 // particle-major before -> now: 256 x 128 points 29 -> 8.2 us, 4096 x 512 147
 // -> 26.7 us, 10000 x 2048 688 -> 178 us, 16000 x 1021 in BF16 593 -> 147 us,
 // 50021 x 4999 (outdoor, one particle a thread) 3.53 -> 2.07 ms; particle-major in
-// parts, 2^17 x 512
-// 426 -> 392 us, 2^17 x 8192 10.4 -> 8.2 ms, 2^18 x 8192 around the sensor 17.7
-// -> 16.7 ms, 2^20 x 8192 52.8 -> 52.4 ms.
+// parts, 2^17 x 512 426 -> 392 us, 2^17 x 8192 10.4 -> 8.2 ms, 2^18 x 8192 around
+// the sensor 17.7 -> 16.7 ms, 2^20 x 8192 52.8 -> 52.4 ms.
 #include "mp_internal.cuh"
 
 #include <cuda_bf16.h>
