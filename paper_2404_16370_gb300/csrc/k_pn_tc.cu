@@ -170,9 +170,6 @@ __device__ __forceinline__ bool group_sync_or(int group, bool v) {
         : "memory");
     return r != 0;
 }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // the value at p, an address of this CTA's shared memory, in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t ld_cluster(const void* p, uint32_t rank) {
     uint32_t a, v;

@@ -439,6 +439,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Barrier of the cluster's threads, with their writes made visible to each other.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Grid-wide barrier of a cooperative (persistent) launch, whose CTAs are all
 // resident at once. Thread 0 of each CTA arrives on a counter that only grows
 // and spins until it reaches this barrier's target, the arrivals of all
@@ -719,6 +724,21 @@ cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned block, size_t 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// One cluster of `ctas` CTAs.
+inline cudaError_t launch_cluster(const void* func, unsigned ctas, unsigned block, void* arg, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    void* args[1] = {arg};
+    return cudaLaunchKernelExC(&cfg, func, args);
 }
 inline cudaError_t launch_coop(const void* func, unsigned grid, unsigned block, void* arg, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};

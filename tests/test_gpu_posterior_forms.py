@@ -9,7 +9,7 @@ from paper_2404_16370_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,K,iters", [(1, 4, 3), (256, 16, 10), (257, 5, 0), (3001, 17, 9), (38000, 32, 2),
+@pytest.mark.parametrize("n,K,iters", [(1, 4, 3), (128, 16, 10), (129, 32, 3), (256, 16, 10), (257, 5, 0), (700, 16, 9), (1024, 32, 10), (1025, 16, 2), (3001, 17, 9), (38000, 32, 2),
                                        (40001, 32, 3), (79001, 16, 3), (300, 16, 10), (19456, 32, 3), (19457, 16, 3)])
 def test_posterior_forms(oracle, n, K, iters):
     from paper_2404_16370_gb300 import mp
