@@ -170,7 +170,6 @@ struct HeadArgs {
 struct HeadSmem {
     __align__(16) float As[HM][HK + 4];
     __align__(16) float Bs[HK][HN + 4];
-    float cs[4][HN];
 };
 
 // PDL: op(B) is a weight matrix, which the kernels just before do not write: its
@@ -185,7 +184,6 @@ __device__ __forceinline__ void head_tile(const HeadArgs& H, HeadSmem& S, int bx
     const int M = H.M, N = H.N, K = H.K, lda = H.lda, ldb = H.ldb, ldc = H.ldc;
     auto& As = S.As;
     auto& Bs = S.Bs;
-    auto& cs = S.cs;
     const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
     const int m0 = by * HM, n0 = bx * HN;
     float acc[4] = {0.f, 0.f, 0.f, 0.f}, col = 0.f;
@@ -264,14 +262,12 @@ __device__ __forceinline__ void head_tile(const HeadArgs& H, HeadSmem& S, int bx
                 acc[3] = fmaf(av[q], b.w, acc[3]);
             }
         }
-        if ((EPI & HEAD_COLSUM) && m0 == 0)
-            for (int k = tid / HN * (HK / 4); k < (tid / HN + 1) * (HK / 4); ++k) col += Bs[k][tid % HN];
+        if ((EPI & HEAD_COLSUM) && m0 == 0 && tid < HN) {   // (one chain over k too)
+#pragma unroll 16
+            for (int k = 0; k < HK; ++k) col += Bs[k][tid];
+        }
     }
-    if ((EPI & HEAD_COLSUM) && m0 == 0) {
-        cs[tid / HN][tid % HN] = col;
-        __syncthreads();
-        if (tid < HN && n0 + tid < N) colsum[n0 + tid] = cs[0][tid] + cs[1][tid] + cs[2][tid] + cs[3][tid];
-    }
+    if ((EPI & HEAD_COLSUM) && m0 == 0 && tid < HN && n0 + tid < N) colsum[n0 + tid] = col;
     const int m = m0 + ty, n = n0 + tx * 4;
     if (m >= M || n >= N) return;
     if (EPI & HEAD_BIAS) {
@@ -532,10 +528,18 @@ __global__ void __launch_bounds__(64) k_mdn_loss(const float* __restrict__ o, co
         for (int k = 16; k > 0; k >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, k));
         return v;
     };
+    // the components' sum in their order: the same bits as one thread's, and the same
+    // Adam step where a gradient is nearly zero
+    auto ordered_sum = [](float v) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < NCOMP; ++k) s += __shfl_sync(0xffffffffu, v, k);
+        return s;
+    };
     // log pi = a - logsumexp(a)
     const float a = ob[c];
     const float amax = warp_max(a);
-    const float lse_a = amax + logf(warp_sum(expf(a - amax)));
+    const float lse_a = amax + logf(ordered_sum(expf(a - amax)));
     const float half_log_2pi6 = 3.f * 1.8378770664093453f;
     float th[6], dl[6], s = 0.f;
 #pragma unroll
@@ -549,7 +553,7 @@ __global__ void __launch_bounds__(64) k_mdn_loss(const float* __restrict__ o, co
     }
     const float lj = a - lse_a + s - half_log_2pi6;
     const float jmax = warp_max(lj);
-    const float L = -(jmax + logf(warp_sum(expf(lj - jmax))));
+    const float L = -(jmax + logf(ordered_sum(expf(lj - jmax))));
     if (c == 0) atomicAdd(loss, L / B);
     const float invB = 1.f / B;
     const float r = expf(lj + L);               // responsibility
