@@ -3,7 +3,8 @@
 // (target), and Sigma^DeltaT from the Gauss-Newton Hessian at the result.
 //
 // One cooperative kernel runs all iterations on the sorted points of both scans
-// (those without a normal at 1e18 m: out of reach as targets, skipped as sources). For the current estimate T = (R, t) (FP64, in shared memory):
+// (those without a normal at 1e18 m: out of reach as targets, skipped as sources).
+// For the current estimate T = (R, t) (FP64, in shared memory):
 //  * decisions in FP32 on T's rounding to float (R from the unit quaternion,
 //    q = R mu + t by the fixed sequence, squared distances un-fused); the
 //    correspondence is the target point of smallest squared distance, ties to
