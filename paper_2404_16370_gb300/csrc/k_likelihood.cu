@@ -1474,7 +1474,7 @@ int launch_point_major(mp_ctx* c, LkArgs A) {
     // zeroed output
     if (A.split > 1) MP_CUDA(c, cudaMemsetAsync(c->gn, 0, sizeof(float) * MP_GN * (size_t)c->cap, c->stream));
     const dim3 grid((unsigned)lk_blocks(A), (unsigned)A.split);
-    const int segs = lk_segments(c->n_scan, A);
+    const int segs = lk_segments(c->n_prep, A);
     for (A.seg = 0; A.seg < segs; ++A.seg) {
         MP_CUDA(c, launch_next(A.wpp > 1 ? k_likelihood<LK_WARPS, V> : k_likelihood<1, V>, grid, LK_THREADS, 0, c->stream, A));
         MP_LAUNCHED(c);
@@ -1484,8 +1484,8 @@ int launch_point_major(mp_ctx* c, LkArgs A) {
 
 template <typename H2>
 int launch_particle_major_16(mp_ctx* c, const LkArgs& A) {
-    if (c->n_scan > 0) {
-        k_scan_to_h2<H2><<<grid_for(c->n_scan, 256), 256, 0, c->stream>>>(c->scan_pair, c->scan_nvalid, c->n_scan,
+    if (c->n_prep > 0) {
+        k_scan_to_h2<H2><<<grid_for(c->n_prep, 256), 256, 0, c->stream>>>(c->scan_pair, c->scan_nvalid, c->n_prep,
                                                                           c->scan_h2);
         MP_LAUNCHED(c);
     }
@@ -1509,7 +1509,7 @@ int mp_launch_likelihood(mp_ctx* c) {
     const int64_t slots = 152 * PM_MINB;
     if (lk_wide(c) && c->n <= LK_PM1_MAX) {
         k_likelihood_pm1<<<grid_for(c->n, PM_THREADS), PM_THREADS, 0, c->stream>>>(A);
-    } else if (blocks <= slots || c->n_scan <= PM_CHUNK) {
+    } else if (blocks <= slots || c->n_prep <= PM_CHUNK) {
         k_likelihood_pm<<<(unsigned)blocks, PM_THREADS, 0, c->stream>>>(A);
     } else {
         MP_CUDA(c, cudaMemsetAsync(c->lk_ticket, 0, sizeof(int) * (size_t)(blocks + 1), c->stream));

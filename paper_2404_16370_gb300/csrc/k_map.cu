@@ -884,7 +884,7 @@ ScanArgs scan_args(mp_ctx* c, const float* raw, int n) {
 // Per-step scan Gaussians (brute-force radius kNN in shared-memory tiles) and
 // the valid points, sorted and in input order.
 int mp_launch_scan_prepare(mp_ctx* c, cudaStream_t s) {
-    int n = c->n_scan;
+    const int n = c->n_prep = c->n_scan;
     if (n == 0) {
         MP_CUDA(c, cudaMemsetAsync(c->scan_nvalid, 0, sizeof(int32_t), s));
         return MP_OK;

@@ -351,7 +351,7 @@ int mp_batch_step(mp_batch* b, const float* const* scans, const double* odom_T, 
         mp_ctx* c = b->G.ctx[i];
         // later calls on the instance (mp_get_posterior, mp_step) wait for the graph
         B_CUDA(cudaStreamWaitEvent(c->stream, b->done[p], 0));
-        c->n_scan = b->G.n_scan[i];
+        c->n_scan = c->n_prep = b->G.n_scan[i];
         c->nbr_cur ^= 1;
         c->step++;
     }

@@ -112,6 +112,7 @@ struct mp_ctx {
 
     // scan
     int32_t n_scan;
+    int32_t n_prep;         // points of the scan the scan stage prepared last (scan_nvalid counts the valid ones)
     float* scan_raw;        // max_scan x 3
     float* scan_normals;    // max_scan x 3
     uint8_t* scan_valid;    // max_scan

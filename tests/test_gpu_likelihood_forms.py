@@ -78,6 +78,27 @@ def test_particle_major_equals_point_major(room, precision, n, m):
     assert np.array_equal(pm[n - 1], pm[(n - 1) % 8192])
 
 
+@pytest.mark.parametrize("n,precision", [(600, 0), (1500, 0), (1500, 1), (82001, 0), (82001, 1)])
+def test_likelihood_reads_the_prepared_scan(room, n, precision):
+    """A scan that is set but not prepared changes no sums: the likelihood
+    reads the one the scan stage prepared last, all of it, though the new one
+    is shorter."""
+    from paper_2404_16370_gb300 import mp
+    poses = np.tile(room["w"].particles, (11, 1))[:n]
+    ctx = mp.mp_init_map(room["w"].map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n))
+    try:
+        mp.mp_set_precision(ctx, precision)
+        mp.mp_init_particles(ctx, n, poses=poses)
+        mp.mp_set_scan(ctx, room["scan"])
+        mp.mp_run_stages(ctx, mp.MP_STAGE_SCAN | mp.MP_STAGE_LIKELIHOOD)
+        want = mp.mp_get_buffer(ctx, mp.MP_BUF_GN)
+        mp.mp_set_scan(ctx, room["scan"][:20])
+        mp.mp_run_stages(ctx, mp.MP_STAGE_LIKELIHOOD)
+        np.testing.assert_array_equal(mp.mp_get_buffer(ctx, mp.MP_BUF_GN), want)
+    finally:
+        mp.mp_destroy(ctx)
+
+
 @pytest.fixture(scope="module")
 def wide(room, oracle):
     """The room on a map of more than 512 voxels across (two far patches)."""
