@@ -573,12 +573,13 @@ __device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned b
     }
     if (bx == 0) {
         if (threadIdx.x == 0) *args.nvalid = (int32_t)all;
-        // the last chunk's unused slots hold a point 1e18 m away, which no pose
-        // brings into a grid: the likelihood looks up whole chunks
+        // the last chunk's unused slots hold NaN, which no pose brings into a
+        // grid (a far point would do for unit quaternions only: others can map
+        // it to 0): the likelihood looks up whole chunks
         static_assert(MP_SCAN_CHUNK == SCAN_CTA, "one thread per slot of a chunk");
         const int64_t slot = (int64_t)(all / MP_SCAN_CHUNK) * MP_SCAN_CHUNK + threadIdx.x;
         if (slot >= all && all % MP_SCAN_CHUNK != 0)
-            for (int k = 0; k < 6; ++k) args.soa[scan_word(slot, k)] = 1e18f;
+            for (int k = 0; k < 6; ++k) args.soa[scan_word(slot, k)] = __uint_as_float(0x7fffffffu);
     }
     if (part != 0 || key == NONE) return;
     int64_t o = before, oe = earlier;

@@ -99,6 +99,25 @@ def test_likelihood_reads_the_prepared_scan(room, n, precision):
         mp.mp_destroy(ctx)
 
 
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("m", [1, 129])
+def test_unused_slots_count_for_no_pose(room, precision, m):
+    """The staged chunk's slots beyond the valid points stay outside the grid
+    also for a stored quaternion that is not a unit one: (0.5, -0.5, 0, 0) maps
+    (1, 1, 1) to 0, so the slot would land on the particle itself."""
+    poses = np.zeros((82001, 7), np.float32)
+    poses[:, :2] = 0.5, -0.5
+    poses[:, 4:] = np.resize(room["w"].map_points, (82001, 3))
+    order = np.argsort(np.linalg.norm(room["scan"], axis=1), kind="stable")
+    sc = np.ascontiguousarray(room["scan"][order][:m])
+    pm, valid = sums(room, poses, sc, precision)                # particle-major: the valid points alone
+    for n in (600, 1500):
+        pt, _ = sums(room, poses[:n], sc, precision)
+        assert np.array_equal(pm[:n, 28], pt[:, 28]) and pt[:, 28].max() <= valid.sum()
+        # roundings of FP32 (6e-8) over 129 points, with the cancellation between terms
+        assert np.all(np.abs(pm[:n] - pt) <= 2e-5 * (np.abs(pt).max(axis=0, keepdims=True) + 1e-6))
+
+
 @pytest.fixture(scope="module")
 def wide(room, oracle):
     """The room on a map of more than 512 voxels across (two far patches)."""
