@@ -4,6 +4,8 @@
 // buffer access for tests and state import/export.
 #include "mp_internal.cuh"
 
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
@@ -329,28 +331,66 @@ void chol6(const double S[36], double L[6][6]) {
     }
 }
 
-// p where a kernel on the context's device can use it as an array of T, else
-// null: poses go to and from such memory by one kernel, from anywhere else
-// through c->io (a call that allocated and freed a scratch took 0.2 ms longer).
+// A driver function, without a link to the driver (null: not found).
+template <typename F>
+F driver_entry(const char* name) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &found) != cudaSuccess) cudaGetLastError();
+    return found == cudaDriverEntryPointSuccess ? reinterpret_cast<F>(f) : nullptr;
+}
+
+enum class Extent { WHOLE, BEYOND, UNKNOWN };
+// Whether the bytes at device address p lie in one allocation, end beyond it, or
+// lie in memory mapped piece by piece (cuMemMap), whose pieces the driver gives
+// one at a time.
+Extent device_extent(const void* p, size_t bytes) {
+    static const auto range = driver_entry<decltype(&cuMemGetAddressRange)>("cuMemGetAddressRange");
+    static const auto retain = driver_entry<decltype(&cuMemRetainAllocationHandle)>("cuMemRetainAllocationHandle");
+    static const auto release = driver_entry<decltype(&cuMemRelease)>("cuMemRelease");
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<uintptr_t>(p);
+    if (!range || !retain || !release || range(&base, &size, at) != CUDA_SUCCESS) return Extent::UNKNOWN;
+    if (at - base <= size && bytes <= size - (at - base)) return Extent::WHOLE;
+    CUmemGenericAllocationHandle piece;
+    if (retain(&piece, const_cast<void*>(p)) != CUDA_SUCCESS) return Extent::BEYOND;
+    release(piece);
+    return Extent::UNKNOWN;
+}
+
+// *out = p where a kernel on the context's device can use it as an array of
+// count T, else null: poses go to and from such memory by one kernel, from
+// anywhere else through c->io (a call that allocated and freed a scratch took
+// 0.2 ms longer). An array that ends beyond its allocation is refused, as the
+// copy of it was that the kernel takes the place of.
 template <typename T>
-T* on_device(mp_ctx* c, const void* p) {
+int on_device(mp_ctx* c, const void* p, int64_t count, T** out) {
+    *out = nullptr;
     cudaPointerAttributes at;
     if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return MP_OK;
     }
-    const bool here = at.type == cudaMemoryTypeDevice && at.device == c->device;
-    return here && reinterpret_cast<uintptr_t>(p) % sizeof(T) == 0 ? static_cast<T*>(const_cast<void*>(p)) : nullptr;
+    if (at.type != cudaMemoryTypeDevice || at.device != c->device || reinterpret_cast<uintptr_t>(p) % sizeof(T) != 0)
+        return MP_OK;
+    const Extent ext = device_extent(p, sizeof(T) * (size_t)count);
+    if (ext == Extent::BEYOND)
+        return mp_cuda_check(c, cudaErrorInvalidValue, "the array ends beyond its device allocation");
+    if (ext == Extent::WHOLE) *out = static_cast<T*>(const_cast<void*>(p));
+    return MP_OK;
 }
 
 int io_floats(mp_ctx* c) { return dalloc(c, &c->io, 7 * (size_t)c->cap); }
 
 // c->n poses of seven floats at src, host or device memory, into dst; the caller waits
 int put_poses(mp_ctx* c, const void* src, float4* dst) {
-    const float* from = on_device<float>(c, src);
+    float* dev;
+    int rc = on_device(c, src, 7 * c->n, &dev);
+    if (rc) return rc;
+    const float* from = dev;
     if (!from) {
-        const int rc = io_floats(c);
-        if (rc) return rc;
+        if ((rc = io_floats(c))) return rc;
         MP_CUDA(c, cudaMemcpyAsync(c->io, src, sizeof(float) * 7 * (size_t)c->n, cudaMemcpyDefault, c->stream));
         from = c->io;
     }
@@ -359,9 +399,11 @@ int put_poses(mp_ctx* c, const void* src, float4* dst) {
 
 // the current poses, seven floats each, into dst, host or device memory; the caller waits
 int get_poses(mp_ctx* c, void* dst) {
-    if (float* to = on_device<float>(c, dst)) return mp_launch_unpack_poses(c, c->poses[c->cur], to);
-    int rc = io_floats(c);
-    if (rc || (rc = mp_launch_unpack_poses(c, c->poses[c->cur], c->io))) return rc;
+    float* to;
+    int rc = on_device(c, dst, 7 * c->n, &to);
+    if (rc) return rc;
+    if (to) return mp_launch_unpack_poses(c, c->poses[c->cur], to);
+    if ((rc = io_floats(c)) || (rc = mp_launch_unpack_poses(c, c->poses[c->cur], c->io))) return rc;
     MP_CUDA(c, cudaMemcpyAsync(dst, c->io, sizeof(float) * 7 * (size_t)c->n, cudaMemcpyDefault, c->stream));
     return MP_OK;
 }
@@ -754,9 +796,10 @@ int mp_get_posterior(mp_ctx* c, float* poses_out, double* prob_out, float best_p
     if (!c) return MP_EINVAL;
     if (c->n == 0) return mp_fail(c, MP_ENOTINIT, "particles not initialised");
     const PostHost* h = &c->host->post;
-    float* poses = on_device<float>(c, poses_out);
-    double* prob = on_device<double>(c, prob_out);
+    float* poses;
+    double* prob;
     int rc;
+    if ((rc = on_device(c, poses_out, 7 * c->n, &poses)) || (rc = on_device(c, prob_out, c->n, &prob))) return rc;
     if ((rc = mp_launch_read_posterior(c, poses, prob))) return rc;
     if (poses_out && !poses && (rc = get_poses(c, poses_out))) return rc;
     if (prob_out && !prob)
@@ -823,7 +866,9 @@ int mp_get_buffer(mp_ctx* c, int which, void* dst, int64_t count) {
             return MP_OK;
         }
         case MP_BUF_GN: {
-            if (float* to = on_device<float>(c, dst)) {
+            float* to;
+            if ((rc = on_device(c, dst, MP_GN * n, &to))) return rc;
+            if (to) {
                 if ((rc = mp_launch_gather_gn(c, to))) return rc;
                 MP_CUDA(c, cudaStreamSynchronize(c->stream));
                 return MP_OK;

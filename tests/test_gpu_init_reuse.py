@@ -1,6 +1,9 @@
 """Particles set again in a context that has stepped: as many (its buffers are
 kept), more and fewer. The state is the one a fresh context starts from, and
-poses go in and out of host and device memory alike."""
+poses go in and out of host and device memory alike; a device buffer that ends
+beyond its allocation is refused."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -44,3 +47,44 @@ def test_particles_set_again_start_afresh():
                 assert np.any(np.all(on_host == best, 1)) and 0 < prob <= 1
     finally:
         mp.mp_destroy(c)
+
+
+def test_device_buffers_beyond_their_allocation_are_refused():
+    """Poses, probabilities and sums go straight to device memory by a kernel:
+    where the caller's allocation is too short for them the call is refused, as
+    the copy of the same size is, and the context goes on."""
+    import torch
+    from paper_2404_16370_gb300 import mp
+    torch.zeros(1, device="cuda")
+    cu, L = C.CDLL("libcuda.so.1"), mp.lib()
+    room = synth.box_room(1)
+    n = 300
+    p = synth.box_room_particles(n, 3, room.half).astype(np.float32)
+    c = mp.mp_init_map(room.map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n))
+
+    def alloc(count):
+        d = C.c_uint64()
+        assert cu.cuMemAlloc_v2(C.byref(d), C.c_size_t(count)) == 0
+        return d
+
+    short, whole = alloc(1024), alloc(29 * 4 * n)
+    try:
+        mp.mp_init_particles(c, n, poses=p)
+        calls = {"posterior": lambda d: L.mp_get_posterior(c, C.c_void_p(d), None, None, None),
+                 "probabilities": lambda d: L.mp_get_posterior(c, None, C.c_void_p(d), None, None),
+                 "poses": lambda d: L.mp_get_buffer(c, mp.MP_BUF_POSES, C.c_void_p(d), C.c_int64(7 * n)),
+                 "sums": lambda d: L.mp_get_buffer(c, mp.MP_BUF_GN, C.c_void_p(d), C.c_int64(29 * n)),
+                 "set": lambda d: L.mp_set_buffer(c, mp.MP_BUF_POSES, C.c_void_p(d), C.c_int64(7 * n))}
+        for name, call in calls.items():
+            assert call(short.value) == mp.MP_ECUDA, name
+            assert "beyond its device allocation" in mp.mp_last_error(c), name
+            assert call(whole.value + 29 * 4 * n - 1024) == mp.MP_ECUDA, name     # in the middle of one
+        for name in ("sums", "probabilities", "posterior", "poses", "set"):      # the last: what "poses" wrote
+            assert calls[name](whole.value) == mp.MP_OK, name
+        end = whole.value + (29 - 7) * 4 * n                                     # up to the allocation's last byte
+        assert calls["poses"](end) == mp.MP_OK and calls["set"](end) == mp.MP_OK
+        np.testing.assert_array_equal(mp.mp_get_buffer(c, mp.MP_BUF_POSES).reshape(n, 7), p)
+    finally:
+        mp.mp_destroy(c)
+        for d in (short, whole):
+            cu.cuMemFree_v2(C.c_uint64(d.value))
