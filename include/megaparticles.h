@@ -344,10 +344,13 @@ int mp_kernel_launches(mp_ctx* ctx, int64_t* count);
  * for every instance it serves and returns. In a batch the first instance's
  * knob and wait budget when mp_batch_create captures the step apply, to the
  * posterior and, with instances of more than 16384 particles, to the batch's
- * LSH/sort phase (also one cooperative launch). */
+ * LSH/sort phase (also one cooperative launch). MP_DEBUG_FAIL_GICP_ALLOC: the
+ * value-th device allocation of the next mp_gicp on a context without GICP
+ * buffers fails as if out of memory (0: none). */
 #define MP_DEBUG_WAIT_BUDGET 1
 #define MP_DEBUG_STARVE_TX 2
 #define MP_DEBUG_STARVE_BARRIER 3
+#define MP_DEBUG_FAIL_GICP_ALLOC 4
 int mp_debug_set(mp_ctx* ctx, int what, int64_t value);
 
 /* ---------------------------------------------------------------------------

@@ -503,8 +503,9 @@ int gicp_alloc(mp_ctx* c) {
     const int cap = c->p.max_scan;
     g->cap = cap;
     cudaError_t e = cudaSuccess;
+    int left = c->fail_gicp_alloc;   // test knob: the allocation of this number fails (0: none)
     auto A = [&](auto** p, size_t n) {
-        if (e == cudaSuccess) e = galloc(p, n);
+        if (e == cudaSuccess) e = left > 0 && --left == 0 ? cudaErrorMemoryAllocation : galloc(p, n);
     };
     A(&g->src_raw, 3 * (size_t)cap); A(&g->tgt_raw, 3 * (size_t)cap); A(&g->src_n, 3 * (size_t)cap);
     A(&g->tgt_n, 3 * (size_t)cap); A(&g->src_v, cap); A(&g->tgt_v, cap); A(&g->tmp4, 2 * (size_t)cap);
@@ -519,9 +520,10 @@ int gicp_alloc(mp_ctx* c) {
     A(&g->partial, 2 * (size_t)NPART * std::max(g->grid, 1));
     A(&g->state, ST_N); A(&g->prev, 3 * (size_t)cap);
     c->gicp = g;
+    if (e == cudaSuccess && g->grid >= 1) return MP_OK;
+    mp_gicp_free(c);   // so that another call allocates again
     if (e != cudaSuccess) return mp_cuda_check(c, e, "GICP buffers");
-    if (g->grid < 1) return mp_fail(c, MP_ECUDA, "GICP: no resident CTAs for the cooperative launch");
-    return MP_OK;
+    return mp_fail(c, MP_ECUDA, "GICP: no resident CTAs for the cooperative launch");
 }
 
 // 6x6 SPD inverse on the host (Gauss-Jordan, FP64); false if singular

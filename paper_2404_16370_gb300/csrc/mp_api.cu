@@ -6,6 +6,7 @@
 
 #include <cuda.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
@@ -37,6 +38,7 @@ int mp_fail_noctx(int code, const char* fmt, ...) {
 }
 
 int mp_cuda_check(mp_ctx* c, cudaError_t e, const char* what) {
+    cudaGetLastError();   // reported here: not again by the next launch's check
     int code = (e == cudaErrorMemoryAllocation) ? MP_ENOMEM : MP_ECUDA;
     return mp_fail(c, code, "%s: %s", what, cudaGetErrorString(e));
 }
@@ -1066,6 +1068,7 @@ int mp_debug_set(mp_ctx* c, int what, int64_t value) {
         case MP_DEBUG_WAIT_BUDGET: c->wait_budget = value > 0 ? (long long)value : 0; return MP_OK;
         case MP_DEBUG_STARVE_TX: c->starve_tx = value ? 1 : 0; return MP_OK;
         case MP_DEBUG_STARVE_BARRIER: c->starve_bar = value ? 1 : 0; return MP_OK;
+        case MP_DEBUG_FAIL_GICP_ALLOC: c->fail_gicp_alloc = value > 0 ? (int)std::min<int64_t>(value, 1000) : 0; return MP_OK;
     }
     return mp_fail(c, MP_EINVAL, "unknown debug knob %d", what);
 }

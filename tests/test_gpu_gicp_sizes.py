@@ -2,7 +2,8 @@
 scans that end inside a tile of 64 target points, one scan much smaller than
 the other, more source points than one round of the grid, every target point
 twice (ties go to the smaller index), and a start too far for the last
-iteration's correspondence to be the nearest point."""
+iteration's correspondence to be the nearest point. A call whose buffers could
+not be allocated leaves the context able to try again."""
 import numpy as np
 import pytest
 from scipy.spatial.transform import Rotation
@@ -49,3 +50,26 @@ def test_gicp_sizes(oracle, n_src, n_tgt, twice, far):
     D = np.linalg.inv(g["T"]) @ r["T"]
     assert Rotation.from_matrix(D[:3, :3]).magnitude() < 1e-5 and np.linalg.norm(D[:3, 3]) < 1e-5
     assert np.abs(g["cov"] - r["cov"]).max() <= 1e-3 * np.abs(r["cov"]).max()
+
+
+@pytest.mark.parametrize("which", [1, 2, 9, 13, 15])
+def test_gicp_after_a_failed_allocation(which):
+    """The knob makes one of the buffers' allocations fail: the call reports it,
+    and the next one allocates all of them afresh and gives the same motion."""
+    from paper_2404_16370_gb300 import mp
+    room = synth.box_room(1)
+    p0 = synth.box_room_gt_pose(room, 3)
+    s0, s1 = (synth.scan(room, p0, synth.spherical_dirs(500), 0.02, k) for k in (1, 2))
+    c, d = (mp.mp_init_map(room.map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, 64)) for _ in range(2))
+    try:
+        mp.mp_debug_set(c, mp.MP_DEBUG_FAIL_GICP_ALLOC, which)
+        for _ in range(2):
+            with pytest.raises(mp.MPError) as e:
+                mp.mp_gicp(c, s1, s0)
+            assert e.value.code == mp.MP_ENOMEM
+        mp.mp_debug_set(c, mp.MP_DEBUG_FAIL_GICP_ALLOC, 0)
+        a, b = mp.mp_gicp(c, s1, s0), mp.mp_gicp(d, s1, s0)
+        assert np.array_equal(a["T"], b["T"]) and np.array_equal(a["cov"], b["cov"]) and a["n_corr"] == b["n_corr"]
+    finally:
+        mp.mp_destroy(c)
+        mp.mp_destroy(d)
