@@ -664,17 +664,24 @@ int mp_init_particles(mp_ctx* c, int64_t n, const float lo[6], const float hi[6]
     if (!c) return MP_EINVAL;
     if (n <= 0 || n > ((int64_t)1 << 26)) return mp_fail(c, MP_EINVAL, "n_particles must lie in [1, 2^26]");
     if (!poses && (!lo || !hi)) return mp_fail(c, MP_EINVAL, "need poses or bounds");
+    for (int a = 0; a < 6 && !poses; ++a)
+        if (!(hi[a] >= lo[a])) return mp_fail(c, MP_EINVAL, "bounds: hi < lo");
     MP_CUDA(c, cudaStreamSynchronize(c->stream));
     int rc = alloc_particles(c, n);
     if (rc) return rc;
     c->n = n;
     c->step = 0;
+    // until all is set there are no particles: a step would index by lists never written
+    struct Unset {
+        mp_ctx* c;
+        ~Unset() {
+            if (c) c->n = 0;
+        }
+    } unset{c};
     if (poses) {
         if ((rc = put_poses(c, poses, c->poses[0]))) return rc;
-    } else {
-        for (int a = 0; a < 6; ++a)
-            if (!(hi[a] >= lo[a])) return mp_fail(c, MP_EINVAL, "bounds: hi < lo");
-        if ((rc = mp_launch_init_uniform(c, lo, hi))) return rc;
+    } else if ((rc = mp_launch_init_uniform(c, lo, hi))) {
+        return rc;
     }
     if (log_prior) {
         MP_CUDA(c, cudaMemcpyAsync(c->logprior, log_prior, sizeof(double) * (size_t)n, cudaMemcpyDefault, c->stream));
@@ -688,6 +695,7 @@ int mp_init_particles(mp_ctx* c, int64_t n, const float lo[6], const float hi[6]
     MP_CUDA(c, cudaMemsetAsync(c->psi, 0, sizeof(float) * 8 * (size_t)n, c->stream));
     MP_CUDA(c, cudaMemsetAsync(c->phi, 0, sizeof(float) * 8 * (size_t)n, c->stream));
     MP_CUDA(c, cudaStreamSynchronize(c->stream));
+    unset.c = nullptr;
     return MP_OK;
 }
 

@@ -1,7 +1,8 @@
 """Particles set again in a context that has stepped: as many (its buffers are
 kept), more and fewer. The state is the one a fresh context starts from, and
 poses go in and out of host and device memory alike; a device buffer that ends
-beyond its allocation is refused."""
+beyond its allocation is refused; a refused call leaves the particles as they
+were, and one that fails half-way leaves none."""
 import ctypes as C
 
 import numpy as np
@@ -88,3 +89,36 @@ def test_device_buffers_beyond_their_allocation_are_refused():
         mp.mp_destroy(c)
         for d in (short, whole):
             cu.cuMemFree_v2(C.c_uint64(d.value))
+
+
+def test_refused_and_failed_initialisation():
+    import torch
+    from paper_2404_16370_gb300 import mp
+    torch.zeros(1, device="cuda")
+    cu = C.CDLL("libcuda.so.1")
+    room = synth.box_room(1)
+    n = 300
+    p = synth.box_room_particles(n, 3, room.half).astype(np.float32)
+    scan = synth.scan(room, synth.box_room_gt_pose(room, 3), synth.spherical_dirs(300), 0.02, 1)
+    c = mp.mp_init_map(room.map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n))
+    short = C.c_uint64()
+    assert cu.cuMemAlloc_v2(C.byref(short), C.c_size_t(1024)) == 0
+    try:
+        mp.mp_init_particles(c, n, poses=p)
+        with pytest.raises(mp.MPError) as e:
+            mp.mp_init_particles(c, 2 * n, lo=np.ones(6, np.float32), hi=np.zeros(6, np.float32))
+        assert e.value.code == mp.MP_EINVAL
+        np.testing.assert_array_equal(mp.mp_get_buffer(c, mp.MP_BUF_POSES).reshape(-1, 7), p)
+        mp.mp_step(c, scan)
+        mp.mp_get_posterior(c)
+        assert mp.lib().mp_init_particles(c, 2 * n, None, None, C.c_void_p(short.value), None) == mp.MP_ECUDA
+        with pytest.raises(mp.MPError) as e:
+            mp.mp_step(c, scan)
+        assert e.value.code == mp.MP_ENOTINIT
+        mp.mp_init_particles(c, n, poses=p)
+        mp.mp_step(c, scan)
+        best, prob = mp.mp_get_posterior(c)
+        assert np.isfinite(best).all() and 0 < prob <= 1
+    finally:
+        mp.mp_destroy(c)
+        cu.cuMemFree_v2(short)
