@@ -264,7 +264,11 @@ int mp_set_precision(mp_ctx* ctx, int precision);
  * CTAs per block of particles (1 to 64; default 1), whose partial sums are
  * added atomically into the Gauss-Newton sums (summation order, so the last
  * bits, then depend on scheduling). Splitting puts more CTAs to work when the
- * particles are very few; mp_batch_create picks it per instance by timing. */
+ * particles are very few. Unsplit, the sums of a map of more than 512 voxels
+ * across or of 81920 particles and more are added in the order of the scan;
+ * a split takes another form of the kernel there too, and outdoors the last
+ * bits of one step move points to other voxels in the next. mp_batch_create
+ * therefore picks a split, by timing, for the other instances only. */
 int mp_set_likelihood_split(mp_ctx* ctx, int split);
 
 /* ---- Scan-to-scan GICP odometry (Sec. III-B, prediction step) ----------
@@ -303,7 +307,8 @@ int mp_step_gicp(mp_ctx* ctx, const float* scan, int32_t n_scan, double cov_scal
  * runs all stages, the prediction included (identity odometry without noise
  * is applied, not skipped). tune_scans (may be NULL; else one host scan per
  * instance) is used to pick, by timing, each instance's likelihood split
- * (mp_set_likelihood_split): alone first, then as a policy over the grouped
+ * (mp_set_likelihood_split; 1 on maps of more than 512 voxels across and from
+ * 81920 particles on): alone first, then as a policy over the grouped
  * launch; the pick runs the scan, LSH and sort stages of each instance once on
  * its own stream. Contexts must use the FP32 likelihood and must not have
  * timing enabled; their streams only order other calls on them before and

@@ -153,10 +153,13 @@ int plan_step(mp_group* G, int p, std::vector<GOp>& plan) {
 
 // Time the likelihood of c (its current particles and scan) for each split
 // and keep the fastest. The scan, LSH and sort stages run first so that the
-// particle order the kernel reads is set.
+// particle order the kernel reads is set. Where the unsplit form adds the sums
+// in scan order (wide maps, many particles) a split would take another form and
+// order, and the results would hang on a clock: there it stays 1.
 int autotune_split(mp_ctx* c) {
     int rc;
     if ((rc = mp_run_stages(c, MP_STAGE_SCAN | MP_STAGE_LSH | MP_STAGE_SORT))) return rc;
+    if (mp_likelihood_in_scan_order(c)) return MP_OK;   // (lk_split is 1)
     cudaEvent_t e0, e1;
     B_CUDA(cudaEventCreate(&e0));
     B_CUDA(cudaEventCreate(&e1));

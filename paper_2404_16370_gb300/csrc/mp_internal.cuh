@@ -572,6 +572,7 @@ static inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + b
 void draw_lsh(mp_ctx* c);
 void odom_to_pose_host(const double T[16], double q[4], double t[3]);   // identity for NULL
 void mp_gicp_free(mp_ctx* c);
+bool mp_likelihood_in_scan_order(const mp_ctx* c);   // unsplit: a split would change the order of the sums
 void fill_step_host(mp_ctx* c, StepDev* h);
 int upload_step(mp_ctx* c);
 int mp_launch_map_prepare(mp_ctx* c, const float* xyz_dev);

@@ -171,6 +171,46 @@ def test_autotuned_batch_runs(torch):
         mp.mp_stream_destroy(st)
 
 
+def test_tuned_batch_keeps_the_scan_order(torch):
+    """The tuning splits no scan where the unsplit form adds the sums in scan
+    order: an instance on a map of more than 512 voxels across (the room with
+    two far patches) and one of 82001 particles keep split 1 and equal their
+    own steps bit for bit, beside one whose split is picked."""
+    from paper_2404_16370_gb300 import mp
+    specs = [(11, 1024, 2048), (12, 82001, 300), (13, 1024, 512)]
+    data = [_room_instance(*sp) for sp in specs]
+    y, z = (0.1 * g.ravel() for g in np.meshgrid(np.arange(5), np.arange(5)))
+    far = [np.c_[np.full(25, x), y, z] for x in (-30.0, 30.0)]
+    maps = [d[0].map_points for d in data]
+    maps[0] = np.concatenate([maps[0], *far]).astype(np.float32)
+    st = mp.mp_stream_create()
+
+    def make():
+        cs = []
+        for k, (_, sc, parts) in enumerate(data):
+            n = specs[k][1]
+            cs.append(mp.mp_init_map(maps[k], mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n), cuda_stream=st))
+            mp.mp_init_particles(cs[-1], n, poses=parts)
+        return cs
+
+    A, B = make(), make()
+    scans = [d[1] for d in data]
+    batch = mp.mp_batch_create(A, [len(s) for s in scans], st, tune_scans=scans)
+    try:
+        assert [mp.mp_batch_split(batch, i) for i in (0, 1)] == [1, 1]
+        for step in range(2):
+            T, cov = _odometry(len(specs), step)
+            mp.mp_batch_step(batch, scans, T, cov)
+            for i, ctx in enumerate(B):
+                mp.mp_step(ctx, scans[i], T[i], cov[i])
+        _compare(A[:2], B[:2])
+    finally:
+        mp.mp_batch_destroy(batch)
+        for c in A + B:
+            mp.mp_destroy(c)
+        mp.mp_stream_destroy(st)
+
+
 def test_batch_refuses_outside_steps(torch):
     """A batched context stepped with mp_step is refused by the next batch
     step (its neighbour-list index no longer matches the captured graph)."""
