@@ -1157,10 +1157,18 @@ __global__ void __launch_bounds__(PM_THREADS, PM_MINB) k_likelihood_pm(const LkA
 // now: 1024 particles x 8192 points 6.2 -> 1.9 ms, 8192 5.7 -> 1.9, 32768 5.5 ->
 // 2.6, 65536 6.2 -> 5.0, 98304 7.2 -> 6.7; 131072 8.15 and 8.19; 50021 x 4999 3.59
 // -> 2.07). The sums are the packed form's, bit for bit.
+struct LkPm1Op {
+    using Args = LkArgs;
+    static constexpr int THREADS = PM_THREADS, MINB = PM1_MINB;
+    static __device__ __forceinline__ void run(const LkArgs& A, unsigned bxi, unsigned) {
+        __shared__ __align__(128) LkPmStage st;
+        const int nv = lk_pm_begin(A, st, bxi);
+        lk_pm_block<false, float>(A, st, bxi, nv, 0, (nv + PM_CHUNK - 1) / PM_CHUNK, 0);
+    }
+};
+
 __global__ void __launch_bounds__(PM_THREADS, PM1_MINB) k_likelihood_pm1(const LkArgs A) {
-    __shared__ __align__(128) LkPmStage st;
-    const int nv = lk_pm_begin(A, st, blockIdx.x);
-    lk_pm_block<false, float>(A, st, blockIdx.x, nv, 0, (nv + PM_CHUNK - 1) / PM_CHUNK, 0);
+    LkPm1Op::run(A, blockIdx.x, 0);
 }
 
 // The same over parts of the scan: item t of A.items x blocks is part t /
@@ -1524,14 +1532,18 @@ int mp_launch_likelihood(mp_ctx* c) {
 }
 
 // Grouped likelihood (FP32): one launch for the instances in particle-major
-// form; of the others, per segment of the scan, one for those whose particles
+// form, or, while those on wide maps have at most LK_PM1_MAX particles in all,
+// one for them with one particle a thread and one for the rest (the same bits;
+// a step of 24 instances of 1024 x 8192 points on a wide map 7.84 -> 6.00 ms, of 24 of
+// 1024-8192 x 512-2048 2.26 -> 1.69; 8 of 32768, above the line, 6.2); of the others, per segment of the scan, one for those whose particles
 // take a warp each and one for those whose particles take a CTA (the sums of
 // an instance with a scan split zeroed first; block (bx, by) of the map =
 // particle block bx, scan part by).
 int mp_plan_likelihood(mp_group* G, int, std::vector<GOp>& plan) {
     std::vector<LkArgs> tab;
-    std::vector<int64_t> blocks, blocks_pm;
-    std::vector<int> ys, nseg, pm;
+    std::vector<int64_t> blocks, blocks_pm, blocks_pm1;
+    std::vector<int> ys, nseg, pm, wide;
+    int64_t n_wide = 0;
     int segs = 0;
     for (int i = 0; i < G->size(); ++i) {
         mp_ctx* c = G->ctx[i];
@@ -1539,14 +1551,25 @@ int mp_plan_likelihood(mp_group* G, int, std::vector<GOp>& plan) {
         LkArgs& A = tab.back();
         blocks.push_back(lk_blocks(A));
         blocks_pm.push_back((c->n + PM_PER_CTA - 1) / PM_PER_CTA);
+        blocks_pm1.push_back((c->n + PM_THREADS - 1) / PM_THREADS);
         ys.push_back(A.split);
         const bool by_particle = lk_particle_major(c, A.split);
-        if (by_particle) pm.push_back(i);
+        if (by_particle) (lk_wide(c) ? wide : pm).push_back(i);
+        if (by_particle && lk_wide(c)) n_wide += c->n;
         nseg.push_back(by_particle ? 0 : lk_segments(G->n_scan[i], A));
         segs = std::max(segs, nseg.back());
         if (A.split > 1) plan_memset(plan, c->gn, sizeof(float) * MP_GN * (size_t)c->cap);
     }
     unsigned nblk = 0;
+    if (n_wide > LK_PM1_MAX) {
+        pm.insert(pm.end(), wide.begin(), wide.end());
+        wide.clear();
+    }
+    if (!wide.empty()) {
+        const LkArgs* t = G->upload(tab);
+        const GBlk* m = G->block_map(blocks_pm1, &nblk, wide);
+        plan_kernel<LkPm1Op>(plan, t, m, nblk);
+    }
     if (!pm.empty()) {
         const LkArgs* t = G->upload(tab);
         const GBlk* m = G->block_map(blocks_pm, &nblk, pm);

@@ -211,6 +211,48 @@ def test_tuned_batch_keeps_the_scan_order(torch):
         mp.mp_stream_destroy(st)
 
 
+@pytest.mark.parametrize("wide,sizes,buckets", [(False, [3000, 16385, 16384, 40001], [8, 9, 14, 17]),
+                                                (True, [70001, 50000], [0, 0])])
+def test_large_instances_equal_sequential_steps(torch, wide, sizes, buckets):
+    """Instances on both sides of 16384 particles, the line between one sort
+    CTA each and the persistent sort phase, in mixed order and with 1 to 3 radix
+    passes; and two on a wide map with more particles in all than the
+    likelihood gives a thread each: bit for bit their own steps."""
+    from paper_2404_16370_gb300 import mp
+    room, sc, _ = _room_instance(14, 8, 700)
+    y, z = (0.1 * g.ravel() for g in np.meshgrid(np.arange(5), np.arange(5)))
+    far = [np.c_[np.full(25, x), y, z] for x in (-30.0, 30.0)] if wide else []
+    pts = np.concatenate([room.map_points, *far]).astype(np.float32)
+    st = mp.mp_stream_create()
+
+    def make():
+        cs = []
+        for n, b in zip(sizes, buckets):
+            p = mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n, **({"n_buckets_log2": b} if b else {}))
+            cs.append(mp.mp_init_map(pts, p, cuda_stream=st))
+            mp.mp_init_particles(cs[-1], n, poses=synth.box_room_particles(n, n, room.half))
+        return cs
+
+    A, B = make(), make()
+    scans = [sc[:700 - 100 * k] for k in range(len(sizes))]
+    batch = mp.mp_batch_create(A, [len(s) for s in scans], st)
+    try:
+        for step in range(2):
+            T, cov = _odometry(len(sizes), step)
+            mp.mp_batch_step(batch, scans, T, cov)
+            for i, ctx in enumerate(B):
+                mp.mp_step(ctx, scans[i], T[i], cov[i])
+        _compare(A, B)
+        for a, b in zip(A, B):
+            for which in (mp.MP_BUF_SORTED_IDS, mp.MP_BUF_SEGMENTS, mp.MP_BUF_VISIT_ORDER):
+                assert np.array_equal(mp.mp_get_buffer(a, which), mp.mp_get_buffer(b, which))
+    finally:
+        mp.mp_batch_destroy(batch)
+        for c in A + B:
+            mp.mp_destroy(c)
+        mp.mp_stream_destroy(st)
+
+
 def test_batch_refuses_outside_steps(torch):
     """A batched context stepped with mp_step is refused by the next batch
     step (its neighbour-list index no longer matches the captured graph)."""
