@@ -5,7 +5,10 @@
  * Particle Filter", ICRA 2024 (arXiv 2404.16370).
  *
  * One filter step (mp_step) runs, on the context's CUDA stream and entirely in
- * this library's kernels:
+ * this library's kernels (the scan Gaussians on a stream of the context's own
+ * beside it, of the same priority, between an event and a wait on the
+ * context's stream: what is queued there before and after a step still comes
+ * before and after all of it):
  *   prediction                 Sec. III-B, Eq. 1
  *   scan Gaussians             Sec. III-C, GICP point model
  *   neighbour list update      Sec. III-C, Eq. 9-10, Algorithm 1
@@ -101,7 +104,8 @@ int mp_default_params(mp_params* p, int preset, int64_t n_particles);
  * than cov_min: the point is unused), then the NNF: for every voxel of the map
  * box padded by r_max, the nearest valid map point to the voxel centre within
  * r_max (-1 if none). cuda_stream: a cudaStream_t the context will use for all
- * its work (NULL = legacy default stream). On success *ctx owns the device
+ * its work (NULL = legacy default stream); the context's own stream for the scan
+ * Gaussians is ordered by it and gets its priority. On success *ctx owns the device
  * memory. Errors: MP_EINVAL (NULL/empty input, bad params, grid too large),
  * MP_ENOMEM, MP_ECUDA; *ctx is NULL on error. */
 int mp_init_map(mp_ctx** ctx, const float* xyz, int64_t n_map, const mp_params* p, void* cuda_stream);

@@ -530,7 +530,9 @@ static int ctx_setup(mp_ctx* c) {
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&c->step_ev[k], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+        int priority = 0;   // the scan's kernels wait in line with the others of the step
+        if (e == cudaSuccess) e = cudaStreamGetPriority(c->stream, &priority);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, priority);
         if (e != cudaSuccess) { rc = mp_cuda_check(c, e, "cudaEventCreate"); break; }
         e = cudaMemsetAsync(c->dev_error, 0, sizeof(int32_t), c->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(c->scan_nvalid, 0, sizeof(int32_t), c->stream);

@@ -1,7 +1,10 @@
 """A step, whose scan kernels run beside the particles' on a second stream,
 against the same stages run one by one: the same lists and scan Gaussians, and
 the same log-likelihoods up to the order of their sums. Scans change from step
-to step, so that one read too early or too late would show."""
+to step, so that one read too early or too late would show. The second stream
+has the priority of the caller's."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -37,3 +40,41 @@ def test_step_equals_its_stages(n):
     finally:
         for c in ctx:
             mp.mp_destroy(c)
+
+
+@pytest.mark.parametrize("priority", [0, -1, -3])
+def test_every_kernel_has_the_callers_priority(priority):
+    """The stages captured into a graph (not run): each kernel node carries the
+    priority of the stream that it was launched on."""
+    import torch
+    from paper_2404_16370_gb300 import mp
+    stream = torch.cuda.Stream(priority=priority)
+    cu, s = C.CDLL("libcuda.so.1"), C.c_void_p(stream.cuda_stream)
+    room = synth.box_room(1)
+    c = mp.mp_init_map(room.map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, 500), cuda_stream=stream.cuda_stream)
+    graph = C.c_void_p()
+    try:
+        mp.mp_init_particles(c, 500, poses=synth.box_room_particles(500, 3, room.half))
+        mp.mp_set_scan(c, synth.scan(room, synth.box_room_gt_pose(room, 3), synth.spherical_dirs(300), 0.02, 1))
+        torch.cuda.synchronize()
+        assert cu.cuStreamBeginCapture_v2(s, 2) == 0
+        try:
+            mp.mp_run_stages(c, mp.MP_STAGE_SCAN | mp.MP_STAGE_MERGE | mp.MP_STAGE_LIKELIHOOD)
+        finally:
+            assert cu.cuStreamEndCapture(s, C.byref(graph)) == 0
+        count = C.c_size_t()
+        assert cu.cuGraphGetNodes(graph, None, C.byref(count)) == 0
+        nodes = (C.c_void_p * count.value)()
+        assert cu.cuGraphGetNodes(graph, nodes, C.byref(count)) == 0
+        got = []
+        for node in nodes:
+            kind, value = C.c_int(), (C.c_int * 16)()
+            assert cu.cuGraphNodeGetType(C.c_void_p(node), C.byref(kind)) == 0
+            if kind.value == 0:   # a kernel; its attribute 8 is the priority
+                assert cu.cuGraphKernelNodeGetAttribute(C.c_void_p(node), 8, value) == 0
+                got.append(value[0])
+    finally:
+        mp.mp_destroy(c)
+        if graph:
+            cu.cuGraphDestroy(graph)
+    assert len(got) == 5 and set(got) == {stream.priority}   # three of the scan, merge, likelihood
