@@ -348,12 +348,16 @@ int mp_kernel_launches(mp_ctx* ctx, int64_t* count);
  * bounded wait gives up; the kernel then records the error (reported as
  * MP_ETIMEOUT by the next mp_get_posterior) and returns. No copy is left in
  * flight. MP_DEBUG_STARVE_BARRIER: when non-zero, the first grid barrier of
- * the posterior stage (one cooperative launch) waits for one CTA more than the
- * grid has, so every CTA's bounded wait gives up; the kernel records the error
- * for every instance it serves and returns. In a batch the first instance's
- * knob and wait budget when mp_batch_create captures the step apply, to the
- * posterior and, with instances of more than 16384 particles, to the batch's
- * LSH/sort phase (also one cooperative launch). MP_DEBUG_FAIL_GICP_ALLOC: the
+ * every cooperative launch waits for one CTA more than the grid has, so every
+ * CTA's bounded wait gives up; the kernel records the error for every instance
+ * it serves and returns. These launches are the posterior stage (with the knob
+ * set also for 129 to 1024 particles, which otherwise take one cluster of CTAs
+ * and its hardware barrier), the sort stage from 3585 to 1245184 particles, and
+ * mp_gicp, which returns MP_ETIMEOUT itself. The likelihood of more than 116736
+ * particles in parts of the scan then waits, as long, for a part that is never
+ * counted. In a batch the first instance's knob and wait budget when
+ * mp_batch_create captures the step apply, to the posterior and, with instances
+ * of more than 16384 particles, to the batch's LSH/sort phase. MP_DEBUG_FAIL_GICP_ALLOC: the
  * value-th device allocation of the next mp_gicp on a context without GICP
  * buffers fails as if out of memory (0: none). */
 #define MP_DEBUG_WAIT_BUDGET 1

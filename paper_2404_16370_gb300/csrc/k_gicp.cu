@@ -76,6 +76,7 @@ struct GicpArgs {
     GridBar* bar;
     int32_t* err;
     long long budget;
+    int starve;              // test knob: the first barrier waits for one CTA more than the grid
 };
 
 __device__ __forceinline__ float gicp_word(const float* s, int i, int k) { return __ldg(s + scan_word(i, k)); }
@@ -427,9 +428,10 @@ __global__ void __launch_bounds__(GB) k_gicp(const GicpArgs A) {
                 A.box[6 * t + 3 + a] = hi[a];
             }
     }
-    unsigned target = 0;
+    unsigned target = 0, expect = gridDim.x + (A.starve ? 1u : 0u);
     auto sync = [&] {
-        const bool ok = grid_sync(A.bar, target, gridDim.x, A.budget);
+        const bool ok = grid_sync(A.bar, target, expect, A.budget);
+        expect = gridDim.x;
         if (!ok && threadIdx.x == 0) atomicOr(A.err, MP_ERR_WAIT);
         return ok;
     };
@@ -612,6 +614,7 @@ int mp_gicp(mp_ctx* c, const float* src, int32_t n_src, const float* tgt, int32_
     A.bar = g->bar;
     A.err = g->counts + 2;
     A.budget = c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET;
+    A.starve = c->starve_bar;
     MP_CUDA(c, cudaMemsetAsync(g->bar, 0, sizeof(GridBar), c->stream));
     MP_CUDA(c, cudaMemsetAsync(A.err, 0, sizeof(int32_t), c->stream));
     MP_CUDA(c, launch_coop((const void*)k_gicp, (unsigned)std::min(g->grid, (n_src + GPTS - 1) / GPTS), GB, &A, c->stream));

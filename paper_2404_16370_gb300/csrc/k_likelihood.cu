@@ -97,6 +97,7 @@ struct LkArgs {
     unsigned long long* pairs;
     long long budget;   // cycle limit of each barrier wait
     int starve;         // test knob: announce 16 bytes more than copied for chunk 0
+    int starve_ticket;  // test knob (k_likelihood_pm_parts): the first block's parts are not counted
     int split;          // CTAs sharing the scan of one particle block (gridDim.y); > 1 adds atomically
     int seg, seg_len;   // the launch's part of the scan, of seg_len <= LK_SEG chunks (times split)
     int wpp;            // warps sharing a particle (1 or LK_WARPS)
@@ -1216,7 +1217,7 @@ __global__ void __launch_bounds__(PM_THREADS, PM_MINB) k_likelihood_pm_parts(con
         q += c1 - c0;
         __threadfence();      // the stored sums before the count
         __syncthreads();
-        if (threadIdx.x == 0) atomicExch(done + blk, part + 1);
+        if (threadIdx.x == 0 && !(A.starve_ticket && blk == 0)) atomicExch(done + blk, part + 1);
     }
 }
 
@@ -1453,6 +1454,7 @@ LkArgs lk_args(mp_ctx* c) {
     A.err = c->dev_error;
     A.budget = c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET;
     A.starve = c->starve_tx;
+    A.starve_ticket = c->starve_bar;
     A.pairs = c->pairs;
     const float a = 1.f - c->p.eps_cov;
     auto pair = [](float v) { return make_float2(v, v); };

@@ -166,7 +166,8 @@ struct mp_ctx {
     long long wait_budget;   // cycles; 0 = MP_WAIT_BUDGET
     int starve_tx;
     int fail_gicp_alloc;     // test knob: the GICP allocation of this number fails (0: none)
-    int starve_bar;          // test knob: the first grid barrier of the posterior (and of a batch's sort phase) waits for one CTA more than the grid
+    int starve_bar;          // test knob: the first grid barrier of a kernel that has them waits for one CTA
+                             // more than the grid, and the likelihood in parts for a part never counted
     struct GridBar* post_bar;   // the persistent posterior's grid barrier (zeroed before each launch)
 };
 

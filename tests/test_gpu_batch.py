@@ -296,6 +296,48 @@ def test_batch_grid_barrier_timeout_reported_for_every_instance(torch):
         mp.mp_stream_destroy(st)
 
 
+def test_batch_sort_phase_timeout(torch):
+    """The same with an instance of more than 16384 particles, whose sort is a
+    persistent launch too: it gives up at its first barrier, so that instance's
+    order stays the initial one, the small one's (one CTA) does not, and every
+    instance reports MP_ETIMEOUT. With the knob cleared a new batch steps."""
+    from paper_2404_16370_gb300 import mp
+    st = mp.mp_stream_create()
+    specs = [(2, 3000, 300), (3, 16385, 300)]
+    A, data = _instances(st, specs)
+    scans = [d[0] for d in data]
+    try:
+        mp.mp_debug_set(A[0], mp.MP_DEBUG_WAIT_BUDGET, 2_000_000)
+        mp.mp_debug_set(A[0], mp.MP_DEBUG_STARVE_BARRIER, 1)
+        batch = mp.mp_batch_create(A, [len(s) for s in scans], st)
+        try:
+            mp.mp_batch_step(batch, scans)
+            order = [mp.mp_get_buffer(c, mp.MP_BUF_SORTED_IDS) for c in A]
+            assert np.array_equal(order[1], np.arange(16385)) and not np.array_equal(order[0], np.arange(3000))
+            for ctx in A:
+                with pytest.raises(mp.MPError) as e:
+                    mp.mp_get_posterior(ctx)
+                assert e.value.code == mp.MP_ETIMEOUT
+        finally:
+            mp.mp_batch_destroy(batch)
+        mp.mp_debug_set(A[0], mp.MP_DEBUG_WAIT_BUDGET, 0)
+        mp.mp_debug_set(A[0], mp.MP_DEBUG_STARVE_BARRIER, 0)
+        for ctx, (_, n, _), (_, parts) in zip(A, specs, data):
+            mp.mp_init_particles(ctx, n, poses=parts)
+        batch = mp.mp_batch_create(A, [len(s) for s in scans], st)
+        try:
+            mp.mp_batch_step(batch, scans)
+            for ctx in A:
+                mp.mp_get_posterior(ctx)
+                assert abs(mp.mp_get_buffer(ctx, mp.MP_BUF_POST).sum() - 1) < 1e-12
+        finally:
+            mp.mp_batch_destroy(batch)
+    finally:
+        for c in A:
+            mp.mp_destroy(c)
+        mp.mp_stream_destroy(st)
+
+
 def _room_params(n, **over):
     from paper_2404_16370_gb300 import mp
     return mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n, **over)

@@ -305,3 +305,49 @@ def test_grid_barrier_gives_up_and_context_recovers(room):
     finally:
         mp.mp_destroy(ctx)
     assert np.isfinite(post).all() and abs(post.sum() - 1) < 1e-12 and 0 < best_p <= 1
+
+
+def test_every_bounded_wait_gives_up_and_the_context_recovers(room):
+    """The grid barriers of the sort and of GICP, and the wait for the part
+    before in the likelihood in parts, made to run out: each is reported, and
+    with the knob cleared the same call gives what a fresh context gives."""
+    from paper_2404_16370_gb300 import mp
+    sc, sc2 = room["w"].scans[0], room["w"].scans[0][:400]
+
+    def starve(ctx, on):
+        mp.mp_debug_set(ctx, mp.MP_DEBUG_WAIT_BUDGET, 2_000_000 if on else 0)
+        mp.mp_debug_set(ctx, mp.MP_DEBUG_STARVE_BARRIER, on)
+
+    def sort(ctx):
+        mp.mp_run_stages(ctx, mp.MP_STAGE_LSH | mp.MP_STAGE_SORT)
+        mp.mp_get_posterior(ctx)
+        return [mp.mp_get_buffer(ctx, w) for w in (mp.MP_BUF_SORTED_IDS, mp.MP_BUF_VISIT_ORDER, mp.MP_BUF_SEGMENTS)]
+
+    def likelihood(ctx):
+        mp.mp_set_scan(ctx, sc)
+        mp.mp_run_stages(ctx, mp.MP_STAGE_SCAN | mp.MP_STAGE_LIKELIHOOD)
+        mp.mp_get_posterior(ctx)
+        return [mp.mp_get_buffer(ctx, mp.MP_BUF_GN)]
+
+    def gicp(ctx):
+        g = mp.mp_gicp(ctx, sc2, sc)
+        return [g["T"], g["cov"]]
+
+    poses = np.tile(room["w"].particles, (20, 1))
+    for n, call in ((3585, sort), (160_001, sort), (120_000, likelihood), (64, gicp)):   # both forms of the sort
+        got = []
+        for knob in (True, False):
+            ctx = mp.mp_init_map(room["w"].map_points, mp.mp_default_params(mp.MP_PRESET_BOX_ROOM, n))
+            try:
+                mp.mp_init_particles(ctx, n, poses=poses[:n])
+                if knob:
+                    starve(ctx, 1)
+                    with pytest.raises(mp.MPError) as e:
+                        call(ctx)
+                    assert e.value.code == mp.MP_ETIMEOUT, call.__name__
+                    starve(ctx, 0)
+                got.append(call(ctx))
+            finally:
+                mp.mp_destroy(ctx)
+        for a, b in zip(*got):
+            np.testing.assert_array_equal(a, b, err_msg=call.__name__)
