@@ -54,6 +54,7 @@ int mp_checked_sync(mp_ctx* c, const char* file, int line) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone) return MP_OK;
     cudaError_t e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess && c->side) e = cudaStreamSynchronize(c->side);   // the scan's kernels
     if (e != cudaSuccess) {
         fprintf(stderr, "MP_CHECKED: kernel launched at %s:%d: %s\n", file, line, cudaGetErrorString(e));
         return mp_fail(c, MP_ECUDA, "kernel launched at %s:%d: %s", file, line, cudaGetErrorString(e));
