@@ -34,8 +34,7 @@
 
 struct GicpBufs {
     int cap;
-    float *src_raw, *tgt_raw, *src_n, *tgt_n;
-    uint8_t *src_v, *tgt_v;
+    float *src_raw, *tgt_raw;
     float *sorted, *src_soa, *tgt_soa;   // the points, sorted (scan_word): two scans' points; with their normals
     int32_t *idx, *tgt_idx, *counts;     // their original indices; points of src and tgt, error bits
     float4* tmp4;
@@ -509,8 +508,7 @@ int gicp_alloc(mp_ctx* c) {
     auto A = [&](auto** p, size_t n) {
         if (e == cudaSuccess) e = left > 0 && --left == 0 ? cudaErrorMemoryAllocation : galloc(p, n);
     };
-    A(&g->src_raw, 3 * (size_t)cap); A(&g->tgt_raw, 3 * (size_t)cap); A(&g->src_n, 3 * (size_t)cap);
-    A(&g->tgt_n, 3 * (size_t)cap); A(&g->src_v, cap); A(&g->tgt_v, cap); A(&g->tmp4, 2 * (size_t)cap);
+    A(&g->src_raw, 3 * (size_t)cap); A(&g->tgt_raw, 3 * (size_t)cap); A(&g->tmp4, 2 * (size_t)cap);
     const size_t soa = scan_word((cap + MP_SCAN_CHUNK - 1) / MP_SCAN_CHUNK * MP_SCAN_CHUNK, 0);
     A(&g->sorted, 2 * soa); A(&g->src_soa, soa); A(&g->tgt_soa, soa); A(&g->idx, cap); A(&g->tgt_idx, cap); A(&g->counts, 3);
     A(&g->box, 6 * (size_t)((cap + GTILE - 1) / GTILE)); A(&g->corr, cap); A(&g->bar, 1);
@@ -558,8 +556,7 @@ bool inv6(const double H[36], double I[36]) {
 void mp_gicp_free(mp_ctx* c) {
     GicpBufs* g = c->gicp;
     if (!g) return;
-    void* bufs[] = {g->src_raw, g->tgt_raw, g->src_n, g->tgt_n, g->src_v, g->tgt_v, g->sorted,
-                    g->src_soa, g->tgt_soa, g->idx, g->tgt_idx, g->counts, g->tmp4, g->box, g->corr, g->bar, g->partial, g->state, g->prev};
+    void* bufs[] = {g->src_raw, g->tgt_raw, g->sorted, g->src_soa, g->tgt_soa, g->idx, g->tgt_idx, g->counts, g->tmp4, g->box, g->corr, g->bar, g->partial, g->state, g->prev};
     for (void* p : bufs)
         if (p) cudaFree(p);
     delete g;
@@ -581,8 +578,8 @@ int mp_gicp(mp_ctx* c, const float* src, int32_t n_src, const float* tgt, int32_
     MP_CUDA(c, cudaMemcpyAsync(g->tgt_raw, tgt, sizeof(float) * 3 * (size_t)n_tgt, cudaMemcpyDefault, c->stream));
     float* sorted = g->sorted + scan_word((g->cap + MP_SCAN_CHUNK - 1) / MP_SCAN_CHUNK * MP_SCAN_CHUNK, 0);
     const PointScan scans[2] = {
-        {g->src_raw, n_src, g->tmp4, g->src_n, g->src_v, g->sorted, g->src_soa, g->idx, g->counts},
-        {g->tgt_raw, n_tgt, g->tmp4 + g->cap, g->tgt_n, g->tgt_v, sorted, g->tgt_soa, g->tgt_idx, g->counts + 1}};
+        {g->src_raw, n_src, g->tmp4, g->sorted, g->src_soa, g->idx, g->counts},
+        {g->tgt_raw, n_tgt, g->tmp4 + g->cap, sorted, g->tgt_soa, g->tgt_idx, g->counts + 1}};
     if ((rc = mp_launch_point_gaussians(c, scans, 2))) return rc;
     // initial state from init_T (identity when NULL)
     double st[ST_N];

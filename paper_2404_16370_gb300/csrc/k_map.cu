@@ -312,9 +312,9 @@ struct ScanArgs {
     int k, kmin;
     float inv_cell;      // 1 / (4 NNF voxels): the cells of scan_key
     float4* tmp4;        // x, y, z and the bits of scan_key
-    float* normals;
+    float* normals;      // (normals and valid null: every point is sorted, without a normal)
     uint8_t* valid;
-    float4* pair;        // the valid points in input order, broadcast pairs (or null),
+    float4* pair;        // the valid points in input order, broadcast pairs (with normals),
     float* soa;          // and sorted, the likelihood's chunks
     int32_t* idx;        // the sorted points' indices (or null)
     int32_t* nvalid;
@@ -533,19 +533,19 @@ __device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned b
     constexpr uint32_t NONE = 0xffffffffu;   // above every key
     const float* __restrict__ raw = args.raw;
     const float* __restrict__ normals = args.normals;
-    const uint8_t* __restrict__ valid = args.valid;
+    const uint8_t* __restrict__ valid = args.valid;   // null: every point
     const float4* __restrict__ pts = args.tmp4;
     const int n = args.n;
     __shared__ __align__(16) uint32_t sk[SCAN_TILE];
     const int part = threadIdx.x % SCAN_PARTS, pl = threadIdx.x / SCAN_PARTS;
     const int i = (int)bx * SCAN_PTS + pl;
-    const uint32_t key = (i < n && valid[i]) ? __float_as_uint(pts[i].w) : NONE;
+    const uint32_t key = (i < n && (!valid || valid[i])) ? __float_as_uint(pts[i].w) : NONE;
     uint32_t before = 0, earlier = 0, all = 0;   // valid points before this one by key, by index; all
     for (int base = 0; base < n; base += SCAN_TILE) {
         __syncthreads();
         for (int t = threadIdx.x; t < SCAN_TILE; t += SCAN_CTA) {
             const int j = base + t;
-            sk[t] = (j < n && valid[j]) ? __float_as_uint(pts[j].w) : NONE;
+            sk[t] = (j < n && (!valid || valid[j])) ? __float_as_uint(pts[j].w) : NONE;
         }
         __syncthreads();
         const uint32_t lim = key + (base + SCAN_TILE <= i ? 1u : 0u);   // equal keys of an earlier tile count
@@ -586,14 +586,11 @@ __device__ __forceinline__ void ScanSortOp::run(const ScanArgs& args, unsigned b
     if (!MP_DCHECK(o < n && oe < n, "compacted scan index", o)) o = oe = 0;
     float v[6];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        v[k] = raw[3 * i + k];
-        v[3 + k] = normals[3 * i + k];
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) args.soa[scan_word(o, k)] = v[k];
+    for (int k = 0; k < 3; ++k) args.soa[scan_word(o, k)] = v[k] = raw[3 * i + k];
     if (args.idx) args.idx[o] = i;
-    if (!args.pair) return;
+    if (!normals) return;   // the points alone
+#pragma unroll
+    for (int k = 3; k < 6; ++k) args.soa[scan_word(o, k)] = v[k] = normals[3 * i + k - 3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) args.pair[3 * oe + k] = make_float4(v[2 * k], v[2 * k], v[2 * k + 1], v[2 * k + 1]);
 }
@@ -910,15 +907,14 @@ int mp_launch_point_gaussians(mp_ctx* c, const PointScan* in, int m) {
         const PointScan& p = in[k < m ? k : 0];
         ScanArgs& a = A.s[k] = scan_args(c, p.raw, p.n);
         a.tmp4 = p.tmp4;
-        a.normals = p.normals;
-        a.valid = p.valid;
+        a.normals = nullptr;
+        a.valid = nullptr;
         a.pair = nullptr;
         a.soa = p.sorted;
         a.idx = p.idx;
         a.nvalid = p.count;
         a.out = p.out;
         n = std::max(n, p.n);
-        if (k < m) MP_CUDA(c, cudaMemsetAsync(p.valid, 1, (size_t)p.n, c->stream));   // the order takes every point
     }
     k_scan_to_float4<<<dim3(grid_for(n, 256), m), 256, 0, c->stream>>>(A);
     MP_LAUNCHED(c);

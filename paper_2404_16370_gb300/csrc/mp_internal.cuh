@@ -582,8 +582,6 @@ struct PointScan {      // n x 3 points, and what is made of them
     const float* raw;
     int n;
     float4* tmp4;
-    float* normals;      // n x 3, which the sort copies along without need
-    uint8_t* valid;
     float *sorted, *out;   // sorted points; with their normals, invalid ones at 1e18 m (scan_word)
     int32_t *idx, *count;  // sorted points' indices, their number
 };
