@@ -354,8 +354,8 @@ int mp_kernel_launches(mp_ctx* ctx, int64_t* count);
  * set also for 129 to 1024 particles, which otherwise take one cluster of CTAs
  * and its hardware barrier), the sort stage from 3585 to 1245184 particles, and
  * mp_gicp, which returns MP_ETIMEOUT itself. The likelihood of more than 116736
- * particles in parts of the scan then waits, as long, for a part that is never
- * counted. In a batch the first instance's knob and wait budget when
+ * particles in parts of the scan then waits, as long, for a part that no CTA
+ * takes. In a batch the first instance's knob and wait budget when
  * mp_batch_create captures the step apply, to the posterior and, with instances
  * of more than 16384 particles, to the batch's LSH/sort phase. MP_DEBUG_FAIL_GICP_ALLOC: the
  * value-th device allocation of the next mp_gicp on a context without GICP

@@ -167,7 +167,7 @@ struct mp_ctx {
     int starve_tx;
     int fail_gicp_alloc;     // test knob: the GICP allocation of this number fails (0: none)
     int starve_bar;          // test knob: the first grid barrier of a kernel that has them waits for one CTA
-                             // more than the grid, and the likelihood in parts for a part never counted
+                             // more than the grid, and the likelihood in parts for a part not handed out
     struct GridBar* post_bar;   // the persistent posterior's grid barrier (zeroed before each launch)
 };
 
