@@ -353,7 +353,7 @@ int mp_kernel_launches(mp_ctx* ctx, int64_t* count);
  * it serves and returns. These launches are the posterior stage (with the knob
  * set also for 129 to 1024 particles, which otherwise take one cluster of CTAs
  * and its hardware barrier), the sort stage from 3585 to 1245184 particles, and
- * mp_gicp, which returns MP_ETIMEOUT itself. The likelihood of more than 116736
+ * mp_gicp from 65 source points on, which returns MP_ETIMEOUT itself. The likelihood of more than 116736
  * particles in parts of the scan then waits, as long, for a part that no CTA
  * takes. In a batch the first instance's knob and wait budget when
  * mp_batch_create captures the step apply, to the posterior and, with instances

@@ -75,7 +75,6 @@ struct GicpArgs {
     GridBar* bar;
     int32_t* err;
     long long budget;
-    int starve;              // test knob: the first barrier waits for one CTA more than the grid
 };
 
 __device__ __forceinline__ float gicp_word(const float* s, int i, int k) { return __ldg(s + scan_word(i, k)); }
@@ -427,10 +426,9 @@ __global__ void __launch_bounds__(GB) k_gicp(const GicpArgs A) {
                 A.box[6 * t + 3 + a] = hi[a];
             }
     }
-    unsigned target = 0, expect = gridDim.x + (A.starve ? 1u : 0u);
+    unsigned target = 0;
     auto sync = [&] {
-        const bool ok = grid_sync(A.bar, target, expect, A.budget);
-        expect = gridDim.x;
+        const bool ok = grid_sync(A.bar, target, gridDim.x, A.budget);
         if (!ok && threadIdx.x == 0) atomicOr(A.err, MP_ERR_WAIT);
         return ok;
     };
@@ -611,8 +609,7 @@ int mp_gicp(mp_ctx* c, const float* src, int32_t n_src, const float* tgt, int32_
     A.bar = g->bar;
     A.err = g->counts + 2;
     A.budget = c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET;
-    A.starve = c->starve_bar;
-    MP_CUDA(c, cudaMemsetAsync(g->bar, 0, sizeof(GridBar), c->stream));
+    MP_CUDA(c, grid_bar_reset(g->bar, c->starve_bar, c->stream));
     MP_CUDA(c, cudaMemsetAsync(A.err, 0, sizeof(int32_t), c->stream));
     MP_CUDA(c, launch_coop((const void*)k_gicp, (unsigned)std::min(g->grid, (n_src + GPTS - 1) / GPTS), GB, &A, c->stream));
     MP_LAUNCHED(c);

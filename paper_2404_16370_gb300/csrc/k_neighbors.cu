@@ -613,7 +613,6 @@ struct MidSortArgs {
     GridBar* bar;
     int32_t* err;
     long long budget;
-    int starve;           // test knob: the first barrier waits for one CTA more than the grid
 };
 
 template <int MS_ITEMS>
@@ -626,10 +625,9 @@ __global__ void __launch_bounds__(MS_THREADS) k_mid_sort(const __grid_constant__
     const int e0 = (int)blockIdx.x * (MS_THREADS * MS_ITEMS) + w * (32 * MS_ITEMS) + lane;   // item it: e0 + 32 it
     uint32_t key[MS_ITEMS];
     int32_t id[MS_ITEMS];
-    unsigned target = 0, expect = gridDim.x + (A.starve ? 1u : 0u);
+    unsigned target = 0;
     auto sync = [&] {
-        const bool ok = grid_sync(A.bar, target, expect, A.budget);
-        expect = gridDim.x;
+        const bool ok = grid_sync(A.bar, target, gridDim.x, A.budget);
         if (!ok && threadIdx.x == 0) atomicOr(A.err, MP_ERR_WAIT);
         return ok;
     };
@@ -1158,9 +1156,8 @@ int mp_launch_sort(mp_ctx* c) {
     const unsigned t4 = mid_sort_grid<4>(c->n, 1), t16 = t4 ? 0 : mid_sort_grid<16>(c->n, 2);
     if (t4 || t16) {
         const SmallSortArgs S = small_sort_args(c);
-        MidSortArgs M = {S.s, S.v, S.visit, c->post_bar, c->dev_error,
-                         c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET, c->starve_bar};
-        MP_CUDA(c, cudaMemsetAsync(c->post_bar, 0, sizeof(GridBar), c->stream));
+        MidSortArgs M = {S.s, S.v, S.visit, c->post_bar, c->dev_error, c->wait_budget > 0 ? c->wait_budget : MP_WAIT_BUDGET};
+        MP_CUDA(c, grid_bar_reset(c->post_bar, c->starve_bar, c->stream));
         MP_CUDA(c, launch_coop(t4 ? (const void*)k_mid_sort<4> : (const void*)k_mid_sort<16>, t4 ? t4 : t16, MS_THREADS,
                                &M, c->stream));
         MP_LAUNCHED(c);
