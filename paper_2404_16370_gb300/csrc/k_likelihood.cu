@@ -38,14 +38,14 @@
 // measured with a random-gather loop on L2-resident data; 11 cycles when they
 // hit), and a pair makes up to two (NNF entry, map record); 64 pairs are 300
 // cycles of a scheduler's FMA pipe; and the sums, the pose and the pipelined
-// gathers of two pairs need 156 to 168 registers, so 12 warps an SM cover the
-// latency of both (issue slots 0.57 used, FMA pipe 55 to 60% busy, L1 data pipe
-// 55 to 72%). Measured on one GB300, likelihood stage, every size
-// particle-major before -> now: 256 x 128 points 29 -> 8.2 us, 4096 x 512 147
-// -> 26.7 us, 10000 x 2048 688 -> 178 us, 16000 x 1021 in BF16 593 -> 147 us,
+// gathers of two pairs need 139 to 168 registers, so 12 warps an SM cover the
+// latency of both (issue slots 0.47 to 0.67 used, FMA pipe 54 to 60% busy, L1 data
+// pipe 53 to 72%). Measured on one GB300, likelihood stage, every size
+// particle-major in one pass -> this rule: 256 x 128 points 29 -> 8.2 us, 4096 x 512
+// 147 -> 26.7 us, 10000 x 2048 688 -> 178 us, 16000 x 1021 in BF16 593 -> 147 us,
 // 50021 x 4999 (outdoor, one particle a thread) 3.53 -> 2.07 ms; particle-major in
 // parts, 2^17 x 512 426 -> 392 us, 2^17 x 8192 10.4 -> 8.2 ms, 2^18 x 8192 around
-// the sensor 17.7 -> 16.7 ms, 2^20 x 8192 52.8 -> 52.4 ms.
+// the sensor 17.7 -> 16.7 ms; 2^20 x 8192 takes 52.5 ms either way.
 #include "mp_internal.cuh"
 
 #include <cuda_bf16.h>
@@ -74,7 +74,7 @@ constexpr int PM_THREADS = 128;                  // particle-major form: two par
 constexpr int PM_PER_CTA = 2 * PM_THREADS;
 constexpr int PM_CHUNK = 128;   // points per stage: 128 x 48 B = 6 KB (smaller stages leave L1 more room
                                 // for the gathers: 3% faster with converged particles than 256)
-constexpr int PM_MINB = 3;      // 163 registers
+constexpr int PM_MINB = 3;      // 163 registers, over parts of the scan 166
 constexpr int PM1_MINB = 3;     // one particle per thread, gathers in groups of four: 139 registers
 constexpr int PMH_MINB = 4;     // its 16-bit forms: their per-pair values take half the registers, so a
                                 // fourth CTA (16 warps per SM) fits in 128 registers
