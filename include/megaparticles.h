@@ -300,12 +300,13 @@ int mp_step_gicp(mp_ctx* ctx, const float* scan, int32_t n_scan, double cov_scal
  * Many independent contexts (each with its own particles and parameters;
  * presets may differ; maps their own or shared through mp_init_map_shared)
  * stepped together. mp_batch_create plans one step of all instances as about
- * thirty grouped launches, each covering the blocks of every instance (one
- * kernel per phase: prediction, scan Gaussians, LSH keys, each radix pass,
- * merge, likelihood, solve, SVGD), and the posterior as one cooperative
- * persistent launch over all instances (bounded grid barriers between its
- * sub-steps; a barrier that gives up is reported as MP_ETIMEOUT by every
- * instance). It captures the plan on cuda_stream into a CUDA graph, twice
+ * a dozen launches: grouped ones, each covering the blocks of every instance
+ * (prediction, three for the scan Gaussians, LSH keys, the sort with a CTA for
+ * each instance of at most 16384 particles, merge, likelihood by form and part
+ * of the scan, solve, SVGD), and one cooperative persistent launch each for the
+ * keys and sort of the larger instances and for the posterior of all (bounded
+ * grid barriers between their sub-steps; a barrier that gives up is reported as
+ * MP_ETIMEOUT by every instance). It captures the plan on cuda_stream into a CUDA graph, twice
  * (two pinned staging slots); mp_batch_step replays one. Per
  * instance the scan size is fixed (n_scan[i] points every step) and every step
  * runs all stages, the prediction included (identity odometry without noise

@@ -20,12 +20,12 @@
 //    (Gauss-Jordan with partial pivoting) and sets T <- T exp(delta); once max
 //    |delta| < tol all stop. The Hessian of the last iteration is kept:
 //    Sigma^DeltaT = H^-1 is taken on the host.
-// Bound by latency: at two scans of 8192 points 37 us an iteration, 13 of them
+// Bound by latency: at two scans of 8192 points 33 us an iteration, 13 of them
 // the barrier and the FP64 step (28 with its instructions on one thread) and the
 // rest the search (75 us without the last correspondence as a bound), before it
-// 57 us for the scans' order and 89 for their normals. mp_gicp at 8192 points and
+// 53 us for the scans' order and 88 for their normals. mp_gicp at 8192 points and
 // six iterations: 3930 us with all pairs of points tested and two launches an
-// iteration, 458 now.
+// iteration, 425 now.
 #include "mp_internal.cuh"
 
 #include <algorithm>

@@ -1,6 +1,7 @@
 """The posterior stage's forms against the oracle's Eq. 11: one CTA (no grid
-barrier), lists of at most 16 and 32 entries held in registers, and lists read
-by every sweep when the particle blocks outnumber the resident CTAs."""
+barrier), one cluster (129 to 1024 particles), blocks of 128 and of 256
+particles with lists of at most 16 and 32 entries held in registers, and lists
+read by every sweep when the particle blocks outnumber the resident CTAs."""
 import numpy as np
 import pytest
 
