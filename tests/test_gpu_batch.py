@@ -1,8 +1,10 @@
 """Batched instances (mp_batch_*) and the likelihood's scan split: the split
 sums equal the unsplit ones up to summation order; a batch step equals the
-same step taken instance by instance with mp_step (bit for bit with split 1);
-the autotuned batch runs with valid splits and posteriors; a starved grid
-barrier in the batched posterior is reported for every instance; contexts
+same step taken instance by instance with mp_step (bit for bit with split 1),
+on both sides of the sizes at which the sort and the likelihood change their
+form; the autotuned batch runs with valid splits and posteriors, and splits no
+scan whose sums are added in order; a starved grid barrier in the batched
+posterior or sort phase is reported for every instance; contexts
 sharing one device map (mp_init_map_shared) compute what contexts with their
 own copies compute, outlive the context that built the map, and refuse map
 parameters that differ; an instance with the preconditioned SVGD reading

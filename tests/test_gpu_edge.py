@@ -3,8 +3,9 @@ the C ABI: a single particle, ragged sizes (particles and scan points not
 multiples of the block/chunk sizes), a scan whose points are all invalid, the
 largest scan, a blackout step (empty scan), device-pointer inputs on a caller
 stream, invalid arguments, and bounded device waits made to give up (test
-knobs withhold 16 announced bytes of a bulk copy, or make a grid barrier wait
-for one CTA more than the grid has; nothing faults or hangs)."""
+knobs withhold 16 announced bytes of a bulk copy, make a grid barrier wait
+for one CTA more than the grid has, or hand out no first part of the
+likelihood; nothing faults or hangs)."""
 import numpy as np
 import pytest
 

@@ -2,7 +2,8 @@
 scan in parts of up to 1536 staged points, looked up 256 or 64 at a time and
 queued in groups of 64) at the edges of those sizes, against the oracle; and
 particle-major (many particles on a small map) against point-major, in every
-precision."""
+precision. The scan that is read is the one prepared last, and the staged slots
+beyond its points count for no pose."""
 import numpy as np
 import pytest
 
